@@ -20,7 +20,7 @@
 // the results do not depend on the order in which voxels are visited.
 #include <algorithm>
 
-#include "k_common.cuh"
+#include "k_walk.cuh"
 
 namespace libcga {
 
@@ -209,36 +209,44 @@ __global__ void k_motion(const long long* ref_c, const unsigned long long* ref_n
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_reconstruct(Levels a, const uint8_t* __restrict__ labels,
-                                                          const long long* __restrict__ mv,
-                                                          int* __restrict__ out) {
-  __shared__ Window s_win;
-  __shared__ uint16_t s_col[kTile], s_slab[kTile];
-  __shared__ uint32_t s_warp[kWarps];
+// A warp per run of voxels (k_walk.cuh); the triples of a step leave through
+// shared memory in whole sectors, by 16-byte stores when the buffer allows.
+constexpr int kReconPerSm = 5;
+__global__ void __launch_bounds__(kThreads, kReconPerSm)
+    k_reconstruct(Levels a, const uint8_t* __restrict__ labels, const long long* __restrict__ mv,
+                  int* __restrict__ out, bool vec) {
   __shared__ int s_step[kKmClusters * 3];
-  const uint32_t u = (uint32_t)a.hdr->cnt[0];
-  const uint32_t start = blockIdx.x * kTile;
-  if (start >= u) return;
-  const uint32_t cnt = min((uint32_t)kTile, u - start);
-  const uint32_t tid = threadIdx.x;
+  __shared__ uint4 s_out[kWarps][3 * kWalk / 4];
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
   // floor((mv + 128) / 256): the arithmetic shift rounds toward -infinity
   if (tid < kKmClusters * 3) s_step[tid] = (int)((mv[tid] + 128) >> 8);
-  if (tid < 32) {
-    const Window wv =
-        warp_window_of(a, (uint32_t)a.hdr->cnt[1], (uint32_t)a.hdr->cnt[2], start, start + cnt - 1);
-    if (tid == 0) s_win = wv;
-  }
   __syncthreads();
-  const Window w = s_win;
-  expand_window(a, w, start, cnt, s_col, s_slab, s_warp);
-  for (uint32_t e = tid; e < cnt; e += kThreads) {
-    const uint32_t cr = s_col[e];
-    const uint32_t L = min((uint32_t)__ldg(labels + start + e), kKmClusters - 1);
-    int* o = out + 3 * (size_t)(start + e);
-    o[0] = (int)__ldg(a.idx2 + w.x0 + s_slab[cr]) + s_step[3 * L];
-    o[1] = (int)__ldg(a.idx1 + w.c0 + cr) + s_step[3 * L + 1];
-    o[2] = (int)__ldg(a.idx0 + start + e) + s_step[3 * L + 2];
-  }
+  uint32_t begin, end;
+  walk_range((uint32_t)a.hdr->cnt[0], begin, end);
+  uint4* so = s_out[tid >> 5];
+  int* sw = reinterpret_cast<int*>(so);
+  walk_voxels(a, begin, end, [&](uint32_t p, uint32_t valid, const uint32_t* x, const uint32_t* y,
+                                 const uint32_t* z) {
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      const uint32_t e = 32 * k + lane;
+      const uint32_t L =
+          ((valid >> k) & 1u) ? min((uint32_t)__ldg(labels + p + e), kKmClusters - 1) : 0u;
+      sw[3 * e] = (int)x[k] + s_step[3 * L];
+      sw[3 * e + 1] = (int)y[k] + s_step[3 * L + 1];
+      sw[3 * e + 2] = (int)z[k] + s_step[3 * L + 2];
+    }
+    __syncwarp();
+    int* dst = out + 3 * (size_t)p;
+    if (vec && end - p >= kWalk) {
+#pragma unroll
+      for (uint32_t i = 0; i < 3; ++i) reinterpret_cast<uint4*>(dst)[32 * i + lane] = so[32 * i + lane];
+    } else {
+      const uint32_t n = 3 * min(end - p, kWalk);
+      for (uint32_t i = lane; i < n; i += 32) dst[i] = sw[i];
+    }
+    __syncwarp();
+  });
 }
 
 // res[i*C + c] = pred[i*C + c] - ref[idx[i]*C + c], or pred[i*C + c] when
@@ -331,9 +339,9 @@ cudaError_t run_motion(const long long* ref_c, const unsigned long long* ref_n,
 
 cudaError_t run_reconstruct(const Levels& a, const uint8_t* labels, const long long* mv, int* out,
                             cudaStream_t stream) {
-  const uint64_t tiles = (a.cap + kTile - 1) / kTile;
-  if (tiles == 0) return cudaSuccess;
-  k_reconstruct<<<(unsigned)tiles, kThreads, 0, stream>>>(a, labels, mv, out);
+  if (a.cap == 0) return cudaSuccess;
+  k_reconstruct<<<walk_blocks(a.cap, kReconPerSm), kThreads, 0, stream>>>(
+      a, labels, mv, out, (reinterpret_cast<uintptr_t>(out) & 15u) == 0);
   count_launch(1);
   return cudaGetLastError();
 }

@@ -3,6 +3,7 @@
 #include <atomic>
 
 #include "k_compact.cuh"
+#include "k_walk.cuh"
 
 namespace libcga {
 
@@ -11,32 +12,39 @@ namespace {
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // ------------------------------------------------------------------ decode
-// Lossless inverse of the build: the walk X -> Y -> Z of Sec. V-A, done per
-// tile of Z positions (the tile's window is expanded into per-position column
-// and slab indices in shared memory).
-__global__ void __launch_bounds__(kThreads) k_decode(Levels a, uint32_t* __restrict__ xyz) {
-  __shared__ Window s_win;
-  __shared__ uint16_t s_col[kTile], s_slab[kTile];
-  __shared__ uint32_t s_warp[kWarps];
-  const uint32_t u = (uint32_t)a.hdr->cnt[0];
-  const uint32_t start = blockIdx.x * kTile;
-  if (start >= u) return;
-  const uint32_t cnt = min((uint32_t)kTile, u - start);
-  if (threadIdx.x < 32) {
-    const Window wv =
-        warp_window_of(a, (uint32_t)a.hdr->cnt[1], (uint32_t)a.hdr->cnt[2], start, start + cnt - 1);
-    if (threadIdx.x == 0) s_win = wv;
-  }
-  __syncthreads();
-  const Window w = s_win;
-  expand_window(a, w, start, cnt, s_col, s_slab, s_warp);
-  for (uint32_t e = threadIdx.x; e < cnt; e += kThreads) {
-    const uint32_t cr = s_col[e];
-    uint32_t* o = xyz + (size_t)(start + e) * 3;
-    o[0] = __ldg(a.idx2 + w.x0 + s_slab[cr]);
-    o[1] = __ldg(a.idx1 + w.c0 + cr);
-    o[2] = __ldg(a.idx0 + start + e);
-  }
+// Lossless inverse of the build: the walk X -> Y -> Z of Sec. V-A, a warp per
+// run of positions (k_walk.cuh).  The 128 triples of a step leave through
+// shared memory so that the output is written in whole sectors, by 16-byte
+// stores when the caller's buffer allows (vec).
+constexpr int kDecodePerSm = 5;
+__global__ void __launch_bounds__(kThreads, kDecodePerSm) k_decode(Levels a, uint32_t* __restrict__ xyz,
+                                                                   bool vec) {
+  __shared__ uint4 s_out[kWarps][3 * kWalk / 4];
+  uint32_t begin, end;
+  walk_range((uint32_t)a.hdr->cnt[0], begin, end);
+  const uint32_t lane = threadIdx.x & 31u;
+  uint4* so = s_out[threadIdx.x >> 5];
+  uint32_t* sw = reinterpret_cast<uint32_t*>(so);
+  walk_voxels(a, begin, end, [&](uint32_t p, uint32_t, const uint32_t* x, const uint32_t* y,
+                                 const uint32_t* z) {
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      uint32_t* o = sw + 3 * (32 * k + lane);
+      o[0] = x[k];
+      o[1] = y[k];
+      o[2] = z[k];
+    }
+    __syncwarp();
+    uint32_t* dst = xyz + 3 * (size_t)p;
+    if (vec && end - p >= kWalk) {
+#pragma unroll
+      for (uint32_t i = 0; i < 3; ++i) reinterpret_cast<uint4*>(dst)[32 * i + lane] = so[32 * i + lane];
+    } else {
+      const uint32_t n = 3 * min(end - p, kWalk);
+      for (uint32_t i = lane; i < n; i += 32) dst[i] = sw[i];
+    }
+    __syncwarp();
+  });
 }
 
 // ------------------------------------------------------------------- merge
@@ -1063,33 +1071,21 @@ __global__ void k_project_xy(Levels a, Levels o) {
 // by row, in order, are the distinct 2D voxels in key order: U_index the
 // non-empty rows, V_index the set columns of each.
 
-// Set the bits of a's voxels (a tile of Z positions per block, decoded by the
-// X -> Y -> Z walk of Sec. V-A as in k_decode).
-__global__ void __launch_bounds__(kThreads) k_proj_set(Levels a, int plane,
+// Set the bits of a's voxels, decoded by the walk of Sec. V-A (k_walk.cuh).
+constexpr int kProjPerSm = 6;
+__global__ void __launch_bounds__(kThreads, kProjPerSm) k_proj_set(Levels a, int plane,
                                                        uint32_t* __restrict__ bits) {
-  __shared__ Window s_win;
-  __shared__ uint16_t s_col[kTile], s_slab[kTile];
-  __shared__ uint32_t s_warp[kWarps];
-  const uint32_t u = (uint32_t)a.hdr->cnt[0];
-  const uint32_t start = blockIdx.x * kTile;
-  if (start >= u) return;
-  const uint32_t cnt = min((uint32_t)kTile, u - start);
-  if (threadIdx.x < 32) {
-    const Window wv =
-        warp_window_of(a, (uint32_t)a.hdr->cnt[1], (uint32_t)a.hdr->cnt[2], start, start + cnt - 1);
-    if (threadIdx.x == 0) s_win = wv;
-  }
-  __syncthreads();
-  const Window w = s_win;
-  expand_window(a, w, start, cnt, s_col, s_slab, s_warp);
+  uint32_t begin, end;
+  walk_range((uint32_t)a.hdr->cnt[0], begin, end);
   const uint32_t b = a.bits;
-  for (uint32_t e = threadIdx.x; e < cnt; e += kThreads) {
-    const uint32_t cr = s_col[e];
-    const uint32_t r = plane == 1 ? (uint32_t)__ldg(a.idx2 + w.x0 + s_slab[cr])
-                                  : (uint32_t)__ldg(a.idx1 + w.c0 + cr);
-    const uint32_t key = (r << b) | __ldg(a.idx0 + start + e);
-    atomicOr(bits + (key >> 5), 1u << (key & 31u));
-  }
+  walk_voxels(a, begin, end, [&](uint32_t, uint32_t valid, const uint32_t* x, const uint32_t* y,
+                                 const uint32_t* z) {
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      const uint32_t key = ((plane == 1 ? x[k] : y[k]) << b) | z[k];
+      if ((valid >> k) & 1u) atomicOr(bits + (key >> 5), 1u << (key & 31u));
+    }
+  });
 }
 
 // Set bits of each row: one warp per row, each lane a run of the row's words.
@@ -1180,9 +1176,9 @@ __global__ void __launch_bounds__(256) k_proj_write(const uint32_t* __restrict__
 }  // namespace
 
 cudaError_t run_decode(const Levels& a, uint32_t* xyz, cudaStream_t stream) {
-  const uint64_t tiles = (a.cap + kTile - 1) / kTile;
-  if (tiles == 0) return cudaSuccess;
-  k_decode<<<(unsigned)tiles, kThreads, 0, stream>>>(a, xyz);
+  if (a.cap == 0) return cudaSuccess;
+  k_decode<<<walk_blocks(a.cap, kDecodePerSm), kThreads, 0, stream>>>(
+      a, xyz, (reinterpret_cast<uintptr_t>(xyz) & 15u) == 0);
   count_launch(1);
   return cudaGetLastError();
 }
@@ -1320,13 +1316,14 @@ cudaError_t run_project_bitmap(const Levels& a, int plane, const Levels& out, vo
   uint32_t* rowoff = reinterpret_cast<uint32_t*>(p);
   cudaError_t e = cudaMemsetAsync(bits, 0, bit_bytes, stream);
   if (e != cudaSuccess) return e;
-  const uint64_t tiles = (a.cap + kTile - 1) / kTile;
-  if (tiles > 0) k_proj_set<<<(unsigned)tiles, kThreads, 0, stream>>>(a, plane, bits);
+  if (a.cap > 0) {
+    k_proj_set<<<walk_blocks(a.cap, kProjPerSm), kThreads, 0, stream>>>(a, plane, bits);
+  }
   const unsigned row_blocks = ((1u << b) + 7u) / 8u;  // a warp per row
   k_proj_rows<<<row_blocks, 256, 0, stream>>>(bits, b, rowcnt);
   k_proj_scan<<<1, kThreads, 0, stream>>>(rowcnt, b, rowoff, out, a.hdr);
   k_proj_write<<<row_blocks, 256, 0, stream>>>(bits, b, rowoff, out);
-  count_launch(tiles > 0 ? 4 : 3);
+  count_launch(a.cap > 0 ? 4 : 3);
   return cudaGetLastError();
 }
 

@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include "k_compact.cuh"
+#include "k_walk.cuh"
 
 namespace libcga {
 
@@ -55,9 +56,6 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
   constexpr int R = 1 << RB;
   __shared__ uint32_t s_hist[kMaxPasses][R];
   __shared__ float s_pts[kThreads * 3];
-  __shared__ Window s_win;
-  __shared__ uint16_t s_col[kTile], s_slab[kTile];
-  __shared__ uint32_t s_warp[kWarps];
   __shared__ uint32_t s_err;
   const int tid = threadIdx.x;
   const uint32_t t0 = blockIdx.x * tiles_per_cta;
@@ -117,39 +115,45 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
         }
       }
     } else {
-      // projection: decode the source point, keep two axes
+      // projection, coarse level or tree: the block's run of tiles of this
+      // segment, a warp per equal share of its positions (k_walk.cuh)
       const Levels& a = sg.src;
-      if (tid < 32) {
-        const Window wv = warp_window_of(a, (uint32_t)a.hdr->cnt[1], (uint32_t)a.hdr->cnt[2],
-                                         start, start + cnt - 1);
-        if (tid == 0) s_win = wv;
-      }
-      __syncthreads();
-      const Window win = s_win;
-      expand_window(a, win, start, cnt, s_col, s_slab, s_warp);
-      for (uint32_t e = tid; e < cnt; e += kThreads) {
-        const uint32_t cr = s_col[e];
-        const uint32_t x = __ldg(a.idx2 + win.x0 + s_slab[cr]);
-        const uint32_t y = __ldg(a.idx1 + win.c0 + cr);
-        const uint32_t z = __ldg(a.idx0 + start + e);
-        K key;
-        if (sg.plane == 3) {
-          const uint32_t L = sg.shift;
-          key = ((K)(x >> L) << (2 * b)) | ((K)(y >> L) << b) | (K)(z >> L);
-        } else if (sg.plane == 4) {
-          key = (K)tree_key(x, y, z, sg.shift);
-        } else {
-          uint32_t u = x, v = y;
-          if (sg.plane == 1) { u = x; v = z; }
-          if (sg.plane == 2) { u = y; v = z; }
-          key = ((K)u << b) | (K)v;
+      const uint32_t tl = min(t1, sg.tile_base + sg.num_tiles);
+      const uint32_t stop = min(n, (tl - sg.tile_base) * (uint32_t)kTile);
+      const uint32_t per = ((stop - start + kWarps * kWalk - 1) / (kWarps * kWalk)) * kWalk;
+      const uint32_t w0 = min(stop, start + (uint32_t)(tid >> 5) * per);
+      K* kout = keys0 + sg.key_base;
+      walk_voxels(a, w0, min(stop, w0 + per), [&](uint32_t p, uint32_t valid, const uint32_t* x,
+                                                  const uint32_t* y, const uint32_t* z) {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) {
+          K key;
+          if (sg.plane == 3) {
+            const uint32_t L = sg.shift;
+            key = ((K)(x[i] >> L) << (2 * b)) | ((K)(y[i] >> L) << b) | (K)(z[i] >> L);
+          } else if (sg.plane == 4) {
+            key = (K)tree_key(x[i], y[i], z[i], sg.shift);
+          } else {
+            const uint32_t u = sg.plane == 2 ? y[i] : x[i], v = sg.plane == 0 ? y[i] : z[i];
+            key = ((K)u << b) | (K)v;
+          }
+          const bool ok = (valid >> i) & 1u;
+          if (ok) kout[p + 32 * i + (tid & 31)] = key;
+          // neighbouring voxels share their high digits: one count for the
+          // warp where all lanes hold the same digit
+          const uint32_t live = __ballot_sync(0xffffffffu, ok);
+          for (uint32_t q = 0; q < passes; ++q) {
+            const uint32_t d = (uint32_t)(key >> (sg.bit0 + q * RB)) & (R - 1);
+            const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+            if (__all_sync(0xffffffffu, !ok || d == d0)) {
+              if ((tid & 31) == 0 && live) atomicAdd(&s_hist[q][d0], (uint32_t)__popc(live));
+            } else if (ok) {
+              atomicAdd(&s_hist[q][d], 1u);
+            }
+          }
         }
-        out[e] = key;
-        for (uint32_t p = 0; p < passes; ++p) {
-          atomicAdd(&s_hist[p][(uint32_t)(key >> (sg.bit0 + p * RB)) & (R - 1)], 1u);
-        }
-      }
-      __syncthreads();
+      });
+      t = tl - 1;
     }
   }
   flush(cur);

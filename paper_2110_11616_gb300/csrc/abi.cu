@@ -708,6 +708,17 @@ int cga_kmeans(const cga_t* a, uint32_t max_iter, uint8_t* d_label, int64_t* d_c
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const cga_allocator* A = a->has_alloc ? &a->alloc : nullptr;
+  // by cells when the allocator has room for the voxels in cell order
+  // (5 bytes a voxel of capacity and the cell tables), else voxel by voxel
+  const size_t cells = libcga::kmeans_cells_bytes(a->grid.bits, a->lv.cap);
+  void* cs = cells > 0 ? dalloc(A, cells, s) : nullptr;
+  if (cs != nullptr) {
+    const int rc = cuda_rc(libcga::run_kmeans_cells(
+        a->lv, max_iter, cs, d_label, reinterpret_cast<long long*>(d_centres),
+        reinterpret_cast<unsigned long long*>(d_counts), d_iters, s));
+    dfree(A, a->has_alloc, cs, s);
+    return rc;
+  }
   void* st = dalloc(A, sizeof(libcga::KmState), s);
   if (st == nullptr) return CGA_ERR_OOM;
   const int rc = cuda_rc(libcga::run_kmeans(

@@ -817,9 +817,13 @@ void drop_coarse(cga* a) {
 // The occupancy tree of `a` (errors of its bounded waits land in a's header).
 int build_tree(cga* a, cudaStream_t s) {
   const cga_allocator* A = a->has_alloc ? &a->alloc : nullptr;
-  const libcga::TreeLayout L = libcga::tree_layout(a->grid.bits, a->lv.cap);
+  libcga::TreeLayout L = libcga::tree_layout(a->grid.bits, a->lv.cap, true);
   const libcga::Tuning tu = libcga::tuning_for(a->grid.bits, a->lv.cap);
   void* mem = dalloc(A, L.bytes, s);
+  if (mem == nullptr && L.dense_level > 0) {
+    L = libcga::tree_layout(a->grid.bits, a->lv.cap, false);
+    mem = dalloc(A, L.bytes, s);
+  }
   if (mem == nullptr) return CGA_ERR_OOM;
   void* scratch = dalloc(A, libcga::tree_scratch_bytes(L, tu.radix_bits), s);
   if (scratch == nullptr) {

@@ -376,9 +376,17 @@ __host__ __device__ inline uint32_t tree_box_code(unsigned long long m) {
 // the node): lo_x | hi_x << 4 | lo_y << 8 | hi_y << 12 | lo_z << 16 | hi_z << 20.
 // Every entry of a level l below the root also keeps its box in its parent's
 // frame (pcode): 6-bit bounds counted from the parent's origin in cells of
-// 4^(l-2) voxels (l >= 2) or in voxels (bricks), Lx | Hx << 6 | Ly << 12 |
-// Hy << 18 in .x and Lz | Hz << 6 in .y; the box along x covers
-// [Lx * u, (Hx + 1) * u) voxels from the parent's origin for that unit u.
+// 4^(l-2) voxels (l >= 2) or in voxels (bricks); the box along x covers
+// [Lx * u, (Hx + 1) * u) voxels from the parent's origin for that unit u.  A
+// byte each with the top bit set (0x3F and such a byte are the high half of the
+// float 1 + v / 128): .x holds Lx, Hx, Ly, Hy from the low byte up, .y Lz, Hz,
+// and in its upper half the entry's child number, so a parent's children, which
+// lie side by side, can be read without its child set.
+// The nodes of one level (dense_level) can also be found by position: dense
+// holds the index of the node of cell (X, Y, Z) at X << 2c | Y << c | Z, c =
+// dense_bits (kTreeAbsent: an empty cell), so a search that knows a bound of a
+// few cells starts there instead of at the root.
+constexpr uint32_t kTreeAbsent = 0xffffffffu;
 struct TreeView {
   const unsigned long long* brick;        // level 1: voxel occupancy of each brick
   const uint32_t* bcode;                  // level 1: tree_box_code of each brick (voxel units)
@@ -387,6 +395,8 @@ struct TreeView {
   const uint2* pcode[kTreeMaxLevels + 1]; // level l < levels: box in the parent's frame
   uint32_t cap[kTreeMaxLevels + 1];       // entries reserved per level (a search never reads beyond)
   uint32_t levels;                        // 0: no tree
+  const uint32_t* dense;                  // nodes of dense_level by position (or null)
+  uint32_t dense_level, dense_bits;
 };
 // Capacity of every level (cap[0]: voxels) and the bytes of the tree arrays
 // (offsets from one base: off[1] bricks, off_bcode their box codes, off[l]
@@ -397,10 +407,14 @@ struct TreeLayout {
   size_t off[kTreeMaxLevels + 1];
   size_t off_pcode[kTreeMaxLevels + 1];
   size_t off_bcode;
+  size_t off_dense;
   size_t bytes;
   uint32_t levels;
+  uint32_t dense_level, dense_bits;  // dense_level 0: no position table
 };
-TreeLayout tree_layout(uint32_t bits, uint64_t cap);
+// with_dense: room for the position table of a level (left out when the
+// allocator has no room for it: searches then start at the root).
+TreeLayout tree_layout(uint32_t bits, uint64_t cap, bool with_dense);
 // Scratch of one tree build (the Morton-key sort and the per-level
 // look-back words).
 size_t tree_scratch_bytes(const TreeLayout& L, uint32_t radix_bits);

@@ -258,14 +258,15 @@ constexpr int kQueryLimit = 1 << 30;
 #define CGA_NN_COARSE_BLOCKS 5
 #endif
 #ifndef CGA_NN_TREE_BLOCKS
-#define CGA_NN_TREE_BLOCKS 4
+#define CGA_NN_TREE_BLOCKS 8
 #endif
 #ifndef CGA_NN_HEAD_GROUP
 #define CGA_NN_HEAD_GROUP 16
 #endif
 #ifndef CGA_NN_TREE_GROUP
-#define CGA_NN_TREE_GROUP 4
+#define CGA_NN_TREE_GROUP 8
 #endif
+constexpr int kTreeThreads = 128;  // a block's queues (25 KB) then fit eight times on an SM
 
 // Voxel of query j of a segment, clamped to +-2^30 (so every coordinate
 // difference fits 31 bits); false for a non-finite query point.
@@ -621,9 +622,9 @@ struct BestKey {
 // is max(L u - t, t + ub - H u, 0).
 template <typename D>
 __device__ __forceinline__ D parent_frame_lb(uint2 c, int tx, int ty, int tz, int ub, uint32_t ss) {
-  const int lx = (int)((c.x & 63u) << ss), hx = (int)(((c.x >> 6) & 63u) << ss);
-  const int ly = (int)(((c.x >> 12) & 63u) << ss), hy = (int)(((c.x >> 18) & 63u) << ss);
-  const int lz = (int)((c.y & 63u) << ss), hz = (int)(((c.y >> 6) & 63u) << ss);
+  const int lx = (int)((c.x & 63u) << ss), hx = (int)(((c.x >> 8) & 63u) << ss);
+  const int ly = (int)(((c.x >> 16) & 63u) << ss), hy = (int)(((c.x >> 24) & 63u) << ss);
+  const int lz = (int)((c.y & 63u) << ss), hz = (int)(((c.y >> 8) & 63u) << ss);
   const D dx = (uint32_t)max(max(lx - tx, tx + ub - hx), 0);
   const D dy = (uint32_t)max(max(ly - ty, ty + ub - hy), 0);
   const D dz = (uint32_t)max(max(lz - tz, tz + ub - hz), 0);
@@ -792,17 +793,52 @@ struct TreeWalk {
   }
 };
 
-// CGA index of the stored voxel with key `key` (the Sec. V-A lookup: x
-// directory or X_index, the slab's Y range, the column's Z range).
-__device__ __forceinline__ uint32_t stored_index(const NnSeg& sg, unsigned long long key) {
+// First index in [lo, hi) whose value is >= v, by each group of G lanes of the
+// warp for its own range (all lanes call; empty ranges cost nothing): G probes
+// a round, so a range of n entries takes log_G(n) dependent loads.
+template <int G>
+__device__ __forceinline__ uint32_t group_lower_bound_u16(const uint16_t* __restrict__ a,
+                                                          uint32_t lo, uint32_t hi, uint32_t v,
+                                                          uint32_t g, uint32_t gm) {
+  const uint32_t full = 0xffffffffu;
+  while (__any_sync(full, hi - lo > (uint32_t)G)) {
+    const uint32_t step = (hi - lo + G - 1) / G;
+    const uint32_t probe = min(lo + step * (g + 1), hi) - 1;
+    const bool lt = hi - lo > (uint32_t)G && (uint32_t)__ldg(a + probe) < v;
+    const uint32_t k = (uint32_t)__popc(__ballot_sync(full, lt) & gm);
+    if (hi - lo > (uint32_t)G) {
+      const uint32_t nhi = k == (uint32_t)G ? hi : min(lo + step * (k + 1), hi);
+      lo = min(lo + step * k, hi);
+      hi = nhi;
+    }
+  }
+  const bool lt = lo + g < hi && (uint32_t)__ldg(a + lo + g) < v;
+  return lo + (uint32_t)__popc(__ballot_sync(full, lt) & gm);
+}
+
+// CGA index of the stored voxel with key `key`, by each group of the warp whose
+// `on` is set (the Sec. V-A lookup: x directory or X_index, the slab's Y range,
+// the column's Z range).
+template <int G>
+__device__ __forceinline__ uint32_t stored_index(const NnSeg& sg, unsigned long long key, bool on,
+                                                 uint32_t g, uint32_t gm) {
   const Levels& a = sg.a;
   const uint32_t b = a.bits, mk = (1u << b) - 1u;
-  const uint32_t x = (uint32_t)(key >> (2 * b)), y = (uint32_t)(key >> b) & mk,
+  const uint32_t x = (uint32_t)(key >> (2 * b)) & mk, y = (uint32_t)(key >> b) & mk,
                  z = (uint32_t)key & mk;
-  const uint32_t h = (uint32_t)a.hdr->cnt[2];
-  const uint32_t slab = sg.xdir != nullptr ? __ldg(sg.xdir + x) : lower_bound_u16(a.idx2, 0, h, x);
-  const uint32_t c = lower_bound_u16(a.idx1, __ldg(a.ptr2 + slab), __ldg(a.ptr2 + slab + 1), y);
-  return lower_bound_u16(a.idx0, __ldg(a.ptr1 + c), __ldg(a.ptr1 + c + 1), z);
+  uint32_t slab = 0, ys = 0, ye = 0, zs = 0, ze = 0;
+  if (on) {
+    const uint32_t h = (uint32_t)a.hdr->cnt[2];
+    slab = sg.xdir != nullptr ? __ldg(sg.xdir + x) : lower_bound_u16(a.idx2, 0, h, x);
+    ys = __ldg(a.ptr2 + slab);
+    ye = __ldg(a.ptr2 + slab + 1);
+  }
+  const uint32_t c = group_lower_bound_u16<G>(a.idx1, ys, ye, y, g, gm);
+  if (on) {
+    zs = __ldg(a.ptr1 + c);
+    ze = __ldg(a.ptr1 + c + 1);
+  }
+  return group_lower_bound_u16<G>(a.idx0, zs, ze, z, g, gm);
 }
 
 // The whole descent.  The loop runs while any group of the warp is still
@@ -828,6 +864,307 @@ __device__ void search_tree(const TreeView& tv, const Qry& q, uint32_t b, bool a
   while (__any_sync(0xffffffffu, !w.done)) {
     if (!w.done) w.step(tv, q, b, gm, g, best);
   }
+}
+
+// ---- breadth-first search of the tree ---------------------------------------
+//
+// The same answer as the descent above with far fewer instructions.  What made
+// the descent slow was its steps: a far query took about fifty, each a few
+// hundred warp instructions of picking, pushing and popping in which 9 of 32
+// lanes worked.  Here a group of G lanes keeps a queue of nodes and takes them
+// level by level; a node's children lie side by side, so the lanes bound G of
+// them at once with no child set to decode, and append the survivors.
+//
+// Level by level, a search needs a good distance bound before it reaches the
+// finest levels.  It has one without finding a voxel: the boxes are tight, so
+// every face slab of a child's box holds a stored voxel, and the nearest face
+// bounds the distance to it (all other coordinates at their farthest).  The
+// bound of the best child so far, over every child looked at, prunes the rest of
+// the level and the queue.  With it a far query bounds about as many children as
+// the depth-first order (560 and 550 on the surface world) and reads fewer
+// bricks (17 and 22), and all of them in full groups.
+//
+// The bounds are computed in single precision where every coordinate
+// difference is below 2^17 (queries inside the grid): a box field becomes a
+// float by one byte permute, differences are exact, and the two or three
+// roundings of a bound are covered by widening it by a relative 2^-21 and more
+// (in integers the bounds kept the half-rate integer pipe 67% busy: 17.9 ms for
+// 4M surface-world queries against 16.9).  Distances to voxels, and so answers,
+// are exact integers.
+//
+// Measured, search kernels alone: 4M surface-world queries, half of them far
+// from any voxel, 29.7 -> 17.2 ms; 20M voxels moved about five voxels off the
+// surfaces 31.9 -> 21.4 ms.  Still bound by instruction issue (70%, 24 of 32
+// lanes active; 4.3k warp instructions a far query, 1k a near one): per warp of
+// four far queries 39 nodes and 127 groups of children, the longest child list
+// of the four setting each round.  Sixteen lanes a query take 8% less on far
+// queries and 25-35% more on near ones; four lanes overflow their queues.
+//
+// A queue entry is three words: the node, its parent's cell with its own child
+// number, and the upper half of its lower bound (kept only to drop entries that
+// a later bound rules out).  A group whose queue would overflow (a query with
+// very many nodes at nearly the same distance) finishes by the descent above,
+// from the bound it has.
+template <int G>
+struct BfsQueue {
+  static constexpr uint32_t kCap = 16 * G;
+  uint32_t w[3][kCap + G];  // the pad keeps the groups of a warp on other banks
+};
+
+// Bounds of the distance from a query to a box: it holds a voxel, and one in
+// every face slab of 2^ss voxels.  (L, H) are the box in units of 2^ss from an
+// origin, t the query from there.  lb: no voxel of the box is nearer; ub: some
+// voxel is at most that far.  In exact integers, then rounded outward.
+template <typename D>
+struct BoxBounds {
+  D lb2 = 0, far2 = 0, gain = 0;
+  __device__ __forceinline__ void axis(uint32_t L, uint32_t H, int t, uint32_t ss, int w) {
+    const int a = (int)(L << ss) - t, b = t - (int)(H << ss) - w;
+    const D m = (uint32_t)max(max(a, b), 0);
+    const uint32_t fa = (uint32_t)abs(a), fb = (uint32_t)abs(b);
+    const uint32_t far = max(fa, fb), near = min(min(fa, fb) + (uint32_t)w, far);
+    lb2 += m * m;
+    const D f2 = (D)far * far;
+    far2 += f2;
+    gain = max(gain, f2 - (D)near * near);
+  }
+  __device__ __forceinline__ float lb() const { return __ull2float_rd(lb2); }
+  __device__ __forceinline__ float ub() const { return __ull2float_ru(far2 - gain); }
+};
+
+// The same in single precision from box bytes (TreeView::pcode): t and 2^ss
+// below 2^17, so every difference is exact.
+struct BoxBoundsF {
+  float lb2 = 0.0f, far2 = 0.0f, gain = 0.0f;
+  // u = 128 * 2^ss; cl = -(u + t), ch = cl + 2^ss - 1
+  template <uint32_t BL, uint32_t BH>
+  __device__ __forceinline__ void axis(uint32_t bytes, float u, float cl, float ch) {
+    const float fl = __uint_as_float(__byte_perm(bytes, 0x3f000000u, 0x7044u | BL << 8));
+    const float fh = __uint_as_float(__byte_perm(bytes, 0x3f000000u, 0x7044u | BH << 8));
+    const float lo = __fmaf_rn(fl, u, cl), hi = __fmaf_rn(fh, u, ch);
+    const float m = fmaxf(fmaxf(lo, -hi), 0.0f);
+    const float far = fmaxf(fabsf(lo), fabsf(hi));
+    const float near = fminf(fabsf(lo), fabsf(hi)) + (ch - cl);
+    lb2 = __fmaf_rn(m, m, lb2);
+    far2 = __fmaf_rn(far, far, far2);
+    gain = fmaxf(gain, (far - near) * (far + near));
+  }
+  __device__ __forceinline__ float lb() const { return lb2 * 0.9999995f; }
+  __device__ __forceinline__ float ub() const { return __fmaf_rn(far2, 1.0000010f, -gain); }
+};
+
+// A float not below the distance, and a distance not below the float.
+__device__ __forceinline__ float bound_up(uint32_t v) { return __uint2float_ru(v); }
+__device__ __forceinline__ float bound_up(unsigned long long v) { return __ull2float_ru(v); }
+template <typename D>
+__device__ __forceinline__ D bound_from(float f) {
+  if constexpr (sizeof(D) == 4) return __float2uint_ru(f); else return __float2ull_ru(f);
+}
+
+// Least value over each group of G lanes (all lanes of the warp call).
+template <int G, typename D>
+__device__ __forceinline__ D group_least(D v) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// Searches for every group of the warp whose `active` is set; all lanes call.
+// best starts from a bound without a voxel (or all ones).  Returns true for a
+// group that gave up (queue full): best.d2 is then still a valid bound.
+template <int G, typename D>
+__device__ __forceinline__ bool search_bfs(const TreeView& tv, const Qry& q, uint32_t b,
+                                           bool active, uint32_t g, uint32_t gm, BfsQueue<G>& Q,
+                                           BestKey<D>& best) {
+  constexpr uint32_t CAP = BfsQueue<G>::kCap, full = 0xffffffffu;
+  const uint32_t sh = __ffs((int)gm) - 1, below = gm & lanemask_lt();
+  float R = bound_up(best.d2);
+  uint32_t head = 0, tail = 0, lend = 0, lvl = tv.levels;
+  bool run = active, gave_up = false;
+  // entry: node; parent cell x | y << 12 | z << 24; lower bound's upper half,
+  // (parent z >> 8) << 6, child number
+  auto put = [&](bool keep, uint32_t ci, uint32_t w1, uint32_t w2) {
+    const uint32_t bal = __ballot_sync(full, keep) & gm;
+    const uint32_t n = (uint32_t)__popc(bal);
+    if (tail + n - head > CAP) {
+      gave_up = true;
+      run = false;
+    } else if (keep) {
+      const uint32_t e = (tail + (uint32_t)__popc(bal & below)) & (CAP - 1);
+      Q.w[0][e] = ci;
+      Q.w[1][e] = w1;
+      Q.w[2][e] = w2;
+    }
+    tail += n;
+  };
+  auto cell_of = [&](uint32_t w1, uint32_t w2, uint32_t& X, uint32_t& Y, uint32_t& Z) {
+    uint32_t cx, cy, cz;
+    tree_cell(w2 & 63u, cx, cy, cz);
+    X = (w1 & 0xfffu) << 2 | cx;
+    Y = ((w1 >> 12) & 0xfffu) << 2 | cy;
+    Z = (w1 >> 24 | ((w2 >> 6) & 0xfu) << 8) << 2 | cz;
+  };
+  // Start: the nodes of the position table that the bound reaches, when they
+  // are at most four per axis; the query's own cell first tightens the bound.
+  bool dense = false;
+  if (tv.dense != nullptr) {
+    const uint32_t ld = tv.dense_level, c = tv.dense_bits, ss = 2 * (ld - 2);
+    const int w = (1 << ss) - 1, top = (int)((1u << (b - min(b, 2 * ld))) - 1u);
+    auto node_box = [&](uint32_t id, uint32_t X, uint32_t Y, uint32_t Z) {
+      const uint32_t code = __ldg(&tv.node[ld][id].w);
+      BoxBounds<D> bb;
+      bb.axis(code & 15u, (code >> 4) & 15u, q.x - (int)(X << (2 * ld)), ss, w);
+      bb.axis((code >> 8) & 15u, (code >> 12) & 15u, q.y - (int)(Y << (2 * ld)), ss, w);
+      bb.axis((code >> 16) & 15u, (code >> 20) & 15u, q.z - (int)(Z << (2 * ld)), ss, w);
+      return bb;
+    };
+    if (run) {
+      const uint32_t X = q.cx >> (2 * ld), Y = q.cy >> (2 * ld), Z = q.cz >> (2 * ld);
+      const uint32_t id = __ldg(tv.dense + ((size_t)X << (2 * c) | Y << c | Z));
+      if (id != kTreeAbsent) R = fminf(R, node_box(id, X, Y, Z).ub());
+    }
+    // the ball's cells per axis, from a root not below the exact one
+    const float rf = __fsqrt_ru(R);
+    const int r = rf < 1.0e9f ? (int)rf + 1 : 1000000000;
+    auto lo_of = [&](int v) { return min(max((v - r) >> (int)(2 * ld), 0), top); };
+    auto hi_of = [&](int v) { return min(max((v + r) >> (int)(2 * ld), 0), top); };
+    const int x0 = lo_of(q.x), y0 = lo_of(q.y), z0 = lo_of(q.z);
+    const int nx = hi_of(q.x) - x0, ny = hi_of(q.y) - y0, nz = hi_of(q.z) - z0;
+    const int most = max(nx, max(ny, nz));
+    dense = run && most < 4;
+    // cell t of the block: t = (dx * (ny + 1) + dy) * (nz + 1) + dz, the two
+    // quotients by a multiplication (exact: t < 64, divisors at most 16)
+    const uint32_t dzs = (uint32_t)nz + 1u, dyz = dense ? ((uint32_t)ny + 1u) * dzs : 1u;
+    const uint32_t cells = dense ? ((uint32_t)nx + 1u) * dyz : 0u;
+    const uint32_t mx = 65536u / dyz + 1u, my = 65536u / (dense ? dzs : 1u) + 1u;
+    for (uint32_t t0 = 0; __any_sync(full, t0 < cells); t0 += G) {
+      const uint32_t t = t0 + g;
+      const bool in = t < cells;
+      const uint32_t dx = (t * mx) >> 16, ty = t - dx * dyz;
+      const uint32_t dy = (ty * my) >> 16, dz = ty - dy * dzs;
+      const uint32_t X = (uint32_t)x0 + dx, Y = (uint32_t)y0 + dy, Z = (uint32_t)z0 + dz;
+      uint32_t id = kTreeAbsent;
+      float lb = 0.0f, ub = 3.0e38f;
+      if (in) id = __ldg(tv.dense + ((size_t)X << (2 * c) | Y << c | Z));
+      if (id != kTreeAbsent) {
+        const BoxBounds<D> bb = node_box(id, X, Y, Z);
+        lb = bb.lb();
+        ub = bb.ub();
+      }
+      R = fminf(R, group_least<G, float>(ub));
+      const uint32_t px = X >> 2, py = Y >> 2, pz = Z >> 2;
+      put(id != kTreeAbsent && lb <= R, id, px | py << 12 | pz << 24,
+          (__float_as_uint(lb) & 0xffff0000u) | (pz >> 8) << 6 | tree_child(X & 3u, Y & 3u, Z & 3u));
+    }
+    if (dense) {
+      lvl = ld;
+      lend = tail;
+    }
+  }
+  if (run && !dense) {  // from the root
+    if (g == 0) {
+      Q.w[0][0] = 0;
+      Q.w[1][0] = 0;
+      Q.w[2][0] = 0;
+    }
+    head = 0;
+    tail = lend = 1;
+  }
+  __syncwarp();
+  // nodes level by level, the nearest level of the queue first
+  while (__any_sync(full, run)) {
+    if (run && head == lend) {
+      --lvl;
+      lend = tail;
+      if (lvl == 1 || head == tail) run = false;
+    }
+    // the next entry that the bound has not ruled out since it was put there
+    const bool have = run && head + g < lend;
+    const bool ok =
+        have && (Q.w[2][(head + g) & (CAP - 1)] >> 16) <= (__float_as_uint(R) >> 16);
+    const uint32_t bal = (__ballot_sync(full, ok) & gm) >> sh;
+    uint32_t n = 0, first = 0, X = 0, Y = 0, Z = 0;
+    if (run) {
+      if (bal == 0u) {
+        head = min(head + (uint32_t)G, lend);
+      } else {
+        head += (uint32_t)__ffs((int)bal) - 1u;
+        const uint32_t e = head & (CAP - 1);
+        const uint4 nd = __ldg(tv.node[lvl] + Q.w[0][e]);
+        cell_of(Q.w[1][e], Q.w[2][e], X, Y, Z);
+        first = nd.z;
+        n = (uint32_t)(__popc(nd.x) + __popc(nd.y));
+        ++head;
+      }
+    }
+    __syncwarp();
+    const uint32_t most = __reduce_max_sync(full, n);
+    if (most == 0) continue;
+    const uint32_t cl = max(lvl, 2u) - 1u;  // the children's level
+    const uint32_t ss = cl == 1 ? 0u : 2 * (cl - 2);
+    const int w = (1 << ss) - 1;
+    const int tx = q.x - (int)(X << (2 * lvl)), ty = q.y - (int)(Y << (2 * lvl)),
+              tz = q.z - (int)(Z << (2 * lvl));
+    const float fu = (float)(128 << ss), fw = (float)w;
+    const float lx = -fu - (float)tx, ly = -fu - (float)ty, lz = -fu - (float)tz;
+    const float hx = lx + fw, hy = ly + fw, hz = lz + fw;
+    const uint32_t w1 = X | Y << 12 | Z << 24, w2 = (Z >> 8) << 6;
+    const uint2* pc = tv.pcode[cl];
+    const uint32_t cap = tv.cap[cl];
+    for (uint32_t k0 = 0; k0 < most; k0 += G) {
+      const uint32_t ci = first + k0 + g;
+      const bool in = k0 + g < n && ci < cap;
+      uint2 v = make_uint2(0u, 0u);
+      float lb = 3.0e38f, ub = 3.0e38f;
+      if (in) {
+        v = __ldg(pc + ci);
+        if constexpr (sizeof(D) == 4) {
+          BoxBoundsF bb;
+          bb.axis<0, 1>(v.x, fu, lx, hx);
+          bb.axis<2, 3>(v.x, fu, ly, hy);
+          bb.axis<0, 1>(v.y, fu, lz, hz);
+          lb = bb.lb();
+          ub = bb.ub();
+        } else {
+          BoxBounds<D> bb;
+          bb.axis(v.x & 63u, (v.x >> 8) & 63u, tx, ss, w);
+          bb.axis((v.x >> 16) & 63u, (v.x >> 24) & 63u, ty, ss, w);
+          bb.axis(v.y & 63u, (v.y >> 8) & 63u, tz, ss, w);
+          lb = bb.lb();
+          ub = bb.ub();
+        }
+      }
+      // (a child beyond the bound cannot tighten it either)
+      if (!__any_sync(full, run && lb <= R)) continue;
+      R = fminf(R, group_least<G, float>(ub));
+      put(run && lb <= R, ci, w1, __byte_perm(v.y, __float_as_uint(lb), 0x7632u) | w2);
+      if (gave_up) n = 0;
+    }
+    __syncwarp();
+  }
+  // bricks: a lane each
+  D cd = (D)~(D)0;
+  unsigned long long ck = ~0ull;
+  const bool bricks = active && !gave_up;
+  while (__any_sync(full, bricks && head < tail)) {
+    if (bricks && head + g < tail) {
+      const uint32_t e = (head + g) & (CAP - 1);
+      const uint32_t w1 = Q.w[1][e], w2 = Q.w[2][e];
+      if ((w2 >> 16) <= (__float_as_uint(R) >> 16)) {
+        uint32_t X, Y, Z;
+        cell_of(w1, w2, X, Y, Z);
+        brick_voxels<D>(__ldg(tv.brick + Q.w[0][e]), X << 2, Y << 2, Z << 2, q, b, cd, ck);
+      }
+    }
+    R = fminf(R, bound_up(group_least<G, D>(cd)));
+    head += G;
+  }
+  __syncwarp();
+  // the least distance and the smallest key at it (all ones: none found)
+  const D least = group_least<G, D>(cd);
+  best.d2 = bricks && least != (D)~(D)0 ? least : bound_from<D>(R);
+  best.key = group_least<G, unsigned long long>(bricks && cd == least ? ck : ~0ull);
+  return gave_up;
 }
 
 // Slots of the Morton order taken by one pass of a sorted search: every
@@ -869,43 +1206,64 @@ __device__ __forceinline__ unsigned long long seed_bound(unsigned long long d0, 
 }
 
 // The seed of slot `slot` (query voxel q) in a pass with seed groups of
-// `parent` slots: the tighter of the bounds that the answers of the slot's
-// own group head and of the next group's head give (all ones: none).
+// `parent` slots: the bound that the answer of the slot's own group head (next
+// = 0) or of the next group's head (next = 1) gives (all ones: none).
 __device__ __forceinline__ unsigned long long seed_of(const NnSeg& sg, uint32_t slot,
                                                       uint32_t parent, bool sorted,
                                                       const unsigned long long* order, int qx,
-                                                      int qy, int qz) {
-  unsigned long long seed = ~0ull;
-  const uint32_t h0 = slot - slot % parent;
-#pragma unroll
-  for (uint32_t e = 0; e < 2; ++e) {
-    const uint32_t s0 = h0 + e * parent, l0 = s0 - sg.tile_base * (uint32_t)kTile;
-    if (l0 >= sg.m) continue;  // (beyond the segment's queries)
-    const uint32_t j0 = sorted ? (uint32_t)__ldg(order + s0) : l0;
-    if (j0 >= sg.m) continue;
-    const unsigned long long d0 = __ldg(sg.d2 + j0);
-    int px, py, pz;
-    if (d0 != ~0ull && query_voxel(sg, j0, px, py, pz)) {
-      seed = min(seed, seed_bound(d0, qx, qy, qz, px, py, pz));
-    }
+                                                      int qy, int qz, uint32_t next) {
+  const uint32_t s0 = slot - slot % parent + next * parent,
+                 l0 = s0 - sg.tile_base * (uint32_t)kTile;
+  if (l0 >= sg.m) return ~0ull;  // (beyond the segment's queries)
+  const uint32_t j0 = sorted ? (uint32_t)__ldg(order + s0) : l0;
+  if (j0 >= sg.m) return ~0ull;
+  const unsigned long long d0 = __ldg(sg.d2 + j0);
+  int px, py, pz;
+  if (d0 == ~0ull || !query_voxel(sg, j0, px, py, pz)) return ~0ull;
+  return seed_bound(d0, qx, qy, qz, px, py, pz);
+}
+
+// The search of every active group of the warp from its seed bound.
+template <int G, typename D>
+__device__ __forceinline__ void tree_answer(const TreeView& tv, const Qry& q, uint32_t b,
+                                            bool active, unsigned long long seed, uint32_t g,
+                                            uint32_t gm, BfsQueue<G>& Q, unsigned long long& d2,
+                                            unsigned long long& key) {
+  constexpr uint32_t full = 0xffffffffu;
+  const D none = (D)~(D)0;
+  BestKey<D> best{seed < (unsigned long long)none ? (D)seed : none, ~0ull};
+  const bool flat = active && tv.levels == 1;  // the root is the only brick
+  bool slow = search_bfs<G, D>(tv, q, b, active && !flat, g, gm, Q, best);
+  slow = slow || flat;
+  if (__any_sync(full, slow)) search_tree<G, D>(tv, q, b, slow, gm, g, best);
+  // (a bound always has a voxel at or below it; searched again without one
+  // should it not)
+  const bool again = active && best.key == ~0ull;
+  if (__any_sync(full, again)) {
+    if (again) best = BestKey<D>{none, ~0ull};
+    search_tree<G, D>(tv, q, b, again, gm, g, best);
   }
-  return seed;
+  if (active && best.key != ~0ull) {
+    d2 = best.d2;
+    key = best.key;
+  }
 }
 
 // G lanes per query slot over every segment with a tree (a segment without
 // one is left to k_nn_warp).  A warp takes 32 / G consecutive slots of the
 // pass at a time (neighbouring queries in Morton order) and moves on when all
-// are answered; the loop is warp-uniform, so that the descent's warp votes
+// are answered; the loop is warp-uniform, so that the search's warp votes
 // see every lane.  The pass takes the slots pass_slot gives; with parent > 0
 // each search starts from the bound that the answer of the slot's parent
 // group head (found by an earlier pass) gives: a bound without a voxel, so
 // the result is the same.
 template <int G>
-__global__ void __launch_bounds__(256, CGA_NN_TREE_BLOCKS)
+__global__ void __launch_bounds__(kTreeThreads, CGA_NN_TREE_BLOCKS)
     k_nn_tree(const NnSeg* __restrict__ segs, int S, NnSeg inline_seg, uint32_t total_slots,
               const unsigned long long* __restrict__ order,
               const unsigned int* __restrict__ order_err, uint32_t stride, uint32_t parent) {
   constexpr uint32_t QW = 32 / G;
+  __shared__ BfsQueue<G> s_q[kTreeThreads / G];
   const bool sorted = order != nullptr && (order_err == nullptr || *order_err == 0u);
   const uint32_t lane = threadIdx.x & 31, g = lane % G;
   const uint32_t gm = G == 32 ? 0xffffffffu : (uint32_t)((1ull << G) - 1ull) << (lane - g);
@@ -933,8 +1291,12 @@ __global__ void __launch_bounds__(256, CGA_NN_TREE_BLOCKS)
         active = false;
       }
     }
-    const unsigned long long seed =
-        parent != 0 && active ? seed_of(sg, slot, parent, sorted, order, qx, qy, qz) : ~0ull;
+    // even lanes take the seed of the slot's own head, odd lanes the next head's
+    unsigned long long seed = ~0ull;
+    if (parent != 0) {
+      if (active) seed = seed_of(sg, slot, parent, sorted, order, qx, qy, qz, g & 1u);
+      seed = group_least<G, unsigned long long>(seed);
+    }
     const uint32_t b = sg.a.bits;
     const int top = (1 << b) - 1;
     const uint32_t cqx = (uint32_t)min(max(qx, 0), top);
@@ -944,35 +1306,15 @@ __global__ void __launch_bounds__(256, CGA_NN_TREE_BLOCKS)
     unsigned long long d2 = ~0ull, key = ~0ull;
     const bool narrow = b <= 15 && (uint32_t)qx == cqx && (uint32_t)qy == cqy &&
                         (uint32_t)qz == cqz;
+    BfsQueue<G>& Q = s_q[threadIdx.x / G];
     if (__all_sync(0xffffffffu, narrow || !active)) {
-      BestKey<uint32_t> best{seed < 0xffffffffull ? (uint32_t)seed : 0xffffffffu, ~0ull};
-      search_tree<G, uint32_t>(sg.tree, qq, b, active, gm, g, best);
-      // (a seeded search always meets the group's first answer; searched
-      // again without the seed should it not)
-      const bool again = active && best.key == ~0ull && seed != ~0ull;
-      if (__any_sync(0xffffffffu, again)) {
-        if (again) best = BestKey<uint32_t>{0xffffffffu, ~0ull};
-        search_tree<G, uint32_t>(sg.tree, qq, b, again, gm, g, best);
-      }
-      if (best.key != ~0ull) {
-        d2 = best.d2;
-        key = best.key;
-      }
+      tree_answer<G, uint32_t>(sg.tree, qq, b, active, seed, g, gm, Q, d2, key);
     } else {
-      BestKey<unsigned long long> best{seed, ~0ull};
-      search_tree<G, unsigned long long>(sg.tree, qq, b, active, gm, g, best);
-      const bool again = active && best.key == ~0ull && seed != ~0ull;
-      if (__any_sync(0xffffffffu, again)) {
-        if (again) best = BestKey<unsigned long long>{~0ull, ~0ull};
-        search_tree<G, unsigned long long>(sg.tree, qq, b, again, gm, g, best);
-      }
-      if (best.key != ~0ull) {
-        d2 = best.d2;
-        key = best.key;
-      }
+      tree_answer<G, unsigned long long>(sg.tree, qq, b, active, seed, g, gm, Q, d2, key);
     }
+    const uint32_t at = stored_index<G>(sg, key, active && d2 != ~0ull, g, gm);
     if (active && g == 0) {
-      __stcs(sg.idx + j, d2 != ~0ull ? stored_index(sg, key) : 0xffffffffu);
+      __stcs(sg.idx + j, d2 != ~0ull ? at : 0xffffffffu);
       __stcs(sg.d2 + j, d2);
     }
   }
@@ -1101,7 +1443,8 @@ static uint32_t resident_blocks(uint32_t kind) {
     if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<1>, 256, 0);
     if (kind == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<2>, 256, 0);
     if (kind == 3) {
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_tree<CGA_NN_TREE_GROUP>, 256, 0);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_tree<CGA_NN_TREE_GROUP>,
+                                                        kTreeThreads, 0);
     }
     if (e != cudaSuccess || n <= 0) {
       cudaGetLastError();
@@ -1126,7 +1469,7 @@ static void launch_search(const NnSeg* d_segs, int S, const NnSeg& inline_seg,
     // in Morton order: every CGA_NN_SEED_TOP-th query, then (seeded by those)
     // every CGA_NN_SEED_MID-th, then the rest; in query order one pass
     // (neighbouring slots are not close queries)
-    constexpr uint32_t qpb = 256 / CGA_NN_TREE_GROUP;  // queries per block and round
+    constexpr uint32_t qpb = kTreeThreads / CGA_NN_TREE_GROUP;  // queries per block and round
     const uint32_t cap_blocks = sms * resident_blocks(3);
     uint32_t pstride[3], pparent[3];
     int np = 0;
@@ -1146,20 +1489,17 @@ static void launch_search(const NnSeg* d_segs, int S, const NnSeg& inline_seg,
     for (int k = 0; k < np; ++k) {
       const uint32_t n = pparent[k] == 0 ? total_slots / pstride[k]
                                          : total_slots / pstride[k] - total_slots / pparent[k];
-#if CGA_NN_HEAD_GROUP
       if (np > 1 && k == 0) {
-        constexpr uint32_t hq = 256 / CGA_NN_HEAD_GROUP;
-        k_nn_tree<CGA_NN_HEAD_GROUP><<<std::min<uint32_t>((n + hq - 1) / hq, cap_blocks), 256, 0,
-                                       stream>>>(d_segs, S, inline_seg, total_slots, order,
-                                                 order_err, pstride[k], pparent[k]);
+        constexpr uint32_t hq = kTreeThreads / CGA_NN_HEAD_GROUP;
+        k_nn_tree<CGA_NN_HEAD_GROUP><<<std::min<uint32_t>((n + hq - 1) / hq, cap_blocks),
+                                       kTreeThreads, 0, stream>>>(
+            d_segs, S, inline_seg, total_slots, order, order_err, pstride[k], pparent[k]);
         count_launch(1);
         continue;
       }
-#endif
       const uint32_t blocks = std::min<uint32_t>((n + qpb - 1) / qpb, cap_blocks);
-      k_nn_tree<CGA_NN_TREE_GROUP><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg,
-                                                               total_slots, order, order_err,
-                                                               pstride[k], pparent[k]);
+      k_nn_tree<CGA_NN_TREE_GROUP><<<blocks, kTreeThreads, 0, stream>>>(
+          d_segs, S, inline_seg, total_slots, order, order_err, pstride[k], pparent[k]);
       count_launch(1);
     }
   }

@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(kThreads) k_tree_level(
     unsigned long long* __restrict__ NP, unsigned long long* __restrict__ brick,
     uint32_t* __restrict__ bcode, uint4* __restrict__ node,
     const uint32_t* __restrict__ ccode1, const uint4* __restrict__ cnode,
-    uint2* __restrict__ cpcode, uint32_t* n_out,
-    uint32_t* look, uint32_t* counter, unsigned int* err) {
+    uint2* __restrict__ cpcode, uint32_t* __restrict__ dense, uint32_t dense_bits,
+    uint32_t* n_out, uint32_t* look, uint32_t* counter, unsigned int* err) {
   __shared__ uint32_t s_warp[kWarps];
   __shared__ uint32_t s_tile, s_excl;
   __shared__ unsigned long long s_k[kTile];
@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(kThreads) k_tree_level(
       lo |= (pos[a] * 4 + (cl >> s)) << (8 * a);
       hi |= (pos[a] * 4 + (ch >> s)) << (8 * a);
     }
-    cpcode[f] = make_uint2(pl[0] | ph[0] << 6 | pl[1] << 12 | ph[1] << 18, pl[2] | ph[2] << 6);
+    cpcode[f] = make_uint2(0x80808080u | pl[0] | ph[0] << 8 | pl[1] << 16 | ph[1] << 24,
+                           0x8080u | pl[2] | ph[2] << 8 | c << 16);
   };
   auto write_node = [&](uint32_t jj, uint32_t first, unsigned long long pr,
                         unsigned long long mask, uint32_t lo, uint32_t hi) {
@@ -137,6 +138,18 @@ __global__ void __launch_bounds__(kThreads) k_tree_level(
         box |= (((lo >> (8 * a)) & 15u) | ((hi >> (8 * a)) & 15u) << 4) << (8 * a);
       }
       node[jj] = make_uint4((uint32_t)mask, (uint32_t)(mask >> 32), first, box);
+      if (dense != nullptr) {
+        // the cell's position from its child numbers, finest level first
+        uint32_t X = 0, Y = 0, Z = 0;
+        for (uint32_t sh = 0; sh < dense_bits; sh += 2) {
+          uint32_t cx, cy, cz;
+          tree_cell((uint32_t)(pr >> (3 * sh)) & 63u, cx, cy, cz);
+          X |= cx << sh;
+          Y |= cy << sh;
+          Z |= cz << sh;
+        }
+        dense[(size_t)X << (2 * dense_bits) | Y << dense_bits | Z] = jj;
+      }
     }
   };
   uint32_t j = s_excl + off;
@@ -265,7 +278,12 @@ size_t level_words(const TreeLayout& L) {
 
 }  // namespace
 
-TreeLayout tree_layout(uint32_t bits, uint64_t cap) {
+// The position table covers the finest level (from level 2 up) whose cells
+// number at most 2^24, and at most twice the points (or 2^12): a search with a
+// bound of a few cells of that level starts at them and skips the levels above.
+// On the 20M-voxel surface world (b = 12) that is level 2, 64 MB, and takes the
+// bounds of a near query from about 240 to 60.
+TreeLayout tree_layout(uint32_t bits, uint64_t cap, bool with_dense) {
   TreeLayout L{};
   L.levels = tree_levels(bits);
   L.cap[0] = cap;
@@ -289,6 +307,18 @@ TreeLayout tree_layout(uint32_t bits, uint64_t cap) {
     L.off_pcode[l] = p;
     p += align_up(std::max<uint64_t>(L.cap[l], 1) * sizeof(uint2));
   }
+  if (with_dense && cap > 0) {
+    const uint64_t most = std::min<uint64_t>(1ull << 24, std::max<uint64_t>(1ull << 12, 2 * cap));
+    for (uint32_t l = 2; l < L.levels; ++l) {
+      const uint32_t c = 2 * (L.levels - l);  // bits per axis of a level-l cell
+      if ((1ull << (3 * c)) > most) continue;
+      L.dense_level = l;
+      L.dense_bits = c;
+      L.off_dense = p;
+      p += align_up(((size_t)4) << (3 * c));
+      break;
+    }
+  }
   L.bytes = p;
   return L;
 }
@@ -302,6 +332,9 @@ TreeView tree_view(const TreeLayout& L, void* mem) {
   for (uint32_t l = 1; l < L.levels; ++l) v.pcode[l] = reinterpret_cast<const uint2*>(b + L.off_pcode[l]);
   for (uint32_t l = 1; l <= L.levels; ++l) v.cap[l] = (uint32_t)std::max<uint64_t>(L.cap[l], 1);
   v.levels = L.levels;
+  if (L.dense_level > 0) v.dense = reinterpret_cast<const uint32_t*>(b + L.off_dense);
+  v.dense_level = L.dense_level;
+  v.dense_bits = L.dense_bits;
   return v;
 }
 
@@ -339,6 +372,9 @@ cudaError_t run_tree_build(const Levels& a, const TreeLayout& L, void* mem, void
   seg.out.hdr = a.hdr;
   cudaError_t e = cudaMemsetAsync(hdr, 0, sizeof(Header), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(lw, 0, level_words(L) * 4, stream);
+  if (e == cudaSuccess && L.dense_level > 0) {
+    e = cudaMemsetAsync(m + L.off_dense, 0xff, ((size_t)4) << (3 * L.dense_bits), stream);
+  }
   if (e == cudaSuccess) {
     e = cudaMemcpyAsync(sc.segs, &seg, sizeof(SortSeg), cudaMemcpyHostToDevice, stream);
   }
@@ -363,8 +399,9 @@ cudaError_t run_tree_build(const Levels& a, const TreeLayout& L, void* mem, void
     const uint32_t* cc1 = l == 2 ? reinterpret_cast<const uint32_t*>(m + L.off_bcode) : nullptr;
     const uint4* cn = l >= 3 ? reinterpret_cast<const uint4*>(m + L.off[l - 1]) : nullptr;
     uint2* cp = l >= 2 ? reinterpret_cast<uint2*>(m + L.off_pcode[l - 1]) : nullptr;
+    uint32_t* dn = l == L.dense_level ? reinterpret_cast<uint32_t*>(m + L.off_dense) : nullptr;
     k_tree_level<<<lt, kThreads, 0, stream>>>(buf[cur], counts + (l - 1), np, br, bc, nd, cc1, cn,
-                                             cp, counts + l, w, w + lt, herr);
+                                             cp, dn, L.dense_bits, counts + l, w, w + lt, herr);
     count_launch(1);
     w += lt + 1;
     cur ^= 1;

@@ -434,7 +434,9 @@ int cga_nn_query_batch(const cga_t* const* a, const cga_queries* q, uint32_t cou
  * input, the merge (bits, capacity of A + capacity of B); a batch looks up
  * its largest item; a pipeline looks up (largest bits, largest n) once at
  * create, for its sort and its merge alike.
- * Entries default to {8, 512, 2048}.  Host-only and thread-safe. */
+ * Entries default to {8, 512, 2048}; a merge whose entry was never set takes its
+ * partition from a rule on the grid and its inputs' capacities instead.
+ * Host-only and thread-safe. */
 typedef struct {
   uint32_t radix_bits;    /* digit width of an LSD pass: 8 or 9 (9 needs sort_threads 512) */
   uint32_t sort_threads;  /* threads per 4096-key tile: 256 (16 keys each) or 512 (8 keys each) */
@@ -449,7 +451,8 @@ typedef struct {
  * grids of `bits` per axis and element counts with n's bit length.
  * CGA_ERR_INVALID_ARG for bits outside 1..16 or a shape not listed above. */
 int cga_tuning_set(uint32_t bits, uint64_t n, const cga_tuning* t);
-/* The shape a call with (bits, n) would use now. */
+/* The shape a call with (bits, n) would use now (an entry never set: the default;
+ * merges then choose their own partition, see above). */
 int cga_tuning_get(uint32_t bits, uint64_t n, cga_tuning* out);
 
 /* Fill the entry for (g->bits, n) by measurement on the caller's cloud d_xyz

@@ -332,7 +332,9 @@ int cga_merge(const cga_t* a, const cga_t* b, const cga_allocator* A, void* stre
   P.b = b->lv;
   P.out = h->lv;
   P.spl_base = 0;
-  const uint32_t half = libcga::tuning_for(bits, a->lv.cap + b->lv.cap).merge_half;
+  const uint64_t points = a->lv.cap + b->lv.cap;
+  const uint32_t half =
+      libcga::merge_half_for(bits, points, bits, points, libcga::merge_key_level(bits));
   P.spl_a = libcga::merge_splitters(a->lv.cap, half);
   P.spl_b = libcga::merge_splitters(b->lv.cap, half);
   P.tile_base = 0;
@@ -1260,17 +1262,20 @@ int plan_merges(const cga_t* const* a, const cga_t* const* b, uint32_t count,
   pairs.assign(count, libcga::MergePair{});
   hs.assign(count, nullptr);
   uint64_t spl = 0, tiles = 0;
-  uint32_t max_bits = 1;
+  uint32_t max_bits = 1, rule_bits = 1;  // rule_bits: the largest pair's grid
   uint64_t max_in = 0;
+  bool key_level = true;
   for (uint32_t i = 0; i < count; ++i) {
     if (a[i] == nullptr || b[i] == nullptr) return CGA_ERR_INVALID_ARG;
     if (!same_grid(a[i]->grid, b[i]->grid)) return CGA_ERR_GRID_MISMATCH;
     const uint64_t cap = std::min<uint64_t>(a[i]->lv.cap + b[i]->lv.cap, pow2(3 * a[i]->grid.bits));
     if (cap > CGA_MAX_POINTS) return CGA_ERR_INVALID_ARG;
     max_bits = std::max(max_bits, a[i]->grid.bits);
+    key_level = key_level && libcga::merge_key_level(a[i]->grid.bits);
+    if (a[i]->lv.cap + b[i]->lv.cap >= max_in) rule_bits = a[i]->grid.bits;
     max_in = std::max<uint64_t>(max_in, a[i]->lv.cap + b[i]->lv.cap);
   }
-  half = libcga::tuning_for(max_bits, max_in).merge_half;
+  half = libcga::merge_half_for(max_bits, max_in, rule_bits, max_in, key_level);
   for (uint32_t i = 0; i < count; ++i) {
     const uint64_t cap = std::min<uint64_t>(a[i]->lv.cap + b[i]->lv.cap, pow2(3 * a[i]->grid.bits));
     hs[i] = new_cga(a[i]->grid, A, s, cap);
@@ -1558,14 +1563,17 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
   p->has_alloc = A != nullptr;
   if (A != nullptr) p->alloc = *A;
   // --- launch shapes: one per pipeline, from its largest item
-  uint32_t max_bits = 1;
+  uint32_t max_bits = 1, rule_bits = 1;  // rule_bits: the largest item's grid
   uint64_t max_n = 0;
+  bool key_level = true;
   for (uint32_t i = 0; i < S; ++i) {
     max_bits = std::max(max_bits, items[i].grid.bits);
+    key_level = key_level && libcga::merge_key_level(items[i].grid.bits);
+    if (items[i].n >= max_n) rule_bits = items[i].grid.bits;
     max_n = std::max<uint64_t>(max_n, items[i].n);
   }
   const libcga::Tuning tu = libcga::tuning_for(max_bits, max_n);
-  const uint32_t half = tu.merge_half;
+  const uint32_t half = libcga::merge_half_for(max_bits, max_n, rule_bits, 2 * max_n, key_level);
   // --- layout
   Bump bump;
   std::vector<size_t> lv_off(4 * (size_t)S);

@@ -47,6 +47,29 @@ Tuning tuning_for(uint32_t bits, uint64_t n) {
   return (v & kSet) ? unpack(v) : kDefaultTuning;
 }
 
+// The partition of merges whose entry was never set, from what the host knows:
+// the grid, and the points the two inputs can hold (of the largest pair of a
+// launch).  Measured per merge on GB300 (512 / 1024 / 2048, us):
+//   column level, 2 x 100k uniform points at b = 10      38.6 / 37.2 /  44.1
+//                 2 x 1M surface points at b = 12       101.6 / 78.6 /  83.8
+//                 2 x 10M surface points at b = 12        482 /  329 /   592
+//                 2 x 10M uniform points at b = 10        280 /  642 /  1069
+//   key level,    2 x 300k LiDAR points at b = 16        84.9 / 63.7 /  61.7
+//                 2 x 3M                                  348 /  218 /   176
+// Small merges want many tiles; when the points outnumber the grid's columns
+// (2^(2b)) four to one, tiles of 1024 columns hold more voxels than shared
+// memory stages and fall back to the column-by-column path.
+uint32_t merge_half_for(uint32_t bits, uint64_t n, uint32_t rule_bits, uint64_t points,
+                        bool key_level) {
+  if (bits >= 1 && bits <= 16) {
+    const uint32_t v = g_table[bits][bucket_of(n)].load(std::memory_order_relaxed);
+    if (v & kSet) return unpack(v).merge_half;
+  }
+  if (points < 150000) return 512;
+  if (key_level) return points < 3000000 ? 1024 : 2048;
+  return points >> (2 * rule_bits + 2) ? 512 : 1024;
+}
+
 void tuning_store(uint32_t bits, uint64_t n, const Tuning* t) {
   if (bits < 1 || bits > 16) return;
   g_table[bits][bucket_of(n)].store(t != nullptr ? pack(*t) : 0u, std::memory_order_relaxed);

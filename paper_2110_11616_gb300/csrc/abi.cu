@@ -485,6 +485,7 @@ libcga::SearchSeg search_segment(const cga_t* a, const float* d_q, uint64_t m) {
   sg.q = d_q;
   sg.m = (uint32_t)m;
   sg.ctab = a->ctab;
+  sg.xdir = a->xdir;
   return sg;
 }
 

@@ -223,7 +223,8 @@ struct SearchSeg {
   float off[3];
   const float* q;  // m points, float32 AoS
   uint32_t m;
-  const uint4* ctab;  // the NN column table of `a` (cga_nn_prepare) or null
+  const uint4* ctab;     // the NN column table of `a` (cga_nn_prepare) or null
+  const uint32_t* xdir;  // its x directory (cga_nn_prepare) or null
 };
 size_t radius_scratch_bytes();
 // order (or null): the queries' Morton keys of the NN search (query index in

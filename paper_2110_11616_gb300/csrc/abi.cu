@@ -305,7 +305,8 @@ int cga_build(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_
     release(h);
     return CGA_ERR_OOM;
   }
-  const libcga::SortScratch sc = libcga::sort_scratch_carve(scratch, keys, tiles, 1, key64, tu);
+  libcga::SortScratch sc = libcga::sort_scratch_carve(scratch, keys, tiles, 1, key64, tu);
+  libcga::plan_bins(&seg, 1, tiles, sc);
   const int rc = cuda_rc(libcga::run_sort_pipeline(&seg, 1, tiles, seg.passes, key64, sc, s));
   dfree(A, A != nullptr, scratch, s);
   if (rc != CGA_OK) {
@@ -1238,8 +1239,9 @@ int cga_build_batch(const cga_cloud* clouds, uint32_t count, const cga_allocator
         A, libcga::sort_scratch_bytes(keys, (uint32_t)tiles, (int)count, key64, tu.radix_bits), s);
     if (scratch == nullptr) rc = CGA_ERR_OOM;
     if (rc == CGA_OK) {
-      const libcga::SortScratch sc =
+      libcga::SortScratch sc =
           libcga::sort_scratch_carve(scratch, keys, (uint32_t)tiles, (int)count, key64, tu);
+      libcga::plan_bins(segs.data(), (int)count, (uint32_t)tiles, sc);
       rc = cuda_rc(libcga::run_sort_pipeline(segs.data(), (int)count, (uint32_t)tiles,
                                              max_passes, key64, sc, s));
       dfree(A, A != nullptr, scratch, s);
@@ -1679,6 +1681,7 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
   }
   p->build = libcga::sort_scratch_carve(base + o_build, build_tiles * libcga::kTile,
                                         (uint32_t)build_tiles, (int)(2 * S), key64, tu);
+  libcga::plan_bins(bsegs.data(), (int)(2 * S), (uint32_t)build_tiles, p->build);
   p->build_tiles = (uint32_t)build_tiles;
   p->build_passes = passes;
   p->key64 = key64;

@@ -16,6 +16,8 @@ constexpr int kRadixBits = 8;  // default digit width (and the NN query sort's)
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kRadixMaxBits = 9;
 constexpr int kMaxPasses = 6;  // 3 * 16 bits / 8 (or / 9)
+constexpr int kCounterWords = 16;  // a tile counter per pass, the compaction's, the
+                                   // jobs' and the grid barrier's
 
 // Launch shape of the sort and merge kernels, chosen per (grid bits, size
 // bucket) by measurement (cga_autotune) and held in a process-wide table.
@@ -90,6 +92,31 @@ struct SortSeg {
   uint32_t tile_base;   // first global tile index
   uint32_t num_tiles;   // tiles reserved (from the capacity)
   Levels out;           // compacted output
+  // build by bins (k_bins.cuh): the top bin_bits of a key name its bin; bins at
+  // bin_base .. of the bin tables, partition tiles from ptile_base, job slots
+  // [job_base, + job_cap)
+  uint32_t bin_bits, bin_base, ptile_base, job_base, job_cap;
+  uint32_t narrow;      // its partitioned keys have 32 bits
+  uint32_t fallback;    // set on the device: sort this segment the general way
+};
+
+// Tables of a build by bins, laid over the look-back words that only the general
+// sort uses.
+struct BinPlan {
+  bool on;            // the build takes this path
+  bool narrow, wide;  // some segments' partitioned keys have 32 bits, some 64
+  bool may_split;     // some segment has more points than a block sorts
+  uint32_t items;     // points per thread of a partition tile: 4, 8 or 16
+  uint32_t ptiles;    // partition tiles of all segments
+  uint32_t slots;     // job slots of all segments
+  uint32_t* cnt;      // points per bin (zeroed before each run)
+  uint32_t zero_words;
+  uint32_t* start;    // offset of each bin (one more per segment)
+  uint32_t* cur;      // next free place of each bin
+  uint4* jobs;
+  uint2* big;         // bins to split (the first word: how many)
+  uint4* info;        // per job: where its distinct keys are, voxels, columns, slabs
+  uint32_t* njobs;    // per segment
 };
 
 // Scratch layout of one sort-pipeline run (all offsets from one base).
@@ -99,12 +126,16 @@ struct SortScratch {
   uint32_t* hist;      // [S][kMaxPasses][2^radix_bits]
   uint32_t* look;      // [kMaxPasses][total_tiles][2^radix_bits]
   uint32_t* clook;     // [total_tiles][3]
-  uint32_t* counters;  // [kMaxPasses + 1]
+  uint32_t* counters;  // [kCounterWords]
   SortSeg* segs;       // [S]
   size_t zero_bytes;   // bytes from hist to the end of counters
   uint32_t radix_bits;    // launch shape of the passes (Tuning)
   uint32_t sort_threads;
+  BinPlan bins;
 };
+// Decide whether the S builds of h_segs go by bins and lay the tables out in sc
+// (fills the segments' bin fields; call before they are uploaded).
+void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc);
 
 // Scratch of a sort run; the digit width sizes the histogram and look-back
 // tables, the thread count only selects the pass kernel.

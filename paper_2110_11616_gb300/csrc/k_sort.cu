@@ -11,21 +11,13 @@
 #include <algorithm>
 #include <mutex>
 
+#include "k_bins.cuh"
 #include "k_compact.cuh"
 #include "k_walk.cuh"
 
 namespace libcga {
 
 namespace {
-
-__device__ __forceinline__ int find_seg(const SortSeg* __restrict__ segs, int S, uint32_t t) {
-  int lo = 0, hi = S - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (segs[mid].tile_base <= t) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
 
 // Element count of a segment: known on the host for a build, read from the
 // source header for a projection (the source is built earlier in the stream).
@@ -47,19 +39,16 @@ __global__ void k_seg_init(const SortSeg* __restrict__ segs, int S) {
 }
 
 // Keys of the tiles [t0, t1) plus per-segment histograms of every pass
-// (digits of RB bits).
+// (digits of RB bits).  marked: only the segments marked for the general sort.
 template <typename K, int RB>
-__global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restrict__ segs, int S,
-                                                        uint32_t total_tiles,
-                                                        uint32_t tiles_per_cta, K* keys0,
-                                                        uint32_t* hist) {
+__device__ __forceinline__ void keys_hist_tiles(const SortSeg* __restrict__ segs, int S,
+                                                uint32_t t0, uint32_t t1, K* keys0,
+                                                uint32_t* hist, bool marked) {
   constexpr int R = 1 << RB;
   __shared__ uint32_t s_hist[kMaxPasses][R];
   __shared__ float s_pts[kThreads * 3];
   __shared__ uint32_t s_err;
   const int tid = threadIdx.x;
-  const uint32_t t0 = blockIdx.x * tiles_per_cta;
-  const uint32_t t1 = min(t0 + tiles_per_cta, total_tiles);
   if (t0 >= t1) return;
   for (int i = tid; i < kMaxPasses * R; i += kThreads) (&s_hist[0][0])[i] = 0;
   if (tid == 0) s_err = 0;
@@ -88,6 +77,7 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
       cur = s;
     }
     const SortSeg& sg = segs[s];
+    if (marked && !sg.fallback) continue;
     const uint32_t n = seg_count(sg);
     const uint32_t start = (t - sg.tile_base) * kTile;
     if (start >= n) continue;
@@ -159,23 +149,13 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
   flush(cur);
 }
 
-// Exclusive scan across a block of TH threads (s_warp: TH/32 words).
-template <int TH, typename T>
-__device__ __forceinline__ T block_scan_th(T v, T& total, T* s_warp) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  T inc = warp_incl_scan(v);
-  if (lane == 31) s_warp[w] = inc;
-  __syncthreads();
-  T before = 0, tot = 0;
-#pragma unroll
-  for (int i = 0; i < TH / 32; ++i) {
-    const T x = s_warp[i];
-    if (i < w) before += x;
-    tot += x;
-  }
-  __syncthreads();
-  total = tot;
-  return before + inc - v;
+template <typename K, int RB>
+__global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restrict__ segs, int S,
+                                                        uint32_t total_tiles,
+                                                        uint32_t tiles_per_cta, K* keys0,
+                                                        uint32_t* hist) {
+  const uint32_t t0 = blockIdx.x * tiles_per_cta;
+  keys_hist_tiles<K, RB>(segs, S, t0, min(t0 + tiles_per_cta, total_tiles), keys0, hist, false);
 }
 
 // Dynamic shared memory of one pass block: the tile's keys, per-warp digit
@@ -197,15 +177,14 @@ constexpr size_t onesweep_smem() {
 #define CGA_SORT_BLOCKS_256 5
 #endif
 
-// One LSD pass over digit `pass` (RB bits) of every segment that still needs
-// it.  A tile of kTile keys is TH threads x kTile/TH keys (warp-striped);
-// threads tid < 2^RB own one digit each for the per-digit steps.
+// One tile of an LSD pass over digit `pass` (RB bits): kTile keys as TH threads
+// x kTile/TH keys (warp-striped); threads tid < 2^RB own one digit each for the
+// per-digit steps.
 template <typename K, int TH, int RB>
-__global__ void __launch_bounds__(TH, TH == 512 ? CGA_SORT_BLOCKS_512 : CGA_SORT_BLOCKS_256) k_onesweep(const SortSeg* __restrict__ segs, int S,
-                                                 int pass, const K* __restrict__ in,
-                                                 K* __restrict__ out,
-                                                 const uint32_t* __restrict__ hist,
-                                                 uint32_t* look, uint32_t* counter) {
+__device__ __forceinline__ void onesweep_tile(const SortSeg* __restrict__ segs, int s, uint32_t t,
+                                              int pass, const K* __restrict__ in,
+                                              K* __restrict__ out,
+                                              const uint32_t* __restrict__ hist, uint32_t* look) {
   constexpr int IT = kTile / TH, WARPS = TH / 32, R = 1 << RB;
   static_assert(IT * TH == kTile && TH >= R, "tile shape");
   extern __shared__ __align__(16) unsigned char s_raw[];
@@ -214,18 +193,9 @@ __global__ void __launch_bounds__(TH, TH == 512 ? CGA_SORT_BLOCKS_512 : CGA_SORT
   uint32_t* s_off = reinterpret_cast<uint32_t*>(s_raw + (size_t)kTile * sizeof(K) +
                                                 (size_t)WARPS * R * 2);
   uint32_t* s_scan = s_off + R;
-  __shared__ uint32_t s_tile;
-  __shared__ int s_seg;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (tid == 0) {
-    const uint32_t t = atomicAdd(counter, 1u);
-    s_tile = t;
-    s_seg = find_seg(segs, S, t);
-  }
   for (int i = tid; i < WARPS * R; i += TH) (&s_wh[0][0])[i] = 0;
   __syncthreads();
-  const uint32_t t = s_tile;
-  const int s = s_seg;
   const SortSeg& sg = segs[s];
   if (pass >= (int)sg.passes) return;
   const uint32_t n = seg_count(sg);
@@ -311,30 +281,36 @@ __global__ void __launch_bounds__(TH, TH == 512 ? CGA_SORT_BLOCKS_512 : CGA_SORT
   if (bad) atomicOr(&sg.out.hdr->err, kErrInternal);
 }
 
-
-template <typename K, int LEVELS>
-__global__ void __launch_bounds__(kThreads) k_compact(const SortSeg* __restrict__ segs, int S,
-                                                      const K* __restrict__ keys0,
-                                                      const K* __restrict__ keys1,
-                                                      uint32_t* clook, uint32_t* counter) {
-  __shared__ CompactSmem sm;
+// One LSD pass over every segment that still needs it, a tile per block.
+template <typename K, int TH, int RB>
+__global__ void __launch_bounds__(TH, TH == 512 ? CGA_SORT_BLOCKS_512 : CGA_SORT_BLOCKS_256)
+    k_onesweep(const SortSeg* __restrict__ segs, int S, int pass, const K* __restrict__ in,
+               K* __restrict__ out, const uint32_t* __restrict__ hist, uint32_t* look,
+               uint32_t* counter) {
   __shared__ uint32_t s_tile;
   __shared__ int s_seg;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     const uint32_t t = atomicAdd(counter, 1u);
     s_tile = t;
     s_seg = find_seg(segs, S, t);
   }
   __syncthreads();
-  const uint32_t t = s_tile;
-  const SortSeg& sg = segs[s_seg];
+  onesweep_tile<K, TH, RB>(segs, s_seg, s_tile, pass, in, out, hist, look);
+}
+
+// Dedupe and compaction of one tile of sorted keys (src: the segment's sorted
+// key buffer).
+template <typename K, int LEVELS>
+__device__ __forceinline__ void compact_sorted_tile(const SortSeg& sg, uint32_t t,
+                                                    const K* __restrict__ sorted,
+                                                    uint32_t* clook, CompactSmem& sm) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t n = seg_count(sg);
   const uint32_t lt = t - sg.tile_base;
   const uint32_t start = lt * kTile;
   if (start >= n) return;
   const uint32_t cnt = min((uint32_t)kTile, n - start);
-  const K* src = ((sg.passes & 1u) ? keys1 : keys0) + sg.key_base + start;
+  const K* src = sorted + sg.key_base + start;
   K k[kItems];
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
@@ -345,6 +321,79 @@ __global__ void __launch_bounds__(kThreads) k_compact(const SortSeg* __restrict_
   const K prev = has_prev ? src[-1] : (K)0;
   const bool last = (start + cnt == n);
   compact_tile<LEVELS, K>(k, cnt, has_prev, prev, t, sg.tile_base, last, sg.out, clook, sm);
+}
+
+template <typename K, int LEVELS>
+__global__ void __launch_bounds__(kThreads) k_compact(const SortSeg* __restrict__ segs, int S,
+                                                      const K* __restrict__ keys0,
+                                                      const K* __restrict__ keys1,
+                                                      uint32_t* clook, uint32_t* counter) {
+  __shared__ CompactSmem sm;
+  __shared__ uint32_t s_tile;
+  __shared__ int s_seg;
+  if (threadIdx.x == 0) {
+    const uint32_t t = atomicAdd(counter, 1u);
+    s_tile = t;
+    s_seg = find_seg(segs, S, t);
+  }
+  __syncthreads();
+  const SortSeg& sg = segs[s_seg];
+  compact_sorted_tile<K, LEVELS>(sg, s_tile, (sg.passes & 1u) ? keys1 : keys0, clook, sm);
+}
+
+// The general sort of the segments that a build by bins marked (usually none:
+// the blocks look and leave): key generation, the 8-bit radix passes and the
+// compaction in one cooperative launch, a grid barrier between the steps.  The
+// tables of the bins lie in the look-back words, so those are cleared here.
+constexpr int kLsdBarrier = kMaxPasses + 2;  // its word of the counters
+template <typename K>
+__global__ void __launch_bounds__(kThreads, 4)
+    k_lsd_all(SortSeg* segs, int S, uint32_t total_tiles, uint32_t max_passes, K* keys0, K* keys1,
+              uint32_t* hist, uint32_t* look, uint32_t* clook, uint32_t* counters,
+              uint32_t zero_words) {
+  __shared__ CompactSmem sm;
+  __shared__ uint32_t s_tile;
+  __shared__ int s_seg;
+  const int tid = threadIdx.x;
+  int any = 0;
+  for (int s = tid; s < S; s += kThreads) any |= (int)segs[s].fallback;
+  if (!__syncthreads_or(any)) return;
+  unsigned int* err = &segs[0].out.hdr->err;
+  uint32_t round = 0;
+  // hist, look and clook lie side by side, up to the counters
+  for (uint32_t i = blockIdx.x * kThreads + tid; i < zero_words; i += gridDim.x * kThreads) {
+    hist[i] = 0;
+  }
+  if (blockIdx.x == 0 && tid <= kMaxPasses) counters[tid] = 0;
+  if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
+  const uint32_t per = (total_tiles + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * per;
+  keys_hist_tiles<K, 8>(segs, S, t0, min(t0 + per, total_tiles), keys0, hist, true);
+  if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
+  for (uint32_t p = 0; p <= max_passes; ++p) {
+    // pass p, and after the last one the compaction
+    const uint32_t c = p < max_passes ? p : (uint32_t)kMaxPasses;
+    for (;;) {
+      __syncthreads();
+      if (tid == 0) {
+        const uint32_t t = atomicAdd(counters + c, 1u);
+        s_tile = t;
+        s_seg = t < total_tiles ? find_seg(segs, S, t) : 0;
+      }
+      __syncthreads();
+      const uint32_t t = s_tile;
+      if (t >= total_tiles) break;
+      const SortSeg& sg = segs[s_seg];
+      if (!sg.fallback) continue;
+      if (p < max_passes) {
+        onesweep_tile<K, kThreads, 8>(segs, s_seg, t, (int)p, (p & 1) ? keys1 : keys0,
+                                      (p & 1) ? keys0 : keys1, hist,
+                                      look + ((size_t)p * total_tiles << 8));
+      } else {
+        compact_sorted_tile<K, 3>(sg, t, (sg.passes & 1u) ? keys1 : keys0, clook, sm);
+      }
+    }
+    if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
+  }
 }
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -360,7 +409,7 @@ size_t sort_scratch_bytes(uint64_t total_keys, uint32_t total_tiles, int S, bool
   b += align_up((size_t)S * kMaxPasses * R * 4);
   b += align_up((size_t)kMaxPasses * total_tiles * R * 4);
   b += align_up((size_t)total_tiles * 3 * 4);
-  b += align_up((kMaxPasses + 1) * 4);
+  b += align_up(kCounterWords * 4);
   b += align_up((size_t)S * sizeof(SortSeg));
   return b;
 }
@@ -385,7 +434,7 @@ SortScratch sort_scratch_carve(void* base, uint64_t total_keys, uint32_t total_t
   sc.clook = reinterpret_cast<uint32_t*>(p);
   p += align_up((size_t)total_tiles * 3 * 4);
   sc.counters = reinterpret_cast<uint32_t*>(p);
-  p += align_up((kMaxPasses + 1) * 4);
+  p += align_up(kCounterWords * 4);
   sc.zero_bytes = (size_t)(p - z0);
   sc.segs = reinterpret_cast<SortSeg*>(p);
   return sc;
@@ -436,6 +485,191 @@ static void launch_passes(int S, uint32_t total_tiles, uint32_t max_passes, cons
   }
 }
 
+// Resident blocks of the bin kernels (set by init_bin_kernels): the job sorts of
+// 32- and 64-bit keys, and the general sort behind them.
+static uint32_t g_bin_sort_blocks[2], g_lsd_blocks[2];
+
+template <typename F>
+static cudaError_t resident(F* kernel, int threads, size_t smem, uint32_t* blocks) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int n = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem);
+  if (e == cudaSuccess && n <= 0) e = cudaErrorInvalidConfiguration;
+  if (blocks != nullptr) *blocks = (uint32_t)std::max(n, 1) * (uint32_t)device_sm_count();
+  return e;
+}
+
+static cudaError_t init_bin_kernels() {
+  const cudaError_t es[] = {
+      resident(k_bin_sort<uint32_t>, kBinThreads, bin_sort_smem<uint32_t>(), &g_bin_sort_blocks[0]),
+      resident(k_bin_sort<unsigned long long>, kBinThreads, bin_sort_smem<unsigned long long>(),
+               &g_bin_sort_blocks[1]),
+      resident(k_bin_part<uint32_t, 4>, 1024, bin_part_smem<uint32_t, 4>(), nullptr),
+      resident(k_bin_part<uint32_t, 8>, 1024, bin_part_smem<uint32_t, 8>(), nullptr),
+      resident(k_bin_part<uint32_t, 16>, 1024, bin_part_smem<uint32_t, 16>(), nullptr),
+      resident(k_bin_part<unsigned long long, 4>, 1024, bin_part_smem<unsigned long long, 4>(), nullptr),
+      resident(k_bin_part<unsigned long long, 8>, 1024, bin_part_smem<unsigned long long, 8>(), nullptr),
+      resident(k_bin_part<unsigned long long, 16>, 1024, bin_part_smem<unsigned long long, 16>(), nullptr),
+      resident(k_lsd_all<uint32_t>, kThreads, onesweep_smem<uint32_t, kThreads, 8>(), &g_lsd_blocks[0]),
+      resident(k_lsd_all<unsigned long long>, kThreads,
+               onesweep_smem<unsigned long long, kThreads, 8>(), &g_lsd_blocks[1])};
+  for (cudaError_t e : es) {
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// Points per segment up to which a build goes by bins: beyond, a bin of the
+// widest table (2^12) holds more than a block sorts.
+constexpr uint64_t kBinMaxPoints = 1ull << 25;
+
+void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
+  BinPlan& B = sc.bins;
+  B = BinPlan{};
+  if (S <= 0 || total_tiles == 0) return;
+  // bins of about 64 points, no finer than a slab (whole slabs per bin), and 32-bit
+  // keys where a bin and 32 bits give the key with room for four bins a job.  On
+  // average a bin may hold a few blocks' worth of points (30M points at b = 10, 29k a
+  // bin: 1377 us by the general sort, 1368 by bins); beyond that every bin goes to a
+  // cluster, which the general sort beats (15k a bin that way: 747 against 1190).
+  uint64_t points = 0;
+  for (int s = 0; s < S; ++s) {
+    SortSeg& g = h_segs[s];
+    if (g.from_cga || g.n_host > kBinMaxPoints) return;
+    uint32_t t = 4;
+    while (t < kBinMaxBits && ((uint64_t)64 << t) < g.n_host) ++t;
+    g.bin_bits = std::min(t, g.bits);
+    g.narrow = 3 * g.bits - g.bin_bits <= 30 ? 1u : 0u;
+    const uint64_t most = g.narrow ? 4 * bin_cap<uint32_t>() : 4 * bin_cap<unsigned long long>();
+    if (g.n_host >> g.bin_bits > most) return;
+    B.may_split = B.may_split || g.n_host > (g.narrow ? bin_cap<uint32_t>() : bin_cap<unsigned long long>());
+    B.narrow = B.narrow || g.narrow;
+    B.wide = B.wide || !g.narrow;
+    points += g.n_host;
+  }
+  // partition tiles: enough of them for the SMs, then as many keys a bin as possible
+  const uint64_t sms = (uint64_t)device_sm_count();
+  B.items = points >= sms * 4 * 16384 ? 16u : (points >= sms * 2 * 8192 ? 8u : 4u);
+  uint64_t bins = 0, slots = 0, ptiles = 0, most_big = 0;
+  for (int s = 0; s < S; ++s) {
+    SortSeg& g = h_segs[s];
+    const uint32_t nb = 1u << g.bin_bits, rem = 3 * g.bits - g.bin_bits;
+    const uint32_t span = g.narrow ? std::min(32u - rem, kBinMaxBits) : kBinMaxBits;
+    const uint32_t target = g.narrow ? bin_target<uint32_t>() : bin_target<unsigned long long>();
+    g.bin_base = (uint32_t)bins;
+    g.ptile_base = (uint32_t)ptiles;
+    g.job_base = (uint32_t)slots;
+    // a job per target's worth of points, two around each larger bin, one per span,
+    // and a split bin's slots
+    g.job_cap = 7 * (g.n_host / target + 1) + (nb >> span) + 4;
+    most_big += g.n_host / (2 * target);
+    bins += nb + 1;
+    slots += g.job_cap;
+    ptiles += (g.n_host + 1024ull * B.items - 1) / (1024ull * B.items);
+    // the general sort behind the bins has 8-bit digits
+    g.passes = radix_passes(g.key_bits, 8);
+  }
+  const size_t room = (size_t)kMaxPasses * total_tiles * ((size_t)4 << sc.radix_bits);
+  char* p = reinterpret_cast<char*>(sc.look);
+  auto take = [&](size_t bytes) {
+    char* r = p;
+    p += align_up(bytes);
+    return r;
+  };
+  B.cnt = reinterpret_cast<uint32_t*>(take(bins * 4));
+  B.big = reinterpret_cast<uint2*>(take((most_big + 1) * 8));
+  B.zero_words = (uint32_t)((p - reinterpret_cast<char*>(sc.look)) / 4);
+  B.start = reinterpret_cast<uint32_t*>(take(bins * 4));
+  B.cur = reinterpret_cast<uint32_t*>(take(bins * 4));
+  B.jobs = reinterpret_cast<uint4*>(take(slots * 16));
+  B.info = reinterpret_cast<uint4*>(take(slots * 16));
+  B.njobs = reinterpret_cast<uint32_t*>(take((size_t)S * 4));
+  if ((size_t)(p - reinterpret_cast<char*>(sc.look)) > room || slots > 0x7fffffffull) return;
+  B.ptiles = (uint32_t)ptiles;
+  B.slots = (uint32_t)slots;
+  B.on = true;
+}
+
+template <typename T>
+static void launch_part(int S, const SortScratch& sc, uint32_t stride, cudaStream_t stream) {
+  const BinPlan& B = sc.bins;
+  T* keys = static_cast<T*>(sc.keys0);
+  if (B.items == 16) {
+    k_bin_part<T, 16><<<B.ptiles, 1024, bin_part_smem<T, 16>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+  } else if (B.items == 8) {
+    k_bin_part<T, 8><<<B.ptiles, 1024, bin_part_smem<T, 8>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+  } else {
+    k_bin_part<T, 4><<<B.ptiles, 1024, bin_part_smem<T, 4>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+  }
+}
+
+template <typename T>
+static void launch_bin_jobs(int S, const SortScratch& sc, uint32_t stride, uint32_t* counter,
+                            cudaStream_t stream) {
+  const BinPlan& B = sc.bins;
+  T *k0 = static_cast<T*>(sc.keys0), *k1 = static_cast<T*>(sc.keys1);
+  k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.start, B.cur, B.jobs, B.njobs, B.big);
+  launch_part<T>(S, sc, stride, stream);
+  if (B.may_split) {
+    const unsigned clusters = std::max(1u, 3 * (unsigned)device_sm_count() / kBinCluster);
+    k_bin_split<T><<<clusters * kBinCluster, kBinThreads, 0, stream>>>(
+        sc.segs, B.jobs, B.big, k0, k1, stride);
+  }
+  const uint32_t blocks = std::min<uint32_t>(B.slots, g_bin_sort_blocks[sizeof(T) / 8]);
+  k_bin_sort<T><<<blocks, kBinThreads, bin_sort_smem<T>(), stream>>>(
+      sc.segs, S, B.jobs, B.njobs, k0, k1, B.info, counter, B.slots, stride);
+}
+
+template <typename T>
+static void launch_bin_write(int S, const SortScratch& sc, uint32_t stride, cudaStream_t stream) {
+  const BinPlan& B = sc.bins;
+  const T *k0 = static_cast<const T*>(sc.keys0), *k1 = static_cast<const T*>(sc.keys1);
+  k_bin_write<T><<<std::min<uint32_t>(B.slots, (uint32_t)device_sm_count() * 8), kThreads, 0,
+                   stream>>>(sc.segs, S, B.jobs, B.njobs, k0, k1, B.info, B.slots, stride);
+}
+
+template <typename K>
+static cudaError_t launch_lsd_all(int S, uint32_t total_tiles, const SortScratch& sc,
+                                  cudaStream_t stream) {
+  SortSeg* segs = sc.segs;
+  K *k0 = static_cast<K*>(sc.keys0), *k1 = static_cast<K*>(sc.keys1);
+  uint32_t passes = kMaxPasses, *hist = sc.hist, *look = sc.look, *clook = sc.clook,
+           *counters = sc.counters;
+  uint32_t words = (uint32_t)((reinterpret_cast<char*>(sc.counters) -
+                               reinterpret_cast<char*>(sc.hist)) / 4);
+  void* args[] = {&segs, &S, &total_tiles, &passes, &k0, &k1, &hist, &look, &clook, &counters, &words};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_lsd_all<K>),
+                                     dim3(g_lsd_blocks[sizeof(K) / 8]), dim3(kThreads), args,
+                                     onesweep_smem<K, kThreads, 8>(), stream);
+}
+
+// The build by bins (the plan is laid out, the segment table uploaded).
+static cudaError_t run_bins(int S, uint32_t total_tiles, bool key64, const SortScratch& sc,
+                            cudaStream_t stream) {
+  const cudaError_t ei = init_sort_kernels();
+  if (ei != cudaSuccess) return ei;
+  const BinPlan& B = sc.bins;
+  const uint32_t sms = (uint32_t)device_sm_count(), stride = key64 ? 8u : 4u;
+  const uint32_t zb = std::min<uint32_t>((std::max<uint32_t>(B.zero_words, (uint32_t)S) + 255) / 256,
+                                         sms * 8);
+  k_bin_init<<<zb, 256, 0, stream>>>(sc.segs, S, B.cnt, B.zero_words, sc.counters);
+  const uint32_t ctas = std::min<uint32_t>(total_tiles, sms * 4);
+  k_bin_hist<<<ctas, kBinThreads, 0, stream>>>(sc.segs, S, total_tiles,
+                                               (total_tiles + ctas - 1) / ctas, B.cnt);
+  // a launch for each key width in the batch
+  if (B.narrow) launch_bin_jobs<uint32_t>(S, sc, stride, sc.counters + kMaxPasses + 1, stream);
+  if (B.wide) launch_bin_jobs<unsigned long long>(S, sc, stride, sc.counters + kMaxPasses + 3, stream);
+  if (B.narrow) launch_bin_write<uint32_t>(S, sc, stride, stream);
+  if (B.wide) launch_bin_write<unsigned long long>(S, sc, stride, stream);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) {
+    e = key64 ? launch_lsd_all<unsigned long long>(S, total_tiles, sc, stream)
+              : launch_lsd_all<uint32_t>(S, total_tiles, sc, stream);
+  }
+  count_launch(3 + (B.may_split ? 5 : 4) * ((B.narrow ? 1 : 0) + (B.wide ? 1 : 0)));
+  return e;
+}
+
 cudaError_t init_sort_kernels() {
   static std::once_flag once;
   static cudaError_t rc = cudaSuccess;
@@ -447,6 +681,8 @@ cudaError_t init_sort_kernels() {
     for (cudaError_t e : es) {
       if (e != cudaSuccess && rc == cudaSuccess) rc = e;
     }
+    const cudaError_t eb = init_bin_kernels();
+    if (eb != cudaSuccess && rc == cudaSuccess) rc = eb;
   });
   return rc;
 }
@@ -516,6 +752,7 @@ cudaError_t run_sort_keys_device(int S, uint32_t total_tiles, uint32_t max_passe
 
 cudaError_t run_sort_device(int S, uint32_t total_tiles, uint32_t max_passes, bool key64,
                             int levels, const SortScratch& sc, cudaStream_t stream) {
+  if (sc.bins.on && total_tiles > 0) return run_bins(S, total_tiles, key64, sc, stream);
   cudaError_t e = cudaMemsetAsync(sc.hist, 0, sc.zero_bytes, stream);
   if (e != cudaSuccess) return e;
   k_seg_init<<<(S + 127) / 128, 128, 0, stream>>>(sc.segs, S);

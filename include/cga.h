@@ -268,9 +268,10 @@ int cga_decode(const cga_t* a, uint32_t* d_xyz, void* stream);
 #define CGA_MERGE_AVERAGE 1
 
 /* cga_build plus the Value array.  d_attr: n * channels uint8 rows, device,
- * point order (the same points as d_xyz).  Each point finds its voxel by the
- * Sec. V-A lookup; sums are exact integers, so the result does not depend
- * on arrival order.  Errors as cga_build; CGA_ERR_INVALID_ARG for channels or
+ * point order (the same points as d_xyz).  Rows are summed per voxel along with
+ * the build's sort or, where its scratch and the sort's cannot be had at once or the
+ * sort is not by bins, afterwards by the Sec. V-A lookup; sums are exact integers, so
+ * the result does not depend on arrival order.  Errors as cga_build; CGA_ERR_INVALID_ARG for channels or
  * policy out of range or a NULL d_attr with n > 0. */
 int cga_build_values(const float* d_xyz, const uint8_t* d_attr, uint32_t channels, uint64_t n,
                      const cga_grid* g, const float* h_xform12, int policy,

@@ -242,35 +242,18 @@ void attach_coarse(const cga* a, libcga::NnSeg& seg) {
   }
 }
 
-}  // namespace
+// What a build fills along with the levels: the Value array, with scratch of two words
+// a point and at least value_scratch_bytes; done: it has (else that is left to
+// run_build_values).
+struct ValueBuild {
+  libcga::ValueInput in;
+  void* scratch;
+  uint8_t* values;
+  bool done;
+};
 
-namespace libcga {
-// The NN search structures prepared on a handle (x directory, column table,
-// coarse levels or occupancy tree), for entry points in other files.
-void nn_attach(const cga_t* a, NnSeg& seg) { attach_coarse(a, seg); }
-}  // namespace libcga
-
-extern "C" {
-
-int cga_grid_from_box(const float lo[3], float extent, uint32_t bits, cga_grid* out) {
-  if (lo == nullptr || out == nullptr || bits < 1 || bits > 16) return CGA_ERR_INVALID_ARG;
-  if (!std::isfinite(extent) || !(extent > 0.0f)) return CGA_ERR_INVALID_ARG;
-  const float s = (float)(1u << bits) / extent;
-  if (!std::isfinite(s)) return CGA_ERR_INVALID_ARG;
-  cga_grid g{};
-  g.bits = bits;
-  g.scale = s;
-  for (int a = 0; a < 3; ++a) {
-    if (!std::isfinite(lo[a])) return CGA_ERR_INVALID_ARG;
-    const float prod = lo[a] * s;
-    g.offset[a] = -prod;
-  }
-  *out = g;
-  return CGA_OK;
-}
-
-int cga_build(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_xform12,
-              const cga_allocator* A, void* stream, cga_t** out) {
+int build_cloud(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_xform12,
+                const cga_allocator* A, void* stream, ValueBuild* vb, cga_t** out) {
   if (out == nullptr || !grid_ok(g) || n > CGA_MAX_POINTS || (n > 0 && d_xyz == nullptr)) {
     return CGA_ERR_INVALID_ARG;
   }
@@ -307,6 +290,13 @@ int cga_build(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_
   }
   libcga::SortScratch sc = libcga::sort_scratch_carve(scratch, keys, tiles, 1, key64, tu);
   libcga::plan_bins(&seg, 1, tiles, sc);
+  if (vb != nullptr && sc.bins.on) {
+    sc.bins.value_in = vb->in;
+    sc.bins.value_out = h->lv;
+    sc.bins.values = vb->values;
+    sc.bins.value_rows = static_cast<uint32_t*>(vb->scratch);
+    vb->done = true;
+  }
   const int rc = cuda_rc(libcga::run_sort_pipeline(&seg, 1, tiles, seg.passes, key64, sc, s));
   dfree(A, A != nullptr, scratch, s);
   if (rc != CGA_OK) {
@@ -315,6 +305,38 @@ int cga_build(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_
   }
   *out = h;
   return CGA_OK;
+}
+
+}  // namespace
+
+namespace libcga {
+// The NN search structures prepared on a handle (x directory, column table,
+// coarse levels or occupancy tree), for entry points in other files.
+void nn_attach(const cga_t* a, NnSeg& seg) { attach_coarse(a, seg); }
+}  // namespace libcga
+
+extern "C" {
+
+int cga_grid_from_box(const float lo[3], float extent, uint32_t bits, cga_grid* out) {
+  if (lo == nullptr || out == nullptr || bits < 1 || bits > 16) return CGA_ERR_INVALID_ARG;
+  if (!std::isfinite(extent) || !(extent > 0.0f)) return CGA_ERR_INVALID_ARG;
+  const float s = (float)(1u << bits) / extent;
+  if (!std::isfinite(s)) return CGA_ERR_INVALID_ARG;
+  cga_grid g{};
+  g.bits = bits;
+  g.scale = s;
+  for (int a = 0; a < 3; ++a) {
+    if (!std::isfinite(lo[a])) return CGA_ERR_INVALID_ARG;
+    const float prod = lo[a] * s;
+    g.offset[a] = -prod;
+  }
+  *out = g;
+  return CGA_OK;
+}
+
+int cga_build(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_xform12,
+              const cga_allocator* A, void* stream, cga_t** out) {
+  return build_cloud(d_xyz, n, g, h_xform12, A, stream, nullptr, out);
 }
 
 int cga_merge(const cga_t* a, const cga_t* b, const cga_allocator* A, void* stream,
@@ -365,35 +387,57 @@ int cga_build_values(const float* d_xyz, const uint8_t* d_attr, uint32_t channel
       (policy != CGA_VALUE_AVERAGE && policy != CGA_VALUE_FIRST) || (n > 0 && d_attr == nullptr)) {
     return CGA_ERR_INVALID_ARG;
   }
-  cga_t* h = nullptr;
-  int rc = cga_build(d_xyz, n, g, h_xform12, A, stream, &h);
-  if (rc != CGA_OK) return rc;
+  if (!grid_ok(g) || n > CGA_MAX_POINTS || (n > 0 && d_xyz == nullptr) ||
+      (A != nullptr && (A->alloc == nullptr || A->free == nullptr))) {
+    return CGA_ERR_INVALID_ARG;
+  }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const uint64_t cap = std::max<uint64_t>(h->lv.cap, 1);
-  void* vm = dalloc(A, cap * channels, s);
-  void* scratch = dalloc(A, libcga::value_scratch_bytes(h->lv.cap, channels, policy), s);
-  if (vm == nullptr || scratch == nullptr) {
-    if (vm) dfree(A, A != nullptr, vm, s);
-    if (scratch) dfree(A, A != nullptr, scratch, s);
-    release(h);
-    return CGA_ERR_OOM;
-  }
-  libcga::ValueInput in{};
-  in.xyz = d_xyz;
-  in.attr = d_attr;
-  in.n = n;
-  in.channels = channels;
-  in.policy = policy;
-  in.scale = g->scale;
-  for (int k = 0; k < 3; ++k) in.off[k] = g->offset[k];
+  const uint64_t cap = std::max<uint64_t>(n, 1);
+  ValueBuild vb{};
+  vb.in.xyz = d_xyz;
+  vb.in.attr = d_attr;
+  vb.in.n = n;
+  vb.in.channels = channels;
+  vb.in.policy = policy;
+  vb.in.scale = g->scale;
+  for (int k = 0; k < 3; ++k) vb.in.off[k] = g->offset[k];
   if (h_xform12 != nullptr) {
-    std::memcpy(in.X, h_xform12, sizeof(in.X));
-    in.has_x = 1;
+    std::memcpy(vb.in.X, h_xform12, sizeof(vb.in.X));
+    vb.in.has_x = 1;
   }
-  rc = cuda_rc(libcga::run_build_values(h->lv, in, scratch, static_cast<uint8_t*>(vm), s));
-  dfree(A, A != nullptr, scratch, s);
+  // rows sorted along with the keys where the scratch of both can be had at once,
+  // else the sums after the build, in scratch of their own
+  const size_t sums = libcga::value_scratch_bytes(cap, channels, policy);
+  vb.scratch = dalloc(A, std::max<size_t>(sums, 8 * n), s);
+  void* vm = vb.scratch != nullptr ? dalloc(A, cap * channels, s) : nullptr;
+  vb.values = static_cast<uint8_t*>(vm);
+  cga_t* h = nullptr;
+  int rc = vm != nullptr ? build_cloud(d_xyz, n, g, h_xform12, A, stream, &vb, &h) : CGA_ERR_OOM;
+  if (rc == CGA_ERR_OOM) {
+    if (vm != nullptr) dfree(A, A != nullptr, vm, s);
+    if (vb.scratch != nullptr) dfree(A, A != nullptr, vb.scratch, s);
+    vb.done = false;
+    rc = build_cloud(d_xyz, n, g, h_xform12, A, stream, nullptr, &h);
+    if (rc != CGA_OK) return rc;
+    vm = dalloc(A, cap * channels, s);
+    vb.scratch = vm != nullptr ? dalloc(A, sums, s) : nullptr;
+    vb.values = static_cast<uint8_t*>(vm);
+    if (vb.scratch == nullptr) {
+      if (vm != nullptr) dfree(A, A != nullptr, vm, s);
+      release(h);
+      return CGA_ERR_OOM;
+    }
+  }
+  if (rc == CGA_OK && !vb.done) {
+    rc = cuda_rc(libcga::run_build_values(h->lv, vb.in, vb.scratch, vb.values, nullptr, s));
+  }
+  dfree(A, A != nullptr, vb.scratch, s);
+  if (h == nullptr) {
+    dfree(A, A != nullptr, vm, s);
+    return rc;
+  }
   h->vmem = vm;
-  h->values = static_cast<uint8_t*>(vm);
+  h->values = vb.values;
   h->channels = channels;
   if (rc != CGA_OK) {
     release(h);

@@ -21,6 +21,7 @@
 //   k_bin_sort   a job per block: its keys ordered in shared memory, the distinct
 //                ones written back with the job's counts
 //   k_bin_write  the CGA arrays, a job per block
+//   k_bin_values the Value array, a job per block (builds with attributes only)
 //
 // A bin holds whole x slabs (bin bits <= grid bits) and a job of a split bin whole
 // columns, so a job's first key always opens a voxel and a column, and a slab
@@ -325,11 +326,54 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
   if (tid == 0) njobs[blockIdx.x] = all;
 }
 
-// Tiles of 1024 * IT points into their bins.
-template <typename T, int IT>
+// What the Value array needs of each of four consecutive points from i (a multiple
+// of four): its row, a channel a byte, or its index where the first point counts.
+__device__ __forceinline__ void load_rows(const ValueInput& in, uint32_t i, uint32_t n, uint32_t* r) {
+  const uint32_t C = in.channels;
+  if (in.policy == kValueFirst) {
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) r[k] = i + k;
+    return;
+  }
+  const uint8_t* p = in.attr + (size_t)i * C;
+  if (i + 4 <= n && (reinterpret_cast<uintptr_t>(in.attr) & 3u) == 0) {
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(p);
+    uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      if (k < C) w[k] = __ldg(q + k);
+    }
+    if (C == 1) {
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) r[k] = (w[0] >> (8 * k)) & 0xffu;
+    } else if (C == 2) {
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) r[k] = (w[k >> 1] >> (16 * (k & 1))) & 0xffffu;
+    } else if (C == 3) {
+      r[0] = w[0] & 0xffffffu;
+      r[1] = __funnelshift_r(w[0], w[1], 24) & 0xffffffu;
+      r[2] = __funnelshift_r(w[1], w[2], 16) & 0xffffffu;
+      r[3] = w[2] >> 8;
+    } else {
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) r[k] = w[k];
+    }
+    return;
+  }
+#pragma unroll
+  for (uint32_t k = 0; k < 4; ++k) {
+    r[k] = 0;
+    for (uint32_t c = 0; c < C && i + k < n; ++c) r[k] |= (uint32_t)__ldg(p + k * C + c) << (8 * c);
+  }
+}
+
+// Tiles of 1024 * IT points into their bins; with ROWS each point's load_rows word
+// goes to the same place of `rows`.
+template <typename T, int IT, bool ROWS>
 __global__ void __launch_bounds__(1024) k_bin_part(const SortSeg* __restrict__ segs, int S,
                                                    uint32_t* __restrict__ cur, T* __restrict__ keys,
-                                                   uint32_t stride) {
+                                                   uint32_t stride, ValueInput in,
+                                                   uint32_t* __restrict__ rows) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   T* s_key = reinterpret_cast<T*>(s_raw);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_raw + sizeof(T) * 1024 * IT);
@@ -398,6 +442,26 @@ __global__ void __launch_bounds__(1024) k_bin_part(const SortSeg* __restrict__ s
     const uint32_t at = s_off[s_bin[e]] + e;
     if (at < sg.n_host) out[at] = s_key[e];
   }
+  if constexpr (ROWS) {
+    __syncthreads();
+    uint32_t* s_row = reinterpret_cast<uint32_t*>(s_raw);
+#pragma unroll
+    for (int q = 0; q < IT / 4; ++q) {
+      const uint32_t i = i0 + 4 * (tid + 1024u * q);
+      uint32_t r[4] = {0, 0, 0, 0};
+      if (i < i1) load_rows(in, i, i1, r);
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        const uint32_t v = br[4 * q + k];
+        if (v != 0xffffffffu) s_row[s_cnt[v >> 16] + (v & 0xffffu)] = r[k];
+      }
+    }
+    __syncthreads();
+    for (uint32_t e = tid; e < i1 - i0; e += 1024) {
+      const uint32_t at = s_off[s_bin[e]] + e;
+      if (at < sg.n_host) rows[at] = s_row[e];
+    }
+  }
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -438,11 +502,12 @@ __device__ __forceinline__ void cluster_store(uint32_t a, uint32_t v) {
 // points, b = 10) took the build from 660 to 1190 us with a cluster each; a bin of 173k
 // keys (1.3M LiDAR points, b = 10), left to the general sort while a block split every
 // bin, cost 313 us there.
-template <typename T>
+template <typename T, bool ROWS>
 __global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(kBinThreads)
     k_bin_split(const SortSeg* __restrict__ segs, uint4* __restrict__ jobs,
                 const uint2* __restrict__ big, const T* __restrict__ keys, T* __restrict__ out,
-                uint32_t stride) {
+                uint32_t stride, const uint32_t* __restrict__ rows_in,
+                uint32_t* __restrict__ rows_out) {
   constexpr uint32_t R = 1u << kBinRowBits, PER = R / kBinThreads;
   __shared__ uint32_t s_cnt[R], s_tot[R / kBinCluster], s_pre[R + 1], s_scan[kBinWarps],
       s_next[kBinWarps];
@@ -584,7 +649,9 @@ __global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(kBinThread
 #pragma unroll
       for (uint32_t k = 0; k < 8; ++k) {
         if (e0 + k * kBinThreads < e_hi) {
-          dst[atomicAdd(&s_cnt[(uint32_t)((T)(v[k] - org) >> shift)], 1u)] = v[k];
+          const uint32_t at = atomicAdd(&s_cnt[(uint32_t)((T)(v[k] - org) >> shift)], 1u);
+          dst[at] = v[k];
+          if constexpr (ROWS) rows_out[job.z + at] = __ldg(rows_in + job.z + e0 + k * kBinThreads);
         }
       }
     }
@@ -1080,10 +1147,11 @@ __global__ void __launch_bounds__(kBinThreads, 2)
 
 // The CGA arrays of every job: heads of columns and slabs among its distinct keys,
 // at the places that the counts of the segment's earlier jobs give (a few thousand
-// at most: summed by the block, which is cheaper than another launch).
+// at most: summed by the block, which is cheaper than another launch).  A job's first
+// voxel stays in its second word.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_bin_write(const SortSeg* __restrict__ segs, int S,
-                                                        const uint4* __restrict__ jobs,
+                                                        uint4* __restrict__ jobs,
                                                         const uint32_t* __restrict__ njobs,
                                                         const T* __restrict__ keys0,
                                                         const T* __restrict__ keys1,
@@ -1126,6 +1194,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_write(const SortSeg* __restric
     __syncthreads();
     const uint3 f = make_uint3(s_f[0], s_f[1], s_f[2]);
     const uint32_t jx = jobs[slot].x;
+    if (tid == 0) jobs[slot].y = f.x;
     const uint32_t b = sg.bits, rem = 3 * b - sg.bin_bits, m = (1u << b) - 1u;
     const unsigned long long org = (unsigned long long)(jx & 0xffffu) << rem;
     const bool goes_on = (jx & kJobGoesOn) != 0u;
@@ -1209,6 +1278,166 @@ __global__ void __launch_bounds__(kThreads) k_bin_write(const SortSeg* __restric
       O.hdr->cnt[0] = U;
       O.hdr->cnt[1] = G;
       O.hdr->cnt[2] = H;
+    }
+  }
+}
+
+// The Value array of the one segment, a job per block: the job's distinct keys and
+// their sums in shared memory, every point of the job added to its voxel's.  A table
+// of the keys' top bits gives the few keys that a point has to be compared with (a
+// bisection of all of them took the kernel from 270 to 526 us, bound by shared-memory
+// loads).  The channels' sums have 16 bits each, two to a word, which the count bounds
+// (257 * 255 < 2^16); a job with a voxel of more points sums its channels again, two
+// at a time in 32 bits.  A point needs no search of the CGA and no atomic in global
+// memory: 15M rows of 3 channels that way took 1010 us for the sums alone.
+template <typename T>
+constexpr uint32_t bin_values_cap() { return sizeof(T) == 4 ? 6144 : 4096; }  // keys at a time
+constexpr uint32_t kBinDirBits = 12;
+template <typename T>
+constexpr size_t bin_values_smem() {
+  return (sizeof(T) + 12) * (size_t)bin_values_cap<T>() + (sizeof(uint32_t) << kBinDirBits);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBinThreads, 2)
+    k_bin_values(const SortSeg* __restrict__ segs, const uint4* __restrict__ jobs,
+                 const uint32_t* __restrict__ njobs, const T* __restrict__ keys0,
+                 const T* __restrict__ keys1, const uint32_t* __restrict__ rows0,
+                 const uint32_t* __restrict__ rows1, const uint4* __restrict__ info,
+                 uint32_t stride, ValueInput in, uint8_t* __restrict__ values) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  constexpr uint32_t CAP = bin_values_cap<T>();
+  T* s_key = reinterpret_cast<T*>(s_raw);
+  uint32_t* s_sum = reinterpret_cast<uint32_t*>(s_key + CAP);  // channels 0, 1
+  uint32_t* s_sum2 = s_sum + CAP;                              // channels 2, 3
+  uint32_t* s_num = s_sum2 + CAP;
+  uint16_t* s_dir = reinterpret_cast<uint16_t*>(s_num + CAP);  // {first, last} key
+  const uint32_t tid = threadIdx.x;
+  const SortSeg& sg = segs[0];
+  if (sg.narrow != (sizeof(T) == 4 ? 1u : 0u) || sg.fallback) return;
+  const uint32_t C = in.channels;
+  const bool first = in.policy == kValueFirst;
+  const uint32_t rem = 3 * sg.bits - sg.bin_bits;
+  for (uint32_t slot = blockIdx.x; slot < njobs[0]; slot += gridDim.x) {
+    const uint4 job = jobs[slot], q = info[slot];
+    const bool split = (job.x & kJobSplit) != 0u;
+    const T org = (T)((unsigned long long)(job.x & 0xffffu) << rem);
+    const T* src = seg_keys(split ? keys1 : keys0, sg, stride) + job.z;
+    const T* key = seg_keys(split ? keys0 : keys1, sg, stride) + q.x;
+    const uint32_t* row = (split ? rows1 : rows0) + job.z;
+    const uint32_t N = job.w;
+    // the count takes the place of a fourth channel where its 16 bits hold it
+    const bool packed = C <= 3 && N < 65536;
+    for (uint32_t u0 = 0; u0 < q.y; u0 += CAP) {
+      const uint32_t n = min(CAP, q.y - u0);
+      const T lo = __ldg(key + u0);
+      const T span = __ldg(key + u0 + n - 1) - lo;
+      uint32_t shift = 0;
+      while ((span >> shift) >> kBinDirBits) ++shift;
+      __syncthreads();
+      for (uint32_t e = tid; e < n; e += kBinThreads) {
+        const T k = __ldg(key + u0 + e) - lo;
+        const uint32_t d = (uint32_t)(k >> shift);
+        s_key[e] = k;
+        if (e == 0 || (uint32_t)((T)(__ldg(key + u0 + e - 1) - lo) >> shift) != d) s_dir[2 * d] = (uint16_t)e;
+        if (e + 1 == n || (uint32_t)((T)(__ldg(key + u0 + e + 1) - lo) >> shift) != d) {
+          s_dir[2 * d + 1] = (uint16_t)e;
+        }
+        s_sum[e] = first ? 0xffffffffu : 0u;
+        s_sum2[e] = s_num[e] = 0;
+      }
+      __syncthreads();
+      // add(voxel, row word) for every point with a voxel among the n
+      const T from = org + lo;
+      const bool all = n == q.y;
+      auto points = [&](auto add) {
+        for (uint32_t e0 = tid; e0 < N; e0 += 4 * kBinThreads) {
+          T v[4];
+          uint32_t r[4];
+#pragma unroll
+          for (uint32_t k = 0; k < 4; ++k) {
+            const uint32_t e = e0 + k * kBinThreads < N ? e0 + k * kBinThreads : e0;
+            v[k] = __ldg(src + e) - from;
+            r[k] = __ldg(row + e);
+          }
+#pragma unroll
+          for (uint32_t k = 0; k < 4; ++k) {
+            if (e0 + k * kBinThreads >= N || (!all && v[k] > span)) continue;
+            const uint32_t d = reinterpret_cast<const uint32_t*>(s_dir)[(uint32_t)(v[k] >> shift)];
+            uint32_t a = d & 0xffffu, b = d >> 16;
+            while (b > a + 3) {
+              const uint32_t mid = (a + b) >> 1;
+              if (s_key[mid] < v[k]) a = mid + 1; else b = mid;
+            }
+            while (a < b && s_key[a] != v[k]) ++a;
+            add(a, r[k]);
+          }
+        }
+      };
+      bool many = false;
+      if (first) {
+        points([&](uint32_t v, uint32_t r) { atomicMin(s_sum + v, r); });
+      } else if (packed) {
+        points([&](uint32_t v, uint32_t r) {
+          atomicAdd(s_sum + v, __byte_perm(r, 0, 0x4140));
+          atomicAdd(s_sum2 + v, ((r >> 16) & 0xffu) + 0x10000u);
+        });
+      } else {
+        points([&](uint32_t v, uint32_t r) {
+          atomicAdd(s_sum + v, __byte_perm(r, 0, 0x4140));
+          if (C > 2) atomicAdd(s_sum2 + v, __byte_perm(r, 0, 0x4342));
+          atomicAdd(s_num + v, 1u);
+        });
+      }
+      __syncthreads();
+      if (!first) {
+        // a sum that runs over carries into the count, which is then more than 257 too
+        for (uint32_t e = tid; e < n; e += kBinThreads) {
+          if (packed) s_num[e] = s_sum2[e] >> 16;
+          many |= s_num[e] > 257u;
+        }
+        many = __syncthreads_or(many);
+      }
+      uint8_t* out = values + ((size_t)job.y + u0) * C;
+      if (first) {
+        for (uint32_t e = tid; e < n; e += kBinThreads) {
+          const uint8_t* p = in.attr + (size_t)s_sum[e] * C;
+          for (uint32_t c = 0; c < C; ++c) out[(size_t)e * C + c] = __ldg(p + c);
+        }
+      } else if (!many) {
+        // round half up by the reciprocal: a quotient that is no whole number is at
+        // least 1/257 from the next one, the product within 1/16000 of the quotient
+        for (uint32_t e = tid; e < n; e += kBinThreads) {
+          const uint32_t k = s_num[e], x = s_sum[e], y = s_sum2[e];
+          const float inv = 1.0f / (float)k;
+          const uint32_t sum[4] = {x & 0xffffu, x >> 16, y & 0xffffu, y >> 16};
+#pragma unroll
+          for (uint32_t c = 0; c < 4; ++c) {
+            if (c < C) out[(size_t)e * C + c] = (uint8_t)((float)(sum[c] + k / 2) * inv + 0x1p-10f);
+          }
+        }
+      } else {
+        if (packed) {  // the counts may have carries in them
+          for (uint32_t e = tid; e < n; e += kBinThreads) s_num[e] = 0;
+          __syncthreads();
+          points([&](uint32_t v, uint32_t) { atomicAdd(s_num + v, 1u); });
+        }
+        for (uint32_t c = 0; c < C; c += 2) {
+          __syncthreads();
+          for (uint32_t e = tid; e < n; e += kBinThreads) s_sum[e] = s_sum2[e] = 0;
+          __syncthreads();
+          points([&](uint32_t v, uint32_t r) {
+            atomicAdd(s_sum + v, (r >> (8 * c)) & 0xffu);
+            if (c + 1 < C) atomicAdd(s_sum2 + v, (r >> (8 * c + 8)) & 0xffu);
+          });
+          __syncthreads();
+          for (uint32_t e = tid; e < n; e += kBinThreads) {
+            const uint32_t k = s_num[e];
+            out[(size_t)e * C + c] = (uint8_t)((s_sum[e] + k / 2) / k);
+            if (c + 1 < C) out[(size_t)e * C + c + 1] = (uint8_t)((s_sum2[e] + k / 2) / k);
+          }
+        }
+      }
     }
   }
 }

@@ -487,7 +487,7 @@ static void launch_passes(int S, uint32_t total_tiles, uint32_t max_passes, cons
 
 // Resident blocks of the bin kernels (set by init_bin_kernels): the job sorts of
 // 32- and 64-bit keys, and the general sort behind them.
-static uint32_t g_bin_sort_blocks[2], g_lsd_blocks[2];
+static uint32_t g_bin_sort_blocks[2], g_lsd_blocks[2], g_bin_values_blocks[2];
 
 template <typename F>
 static cudaError_t resident(F* kernel, int threads, size_t smem, uint32_t* blocks) {
@@ -504,12 +504,22 @@ static cudaError_t init_bin_kernels() {
       resident(k_bin_sort<uint32_t>, kBinThreads, bin_sort_smem<uint32_t>(), &g_bin_sort_blocks[0]),
       resident(k_bin_sort<unsigned long long>, kBinThreads, bin_sort_smem<unsigned long long>(),
                &g_bin_sort_blocks[1]),
-      resident(k_bin_part<uint32_t, 4>, 1024, bin_part_smem<uint32_t, 4>(), nullptr),
-      resident(k_bin_part<uint32_t, 8>, 1024, bin_part_smem<uint32_t, 8>(), nullptr),
-      resident(k_bin_part<uint32_t, 16>, 1024, bin_part_smem<uint32_t, 16>(), nullptr),
-      resident(k_bin_part<unsigned long long, 4>, 1024, bin_part_smem<unsigned long long, 4>(), nullptr),
-      resident(k_bin_part<unsigned long long, 8>, 1024, bin_part_smem<unsigned long long, 8>(), nullptr),
-      resident(k_bin_part<unsigned long long, 16>, 1024, bin_part_smem<unsigned long long, 16>(), nullptr),
+      resident(k_bin_part<uint32_t, 4, false>, 1024, bin_part_smem<uint32_t, 4>(), nullptr),
+      resident(k_bin_part<uint32_t, 4, true>, 1024, bin_part_smem<uint32_t, 4>(), nullptr),
+      resident(k_bin_part<uint32_t, 8, false>, 1024, bin_part_smem<uint32_t, 8>(), nullptr),
+      resident(k_bin_part<uint32_t, 8, true>, 1024, bin_part_smem<uint32_t, 8>(), nullptr),
+      resident(k_bin_part<uint32_t, 16, false>, 1024, bin_part_smem<uint32_t, 16>(), nullptr),
+      resident(k_bin_part<uint32_t, 16, true>, 1024, bin_part_smem<uint32_t, 16>(), nullptr),
+      resident(k_bin_part<unsigned long long, 4, false>, 1024, bin_part_smem<unsigned long long, 4>(), nullptr),
+      resident(k_bin_part<unsigned long long, 4, true>, 1024, bin_part_smem<unsigned long long, 4>(), nullptr),
+      resident(k_bin_part<unsigned long long, 8, false>, 1024, bin_part_smem<unsigned long long, 8>(), nullptr),
+      resident(k_bin_part<unsigned long long, 8, true>, 1024, bin_part_smem<unsigned long long, 8>(), nullptr),
+      resident(k_bin_part<unsigned long long, 16, false>, 1024, bin_part_smem<unsigned long long, 16>(), nullptr),
+      resident(k_bin_part<unsigned long long, 16, true>, 1024, bin_part_smem<unsigned long long, 16>(), nullptr),
+      resident(k_bin_values<uint32_t>, kBinThreads, bin_values_smem<uint32_t>(),
+               &g_bin_values_blocks[0]),
+      resident(k_bin_values<unsigned long long>, kBinThreads,
+               bin_values_smem<unsigned long long>(), &g_bin_values_blocks[1]),
       resident(k_lsd_all<uint32_t>, kThreads, onesweep_smem<uint32_t, kThreads, 8>(), &g_lsd_blocks[0]),
       resident(k_lsd_all<unsigned long long>, kThreads,
                onesweep_smem<unsigned long long, kThreads, 8>(), &g_lsd_blocks[1])};
@@ -590,17 +600,29 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
   B.on = true;
 }
 
-template <typename T>
+template <typename T, bool ROWS>
 static void launch_part(int S, const SortScratch& sc, uint32_t stride, cudaStream_t stream) {
   const BinPlan& B = sc.bins;
   T* keys = static_cast<T*>(sc.keys0);
   if (B.items == 16) {
-    k_bin_part<T, 16><<<B.ptiles, 1024, bin_part_smem<T, 16>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+    k_bin_part<T, 16, ROWS><<<B.ptiles, 1024, bin_part_smem<T, 16>(), stream>>>(
+        sc.segs, S, B.cur, keys, stride, B.value_in, B.value_rows);
   } else if (B.items == 8) {
-    k_bin_part<T, 8><<<B.ptiles, 1024, bin_part_smem<T, 8>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+    k_bin_part<T, 8, ROWS><<<B.ptiles, 1024, bin_part_smem<T, 8>(), stream>>>(
+        sc.segs, S, B.cur, keys, stride, B.value_in, B.value_rows);
   } else {
-    k_bin_part<T, 4><<<B.ptiles, 1024, bin_part_smem<T, 4>(), stream>>>(sc.segs, S, B.cur, keys, stride);
+    k_bin_part<T, 4, ROWS><<<B.ptiles, 1024, bin_part_smem<T, 4>(), stream>>>(
+        sc.segs, S, B.cur, keys, stride, B.value_in, B.value_rows);
   }
+}
+
+template <typename T, bool ROWS>
+static void launch_split(const SortScratch& sc, uint32_t stride, cudaStream_t stream) {
+  const BinPlan& B = sc.bins;
+  T *k0 = static_cast<T*>(sc.keys0), *k1 = static_cast<T*>(sc.keys1);
+  const unsigned clusters = std::max(1u, 3 * (unsigned)device_sm_count() / kBinCluster);
+  k_bin_split<T, ROWS><<<clusters * kBinCluster, kBinThreads, 0, stream>>>(
+      sc.segs, B.jobs, B.big, k0, k1, stride, B.value_rows, B.value_rows + B.value_in.n);
 }
 
 template <typename T>
@@ -609,11 +631,12 @@ static void launch_bin_jobs(int S, const SortScratch& sc, uint32_t stride, uint3
   const BinPlan& B = sc.bins;
   T *k0 = static_cast<T*>(sc.keys0), *k1 = static_cast<T*>(sc.keys1);
   k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.start, B.cur, B.jobs, B.njobs, B.big);
-  launch_part<T>(S, sc, stride, stream);
-  if (B.may_split) {
-    const unsigned clusters = std::max(1u, 3 * (unsigned)device_sm_count() / kBinCluster);
-    k_bin_split<T><<<clusters * kBinCluster, kBinThreads, 0, stream>>>(
-        sc.segs, B.jobs, B.big, k0, k1, stride);
+  if (B.value_rows != nullptr) {
+    launch_part<T, true>(S, sc, stride, stream);
+    if (B.may_split) launch_split<T, true>(sc, stride, stream);
+  } else {
+    launch_part<T, false>(S, sc, stride, stream);
+    if (B.may_split) launch_split<T, false>(sc, stride, stream);
   }
   const uint32_t blocks = std::min<uint32_t>(B.slots, g_bin_sort_blocks[sizeof(T) / 8]);
   k_bin_sort<T><<<blocks, kBinThreads, bin_sort_smem<T>(), stream>>>(
@@ -626,6 +649,13 @@ static void launch_bin_write(int S, const SortScratch& sc, uint32_t stride, cuda
   const T *k0 = static_cast<const T*>(sc.keys0), *k1 = static_cast<const T*>(sc.keys1);
   k_bin_write<T><<<std::min<uint32_t>(B.slots, (uint32_t)device_sm_count() * 8), kThreads, 0,
                    stream>>>(sc.segs, S, B.jobs, B.njobs, k0, k1, B.info, B.slots, stride);
+  if (B.value_rows != nullptr) {
+    k_bin_values<T><<<std::min<uint32_t>(B.slots, g_bin_values_blocks[sizeof(T) / 8]), kBinThreads,
+                      bin_values_smem<T>(), stream>>>(
+        sc.segs, B.jobs, B.njobs, k0, k1, B.value_rows, B.value_rows + B.value_in.n, B.info, stride,
+        B.value_in, B.values);
+    count_launch(1);
+  }
 }
 
 template <typename K>
@@ -667,6 +697,11 @@ static cudaError_t run_bins(int S, uint32_t total_tiles, bool key64, const SortS
               : launch_lsd_all<uint32_t>(S, total_tiles, sc, stream);
   }
   count_launch(3 + (B.may_split ? 5 : 4) * ((B.narrow ? 1 : 0) + (B.wide ? 1 : 0)));
+  // the Value array of a cloud that the general sort had to take
+  if (e == cudaSuccess && B.value_rows != nullptr) {
+    e = run_build_values(B.value_out, B.value_in, B.value_rows, B.values, &sc.segs[0].fallback,
+                         stream);
+  }
   return e;
 }
 

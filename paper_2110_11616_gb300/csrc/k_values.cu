@@ -1,5 +1,8 @@
 // The Value (attribute) array of a CGA (Sec. V): one row of uint8 channels
 // per stored voxel, in CGA point order.
+// Builds by bins sum the rows along with the sort (k_bins.cuh); what follows is the
+// way of the other builds (dense grids of many points, and clouds that the general
+// sort takes over).
 //   k_value_accumulate  each input point finds its voxel by the Sec. V-A
 //                       lookup and adds its attributes (or offers its index)
 //   k_value_finalize    per voxel: round-half-up mean (sum + k/2) / k of its
@@ -19,8 +22,19 @@ namespace libcga {
 
 namespace {
 
+__global__ void k_value_init(uint32_t* scratch, size_t words, uint32_t value,
+                             const uint32_t* only_if) {
+  if (only_if != nullptr && *only_if == 0) return;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < words; i += stride) {
+    scratch[i] = value;
+  }
+}
+
 template <typename S>
-__global__ void k_value_accumulate(Levels a, ValueInput in, void* scratch) {
+__global__ void k_value_accumulate(Levels a, ValueInput in, void* scratch,
+                                   const uint32_t* only_if) {
+  if (only_if != nullptr && *only_if == 0) return;
   const uint32_t h = (uint32_t)a.hdr->cnt[2];
   const uint32_t C = in.channels;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -48,7 +62,9 @@ __global__ void k_value_accumulate(Levels a, ValueInput in, void* scratch) {
 }
 
 template <typename S>
-__global__ void k_value_finalize(Levels a, ValueInput in, const void* scratch, uint8_t* values) {
+__global__ void k_value_finalize(Levels a, ValueInput in, const void* scratch, uint8_t* values,
+                                 const uint32_t* only_if) {
+  if (only_if != nullptr && *only_if == 0) return;
   const uint32_t u = (uint32_t)a.hdr->cnt[0];
   const uint32_t C = in.channels;
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -134,19 +150,28 @@ size_t value_scratch_bytes(uint64_t cap, uint32_t channels, int policy) {
 }
 
 cudaError_t run_build_values(const Levels& a, const ValueInput& in, void* scratch,
-                             uint8_t* values, cudaStream_t stream) {
+                             uint8_t* values, const uint32_t* only_if, cudaStream_t stream) {
   const bool narrow = in.policy != kValueFirst && narrow_sums(in.n);
   const size_t bytes = narrow ? (size_t)std::max<uint64_t>(a.cap, 1) * 4 * (in.channels + 1)
                               : value_scratch_bytes(a.cap, in.channels, in.policy);
-  cudaError_t e = cudaMemsetAsync(scratch, in.policy == kValueFirst ? 0xff : 0, bytes, stream);
-  if (e != cudaSuccess) return e;
-  if (narrow) {
-    k_value_accumulate<uint32_t><<<blocks_for(in.n), 256, 0, stream>>>(a, in, scratch);
-    k_value_finalize<uint32_t><<<blocks_for(a.cap), 256, 0, stream>>>(a, in, scratch, values);
+  const uint32_t init = in.policy == kValueFirst ? 0xffffffffu : 0u;
+  if (only_if == nullptr) {
+    const cudaError_t e = cudaMemsetAsync(scratch, (int)(init & 0xffu), bytes, stream);
+    if (e != cudaSuccess) return e;
   } else {
-    k_value_accumulate<unsigned long long><<<blocks_for(in.n), 256, 0, stream>>>(a, in, scratch);
+    k_value_init<<<blocks_for(bytes / 16), 256, 0, stream>>>(static_cast<uint32_t*>(scratch),
+                                                             bytes / 4, init, only_if);
+    count_launch(1);
+  }
+  if (narrow) {
+    k_value_accumulate<uint32_t><<<blocks_for(in.n), 256, 0, stream>>>(a, in, scratch, only_if);
+    k_value_finalize<uint32_t><<<blocks_for(a.cap), 256, 0, stream>>>(a, in, scratch, values,
+                                                                      only_if);
+  } else {
+    k_value_accumulate<unsigned long long><<<blocks_for(in.n), 256, 0, stream>>>(a, in, scratch,
+                                                                                only_if);
     k_value_finalize<unsigned long long><<<blocks_for(a.cap), 256, 0, stream>>>(a, in, scratch,
-                                                                             values);
+                                                                             values, only_if);
   }
   count_launch(2);
   return cudaGetLastError();

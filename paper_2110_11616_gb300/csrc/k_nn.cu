@@ -1267,10 +1267,13 @@ __global__ void __launch_bounds__(kTreeThreads, CGA_NN_TREE_BLOCKS)
   const bool sorted = order != nullptr && (order_err == nullptr || *order_err == 0u);
   const uint32_t lane = threadIdx.x & 31, g = lane % G;
   const uint32_t gm = G == 32 ? 0xffffffffu : (uint32_t)((1ull << G) - 1ull) << (lane - g);
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  constexpr uint32_t W = kTreeThreads / 32;
+  __shared__ uint32_t s_next;
+  open_slots<W>(&s_next);
   const uint32_t n_pass = pass_count(total_slots, stride, parent);
-  for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * QW; base < n_pass;
-       base += nwarps * QW) {
+  for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
+    const uint32_t base = slot_of_turn<W>(turn) * QW;
+    if (base >= n_pass) break;
     const uint32_t i = base + lane / G;
     bool active = i < n_pass;
     const uint32_t slot = pass_slot(active ? i : base, stride, parent);
@@ -1331,10 +1334,13 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
               const unsigned long long* __restrict__ order,
               const unsigned int* __restrict__ order_err) {
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  constexpr uint32_t W = 256 / 32;
+  __shared__ uint32_t s_next;
+  open_slots<W>(&s_next);
   const bool sorted = order != nullptr && (order_err == nullptr || *order_err == 0u);
-  for (uint32_t slot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; slot < total_slots;
-       slot += nwarps) {
+  for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
+    const uint32_t slot = slot_of_turn<W>(turn);
+    if (slot >= total_slots) break;
     const uint32_t tile = slot / (uint32_t)kTile;
     const NnSeg& sg = segs != nullptr ? segs[find_nn_seg(segs, S, tile)] : inline_seg;
     if (sg.tree.levels > 0) continue;  // searched by k_nn_tree

@@ -205,9 +205,12 @@ __global__ void __launch_bounds__(256, CGA_RADIUS_BLOCKS)
     k_radius_count(SearchSeg sg, D r2, D r, const unsigned long long* __restrict__ order,
                    unsigned long long* counts) {
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
   const uint32_t h = (uint32_t)sg.a.hdr->cnt[2];
-  for (uint32_t sl = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; sl < sg.m; sl += nw) {
+  __shared__ uint32_t s_next;
+  open_slots<256 / 32>(&s_next);
+  for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
+    const uint32_t sl = slot_of_turn<256 / 32>(turn);
+    if (sl >= sg.m) break;
     const uint32_t j = slot_query(order, sl);
     const RQuery q = radius_query(sg, j);
     uint32_t s0, s1;
@@ -235,9 +238,12 @@ __global__ void __launch_bounds__(256, CGA_RADIUS_BLOCKS)
   __shared__ uint32_t s_op[8][32 * kRadiusKeep];
   __shared__ D s_od[8][32 * kRadiusKeep];
   const uint32_t tid = threadIdx.x, lane = tid & 31;
-  const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
   const uint32_t h = (uint32_t)sg.a.hdr->cnt[2];
-  for (uint32_t sl = (blockIdx.x * blockDim.x + tid) >> 5; sl < sg.m; sl += nw) {
+  __shared__ uint32_t s_next;
+  open_slots<256 / 32>(&s_next);
+  for (uint32_t turn = tid >> 5;; turn = next_turn(&s_next)) {
+    const uint32_t sl = slot_of_turn<256 / 32>(turn);
+    if (sl >= sg.m) break;
     const uint32_t j = slot_query(order, sl);
     const RQuery q = radius_query(sg, j);
     uint32_t s0, s1;
@@ -706,7 +712,6 @@ __global__ void __launch_bounds__(LARGE ? kKnnLargeThreads : 256, LARGE ? 1 : CG
           uint32_t* out_idx, unsigned long long* out_d2) {
   extern __shared__ __align__(16) unsigned char s_knn[];
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
   const uint32_t u = (uint32_t)sg.a.hdr->cnt[0], h = (uint32_t)sg.a.hdr->cnt[2];
   typename std::conditional<LARGE, SmemList<NARROW>, RegList<NARROW>>::type list;
   auto answer = [&](uint32_t j) {
@@ -719,10 +724,18 @@ __global__ void __launch_bounds__(LARGE ? kKnnLargeThreads : 256, LARGE ? 1 : CG
     if (q.valid && u > 0) knn_walk<NARROW>(sg, q, h, lane, list);
     list.finish(lane, (size_t)j * k, out_idx, out_d2);
   };
-  const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if constexpr (NARROW) {
-    for (uint32_t sl = w; sl < sg.m; sl += nw) answer(slot_query(order, sl));
+    constexpr uint32_t W = (LARGE ? kKnnLargeThreads : 256) / 32;
+    __shared__ uint32_t s_next;
+    open_slots<W>(&s_next);
+    for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
+      const uint32_t sl = slot_of_turn<W>(turn);
+      if (sl >= sg.m) break;
+      answer(slot_query(order, sl));
+    }
   } else {
+    const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
     const uint32_t need = min(k, u);
     if (need == 0) return;
     for (uint32_t s0 = w * 32; s0 < sg.m; s0 += nw * 32) {

@@ -1071,21 +1071,80 @@ __global__ void k_project_xy(Levels a, Levels o) {
 // by row, in order, are the distinct 2D voxels in key order: U_index the
 // non-empty rows, V_index the set columns of each.
 
-// Set the bits of a's voxels, decoded by the walk of Sec. V-A (k_walk.cuh).
+// Set the bits of a's voxels, decoded by the walk of Sec. V-A (k_walk.cuh).  An atomic
+// a voxel bounds that (110 us a plane of 20M voxels), and most of them set what is set:
+// - yz (plane 2): neighbouring lanes' voxels of one column and word are joined.
+// - xz (plane 1): a warp's run of positions lies in few slabs, so it gathers a slab's
+//   row in shared memory and writes the row's words when the slab ends; what a step
+//   holds of other slabs goes straight to memory.
+// Whole projections of 20M surface voxels at b = 12: xz 197 -> 137 us, yz 204 -> 169
+// (reading a yz word before setting it: 192); 10M uniform voxels, b = 10: 71 -> 49 and
+// 75 -> 67; a 118k LiDAR sweep unchanged at 35.
 constexpr int kProjPerSm = 6;
+constexpr uint32_t kProjMaxBits = 13;
 __global__ void __launch_bounds__(kThreads, kProjPerSm) k_proj_set(Levels a, int plane,
                                                        uint32_t* __restrict__ bits) {
+  __shared__ uint32_t s_row[kWarps][1u << (kProjMaxBits - 5)];
   uint32_t begin, end;
   walk_range((uint32_t)a.hdr->cnt[0], begin, end);
-  const uint32_t b = a.bits;
-  walk_voxels(a, begin, end, [&](uint32_t, uint32_t valid, const uint32_t* x, const uint32_t* y,
+  const uint32_t b = a.bits, lane = threadIdx.x & 31u;
+  if (plane == 2) {
+    walk_voxels(a, begin, end, [&](uint32_t, uint32_t valid, const uint32_t*, const uint32_t* y,
+                                   const uint32_t* z) {
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        const uint32_t w = (valid >> k) & 1u ? ((y[k] << b) | z[k]) >> 5 : 0xffffffffu;
+        uint32_t bit = 1u << (z[k] & 31u);
+#pragma unroll
+        for (uint32_t d = 1; d < 32; d <<= 1) {
+          const uint32_t ow = __shfl_down_sync(0xffffffffu, w, d);
+          const uint32_t ob = __shfl_down_sync(0xffffffffu, bit, d);
+          if (ow == w) bit |= ob;
+        }
+        const uint32_t before = __shfl_up_sync(0xffffffffu, w, 1);
+        if (w != 0xffffffffu && (lane == 0 || before != w)) atomicOr(bits + w, bit);
+      }
+    });
+    return;
+  }
+  uint32_t* row = s_row[threadIdx.x >> 5];
+  const uint32_t words = 1u << (b - 5);
+  for (uint32_t i = lane; i < words; i += 32) row[i] = 0;
+  uint32_t cur = 0xffffffffu;  // the slab whose row is gathered
+  __syncwarp();
+  auto flush = [&]() {
+    __syncwarp();
+    for (uint32_t i = lane; i < words; i += 32) {
+      const uint32_t v = row[i];
+      if (v) atomicOr(bits + ((size_t)cur << (b - 5)) + i, v);
+      row[i] = 0;
+    }
+    __syncwarp();
+  };
+  walk_voxels(a, begin, end, [&](uint32_t, uint32_t valid, const uint32_t* x, const uint32_t*,
                                  const uint32_t* z) {
+    uint32_t last = 0;  // the step's last slab
 #pragma unroll
     for (uint32_t k = 0; k < 4; ++k) {
-      const uint32_t key = ((plane == 1 ? x[k] : y[k]) << b) | z[k];
-      if ((valid >> k) & 1u) atomicOr(bits + (key >> 5), 1u << (key & 31u));
+      if ((valid >> k) & 1u) last = x[k];
+    }
+    last = __reduce_max_sync(0xffffffffu, last);
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      if (!((valid >> k) & 1u)) continue;
+      const uint32_t bit = 1u << (z[k] & 31u);
+      if (x[k] == cur) {
+        atomicOr(row + (z[k] >> 5), bit);
+      } else {
+        atomicOr(bits + (((x[k] << b) | z[k]) >> 5), bit);
+      }
+    }
+    if (last != cur) {
+      if (cur != 0xffffffffu) flush();
+      cur = last;
     }
   });
+  if (cur != 0xffffffffu) flush();
 }
 
 // Set bits of each row: one warp per row, each lane a run of the row's words.

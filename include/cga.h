@@ -441,8 +441,8 @@ int cga_nn_query_batch(const cga_t* const* a, const cga_queries* q, uint32_t cou
 typedef struct {
   uint32_t radix_bits;    /* digit width of an LSD pass: 8 or 9 (9 needs sort_threads 512) */
   uint32_t sort_threads;  /* threads per 4096-key tile: 256 (16 keys each) or 512 (8 keys each) */
-  uint32_t merge_half;    /* merge-path partition: a splitter every 512, 1024 or 2048 points
-                             of each input (tiles of at most 2 * merge_half keys) */
+  uint32_t merge_half;    /* merge partition, 512, 1024 or 2048: tiles of at most
+                             2 * merge_half columns (points, on fine grids) */
 } cga_tuning;
 
 #define CGA_TUNE_SORT_CANDIDATES 3  /* (8, 256), (8, 512), (9, 512) */

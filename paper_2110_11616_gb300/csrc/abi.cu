@@ -356,10 +356,11 @@ int cga_merge(const cga_t* a, const cga_t* b, const cga_allocator* A, void* stre
   P.out = h->lv;
   P.spl_base = 0;
   const uint64_t points = a->lv.cap + b->lv.cap;
-  const uint32_t half =
-      libcga::merge_half_for(bits, points, bits, points, libcga::merge_key_level(bits));
-  P.spl_a = libcga::merge_splitters(a->lv.cap, half);
-  P.spl_b = libcga::merge_splitters(b->lv.cap, half);
+  const bool key_level = libcga::merge_key_level(bits);
+  const uint32_t half = libcga::merge_half_for(bits, points, bits, points, key_level);
+  const uint32_t spacing = libcga::merge_spacing(half, key_level);
+  P.spl_a = libcga::merge_splitters(a->lv.cap, spacing);
+  P.spl_b = libcga::merge_splitters(b->lv.cap, spacing);
   P.tile_base = 0;
   P.num_tiles = P.spl_a + P.spl_b + 1;
   const uint32_t total_spl = P.spl_a + P.spl_b;
@@ -1323,6 +1324,7 @@ int plan_merges(const cga_t* const* a, const cga_t* const* b, uint32_t count,
     max_in = std::max<uint64_t>(max_in, a[i]->lv.cap + b[i]->lv.cap);
   }
   half = libcga::merge_half_for(max_bits, max_in, rule_bits, max_in, key_level);
+  const uint32_t spacing = libcga::merge_spacing(half, key_level);
   for (uint32_t i = 0; i < count; ++i) {
     const uint64_t cap = std::min<uint64_t>(a[i]->lv.cap + b[i]->lv.cap, pow2(3 * a[i]->grid.bits));
     hs[i] = new_cga(a[i]->grid, A, s, cap);
@@ -1331,8 +1333,8 @@ int plan_merges(const cga_t* const* a, const cga_t* const* b, uint32_t count,
     P.a = a[i]->lv;
     P.b = b[i]->lv;
     P.out = hs[i]->lv;
-    P.spl_a = libcga::merge_splitters(a[i]->lv.cap, half);
-    P.spl_b = libcga::merge_splitters(b[i]->lv.cap, half);
+    P.spl_a = libcga::merge_splitters(a[i]->lv.cap, spacing);
+    P.spl_b = libcga::merge_splitters(b[i]->lv.cap, spacing);
     P.spl_base = (uint32_t)spl;
     P.tile_base = (uint32_t)tiles;
     P.num_tiles = P.spl_a + P.spl_b + 1;
@@ -1621,6 +1623,7 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
   }
   const libcga::Tuning tu = libcga::tuning_for(max_bits, max_n);
   const uint32_t half = libcga::merge_half_for(max_bits, max_n, rule_bits, 2 * max_n, key_level);
+  const uint32_t spacing = libcga::merge_spacing(half, key_level);
   // --- layout
   Bump bump;
   std::vector<size_t> lv_off(4 * (size_t)S);
@@ -1643,7 +1646,7 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
     lv_off[4 * i + 3] = bump.take(levels_bytes(pc, pc1, 0, 2));
     const uint64_t t = (n + libcga::kTile - 1) / libcga::kTile;
     build_tiles += 2 * t;
-    const uint64_t sa = libcga::merge_splitters(n, half);
+    const uint64_t sa = libcga::merge_splitters(n, spacing);
     spl += 2 * sa;
     mtiles += 2 * sa + 1;
     if (items[i].m > 0) {
@@ -1736,7 +1739,7 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
     P.a = p->views[3 * i].lv;
     P.b = p->views[3 * i + 1].lv;
     P.out = p->views[3 * i + 2].lv;
-    P.spl_a = P.spl_b = libcga::merge_splitters(items[i].n, half);
+    P.spl_a = P.spl_b = libcga::merge_splitters(items[i].n, spacing);
     P.spl_base = (uint32_t)sb;
     P.tile_base = (uint32_t)mb;
     P.num_tiles = P.spl_a + P.spl_b + 1;

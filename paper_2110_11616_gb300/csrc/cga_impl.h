@@ -202,14 +202,13 @@ cudaError_t run_sort_pipeline(const SortSeg* h_segs, int S, uint32_t total_tiles
 cudaError_t run_decode(const Levels& a, uint32_t* xyz, cudaStream_t stream);
 
 // Merge: sorted union of pairs of 3-level CGAs, column by column (or, on fine
-// grids, key by key).  Splitters are taken at every half-th (x, y) column
-// (or point) of each input (half = Tuning::merge_half <= kTile / 2; `cap`
-// below is a point capacity, which bounds the columns too); between
-// consecutive splitters each input contributes at most half columns (points),
-// so one tile of at most 2 * half of them always holds the merged run.
+// grids, key by key).  Splitters are taken at every spacing-th (x, y) column
+// (or point) of each input (merge_spacing of half = Tuning::merge_half <= kTile / 2;
+// `cap` below is a point capacity, which bounds the columns too); a tile holds the
+// columns (points) between a few consecutive splitters, at most 2 * half of them.
 constexpr int kMergeHalf = kTile / 2;  // largest partition
-inline uint32_t merge_splitters(uint64_t cap, uint32_t half) {
-  return cap > 0 ? (uint32_t)((cap - 1) / half) : 0u;
+inline uint32_t merge_splitters(uint64_t cap, uint32_t spacing) {
+  return cap > 0 ? (uint32_t)((cap - 1) / spacing) : 0u;
 }
 
 struct MergePair {
@@ -222,7 +221,7 @@ struct MergePair {
 
 struct MergeScratch {
   uint32_t* bounds;         // [(total_tiles + S) * 4]; pair p at 4 * (tile_base + p)
-  uint32_t* ntiles;         // [S]
+  uint32_t* ntiles;         // [3][S]: tiles, cuts a tile, cuts
   uint32_t* clook;          // [total_tiles][3]
   uint32_t* counter;        // [1]
   MergePair* pairs;         // [S]
@@ -230,6 +229,9 @@ struct MergeScratch {
   uint32_t half;            // merge-path partition the splitters were counted with
   bool key_level;           // merge the key sequences instead of the columns
 };
+// Columns (or points) of an input from splitter to splitter; a column-level tile takes
+// several intervals (k_merge_init).
+inline uint32_t merge_spacing(uint32_t half, bool key_level) { return key_level ? half : half / 4; }
 // The merge form for pairs on grids of `bits` per axis: key-level from 14 bits
 // on (a column then holds about one voxel), column-level below.
 inline bool merge_key_level(uint32_t bits) { return bits >= 14; }

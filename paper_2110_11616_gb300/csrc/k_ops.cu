@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kThreads, kDecodePerSm) k_decode(Levels a, uin
 // column boundaries.  The (x, y) columns of both inputs are in key order (key
 // x << b | y); a column present in both gets the union of its two sorted z
 // lists, a column of one input keeps its z list.  Splitters sit at every
-// `half`-th column of each input; a cut at column key s takes, from both
+// merge_spacing-th column of each input; a cut at column key s takes, from both
 // inputs, the columns with key < s, so a column present in both never
 // straddles two tiles and every tile can settle its columns alone.  A tile
 // merges its voxels by (column key, z) keys (merge_tile_v), or, when its
@@ -89,9 +89,22 @@ __device__ __forceinline__ uint32_t n_splitters(uint32_t g, uint32_t reserved, u
 // slab holding each of them (h for the end of the input).
 constexpr int kBoundWords = 4;
 
-// Output header, empty-CGA sentinels, first and last tile bounds.
+// Output header, empty-CGA sentinels, first and last tile bounds; ntiles[p] the
+// pair's tiles, ntiles[S + p] the cuts of each and ntiles[2 S + p] all of them.
+//
+// Cuts lie at every quarter of the partition's columns (merge_spacing), and a tile takes
+// the columns of several: seven cut intervals hold at most 8 quarters (2 * half, what a
+// tile has room for), and their sum varies little, where one interval between the cuts
+// at every half-th column had anything from none to twice its mean.  As many as fill
+// four fifths of the voxel-level tile's room, but no fewer than four while that leaves
+// less than a wave of tiles.  Where not even five fit (dense columns), seven, which go
+// column by column: 15M surface points a side, b = 11, 260 us that way and 309 in
+// voxel-level tiles of four.  Per merge on GB300, us, before and after: 20M surface
+// voxels, b = 12: 419 and 368; 1.8M: 79 and 69; 20M uniform points, b = 12: 482 and 375,
+// b = 11: 441 and 330; 5M surface voxels, b = 10: 123 and 121; 200k points: 39 and 38.
+constexpr uint32_t kMergeCuts = 7;
 __global__ void k_merge_init(const MergePair* __restrict__ pairs, int S, uint32_t half,
-                             uint32_t* bounds, uint32_t* ntiles) {
+                             uint32_t voxels, uint32_t wave, uint32_t* bounds, uint32_t* ntiles) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= S) return;
   const MergePair& P = pairs[p];
@@ -99,7 +112,12 @@ __global__ void k_merge_init(const MergePair* __restrict__ pairs, int S, uint32_
   const uint32_t hA = (uint32_t)P.a.hdr->cnt[2], hB = (uint32_t)P.b.hdr->cnt[2];
   const uint32_t NA = n_splitters(gA, P.spl_a, half), NB = n_splitters(gB, P.spl_b, half);
   const uint32_t nt = NA + NB + 1;
-  ntiles[p] = nt;
+  const unsigned long long u = max(P.a.hdr->cnt[0] + P.b.hdr->cnt[0], 1ull);
+  const uint32_t fit = (uint32_t)min((unsigned long long)kMergeCuts, (unsigned long long)voxels * nt / u);
+  const uint32_t k = min(fit < 5 ? kMergeCuts : fit, max(4u, nt / wave));
+  ntiles[p] = (nt + k - 1) / k;
+  ntiles[S + p] = k;
+  ntiles[2 * S + p] = nt;
   uint32_t* bnd = bounds + (size_t)kBoundWords * ((size_t)P.tile_base + p);
   bnd[0] = 0;
   bnd[1] = 0;
@@ -170,6 +188,14 @@ __global__ void k_merge_cuts(const MergePair* __restrict__ pairs, int S, uint32_
   }
 }
 
+// The first bound of tile lt of pair p (of the pair's end past its tiles).
+__device__ __forceinline__ uint4 tile_bound(const MergePair& P, int p, int S,
+                                            const uint32_t* __restrict__ bounds,
+                                            const uint32_t* __restrict__ ntiles, uint32_t lt) {
+  const uint32_t cut = min(lt * ntiles[S + p], ntiles[2 * S + p]);
+  return __ldg(reinterpret_cast<const uint4*>(bounds) + (size_t)P.tile_base + p + cut);
+}
+
 // Size of the union of two ascending z lists (in shared or global memory).
 __device__ __forceinline__ uint32_t union_count(const uint16_t* za, uint32_t na,
                                                 const uint16_t* zb, uint32_t nb) {
@@ -202,8 +228,8 @@ __device__ __forceinline__ void union_write(const uint16_t* za, uint32_t na, con
 template <int MH>
 constexpr int merge_stage() { return MH == 2048 ? 1536 : 6144; }
 
-// Voxels of each input the voxel-level tile path holds in shared memory (a
-// tile with more on either side takes the column-by-column path).
+// Half the voxels of both inputs that the voxel-level tile path holds in shared memory
+// (a tile with more takes the column-by-column path).
 template <int MH>
 constexpr int merge_vstage() { return MH == 512 ? 1536 : (MH == 1024 ? 2560 : 2816); }
 
@@ -232,7 +258,7 @@ constexpr size_t merge_smem_bytes() {
                                                           : merge_vox_bytes<MH>()) + 15) & ~(size_t)15;
 }
 
-// Merge one tile of at most MH columns of each input (one splitter spacing)
+// Merge one tile of at most 2 * MH columns of both inputs together
 // column by column: merge path over the column keys, then per output column
 // its z list (a copy, or the union of two lists).  raw: merge_smem_bytes<MH>()
 // bytes of shared memory, 16-byte aligned.
@@ -248,10 +274,8 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
   constexpr int ZS = merge_stage<MH>();
   uint32_t* s_mk = reinterpret_cast<uint32_t*>(raw);
   uint32_t* s_ka = s_mk + 2 * MH;
-  uint32_t* s_kb = s_ka + MH;
-  uint32_t* s_pa = s_kb + MH;
-  uint32_t* s_pb = s_pa + MH + 1;
-  uint16_t* s_ms = reinterpret_cast<uint16_t*>(s_pb + MH + 1);
+  uint32_t* s_pa = s_ka + 2 * MH;
+  uint16_t* s_ms = reinterpret_cast<uint16_t*>(s_pa + 2 * (MH + 1));
   uint16_t* s_za = s_ms + 2 * MH;
   uint16_t* s_zb = s_za + ZS;
   __shared__ unsigned long long s_warp64[kWarps];
@@ -263,15 +287,17 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
   if (lt >= nt) return;
   const Levels &A = P.a, &B = P.b, &O = P.out;
   const uint32_t b = O.bits, ymask = (1u << b) - 1u;
-  const uint32_t* bnd = bounds + (size_t)kBoundWords * ((size_t)P.tile_base + p + lt);
-  const uint32_t a0 = bnd[0], b0 = bnd[1], sa0 = bnd[2], sb0 = bnd[3];
-  const uint32_t a1 = bnd[4], b1 = bnd[5], sa1 = bnd[6], sb1 = bnd[7];
+  const uint4 lo4 = tile_bound(P, p, S, bounds, ntiles, lt);
+  const uint4 hi4 = tile_bound(P, p, S, bounds, ntiles, lt + 1);
+  const uint32_t a0 = lo4.x, b0 = lo4.y, sa0 = lo4.z, sb0 = lo4.w;
+  const uint32_t a1 = hi4.x, b1 = hi4.y, sa1 = hi4.z, sb1 = hi4.w;
   uint32_t na = a1 - a0, nb = b1 - b0;
-  const bool bad = a1 < a0 || b1 < b0 || na > (uint32_t)MH || nb > (uint32_t)MH;
+  const bool bad = a1 < a0 || b1 < b0 || na + nb > 2u * MH;
   if (bad) {
     na = 0;
     nb = 0;
   }
+  uint32_t *s_kb = s_ka + na, *s_pb = s_pa + na + 1;
   // the slab of the tile's last column: the slab of the next tile's first
   // column, one less when that column opens its slab
   const uint32_t saL = na ? (__ldg(A.ptr2 + sa1) == a1 ? sa1 - 1 : sa1) : sa0;
@@ -322,9 +348,11 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
   for (uint32_t e = tid; e <= nb; e += kThreads) s_pb[e] = nb ? __ldg(B.ptr1 + b0 + e) : 0u;
   __syncthreads();
   // merge path (A first on equal keys); sources: A's column i as i, B's
-  // column j as MH + j
+  // column j as na + j
   const uint32_t n = na + nb;
-  const uint32_t diag = min((uint32_t)(tid * IT), n);
+  // the same number of columns for every thread
+  const uint32_t per = (n + kThreads - 1) / kThreads;
+  const uint32_t diag = min(tid * per, n), dend = min(diag + per, n);
   {
     uint32_t lo = diag > nb ? diag - nb : 0u, hi = min(diag, na);
     while (lo < hi) {
@@ -334,10 +362,10 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
     uint32_t i = lo, j = diag - lo;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
-      if (diag + it >= n) break;
+      if (diag + it >= dend) break;
       const bool takeA = i < na && (j >= nb || s_ka[i] <= s_kb[j]);
       s_mk[diag + it] = takeA ? s_ka[i] : s_kb[j];
-      s_ms[diag + it] = (uint16_t)(takeA ? i : MH + j);
+      s_ms[diag + it] = (uint16_t)(takeA ? i : na + j);
       if (takeA) ++i; else ++j;
     }
   }
@@ -352,20 +380,20 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
   for (int it = 0; it < IT; ++it) {
     cnt[it] = 0;
     const uint32_t ps = diag + it;
-    if (ps >= n) continue;
+    if (ps >= dend) continue;
     const uint32_t key = s_mk[ps];
     if (ps > 0 && s_mk[ps - 1] == key) continue;  // B's copy of a shared column
     const uint32_t src = s_ms[ps];
     const bool pair = ps + 1 < n && s_mk[ps + 1] == key;
     uint32_t c;
     if (pair) {
-      const uint32_t ia = src, ib = s_ms[ps + 1] - MH;
+      const uint32_t ia = src, ib = s_ms[ps + 1] - na;
       const uint32_t za = s_pa[ia], zb = s_pb[ib];
       c = union_count(zAb + za, s_pa[ia + 1] - za, zBb + zb, s_pb[ib + 1] - zb);
-    } else if (src < MH) {
+    } else if (src < na) {
       c = s_pa[src + 1] - s_pa[src];
     } else {
-      c = s_pb[src - MH + 1] - s_pb[src - MH];
+      c = s_pb[src - na + 1] - s_pb[src - na];
     }
     cnt[it] = c;
     const uint32_t x = key >> b;
@@ -402,7 +430,7 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
 #pragma unroll
   for (int it = 0; it < IT; ++it) {
     const uint32_t ps = diag + it;
-    if (ps >= n) continue;
+    if (ps >= dend) continue;
     const uint32_t key = s_mk[ps];
     if (ps > 0 && s_mk[ps - 1] == key) continue;
     const uint32_t src = s_ms[ps];
@@ -415,12 +443,12 @@ __device__ __forceinline__ void merge_tile(const MergePair* __restrict__ pairs, 
     O.idx1[co] = (uint16_t)(key & ymask);
     O.ptr1[co] = vo;
     if (pair) {
-      const uint32_t ia = src, ib = s_ms[ps + 1] - MH;
+      const uint32_t ia = src, ib = s_ms[ps + 1] - na;
       const uint32_t za = s_pa[ia], zb = s_pb[ib];
       union_write(zAb + za, s_pa[ia + 1] - za, zBb + zb, s_pb[ib + 1] - zb, O.idx0 + vo);
     } else {
-      const bool fromA = src < MH;
-      const uint16_t* zz = fromA ? zAb + s_pa[src] : zBb + s_pb[src - MH];
+      const bool fromA = src < na;
+      const uint16_t* zz = fromA ? zAb + s_pa[src] : zBb + s_pb[src - na];
       for (uint32_t q = 0; q < c; ++q) O.idx0[vo + q] = zz[q];
     }
     const uint32_t x = key >> b;
@@ -480,7 +508,7 @@ __device__ __forceinline__ uint32_t next_merge_tile(const MergePair* __restrict_
 // does.  One block scan of (voxels, columns, slabs) and the look-back give the
 // tile's offsets; z entries go out through shared memory in one coalesced
 // pass, column and slab entries straight from the walk.  A tile with more than
-// merge_vstage<MH>() voxels on either side (dense columns) takes the
+// 2 * merge_vstage<MH>() voxels (dense columns) takes the
 // column-by-column path instead.
 template <int MH>
 __device__ __forceinline__ void merge_tile_v(const MergePair* __restrict__ pairs, int S,
@@ -499,11 +527,12 @@ __device__ __forceinline__ void merge_tile_v(const MergePair* __restrict__ pairs
   if (lt >= nt) return;
   const Levels &A = P.a, &B = P.b, &O = P.out;
   const uint32_t b = O.bits, ymask = (1u << b) - 1u;
-  const uint32_t* bnd = bounds + (size_t)kBoundWords * ((size_t)P.tile_base + p + lt);
-  const uint32_t a0 = bnd[0], b0 = bnd[1], sa0 = bnd[2], sb0 = bnd[3];
-  const uint32_t a1 = bnd[4], b1 = bnd[5], sa1 = bnd[6], sb1 = bnd[7];
+  const uint4 lo4 = tile_bound(P, p, S, bounds, ntiles, lt);
+  const uint4 hi4 = tile_bound(P, p, S, bounds, ntiles, lt + 1);
+  const uint32_t a0 = lo4.x, b0 = lo4.y, sa0 = lo4.z, sb0 = lo4.w;
+  const uint32_t a1 = hi4.x, b1 = hi4.y, sa1 = hi4.z, sb1 = hi4.w;
   const uint32_t na = a1 - a0, nb = b1 - b0;
-  const bool bad = a1 < a0 || b1 < b0 || na > (uint32_t)MH || nb > (uint32_t)MH;
+  const bool bad = a1 < a0 || b1 < b0 || na + nb > 2u * MH;
   uint32_t zA0 = 0, zA1 = 0, zB0 = 0, zB1 = 0;
   if (!bad) {
     if (na) {
@@ -516,19 +545,19 @@ __device__ __forceinline__ void merge_tile_v(const MergePair* __restrict__ pairs
     }
   }
   const uint32_t nva = zA1 - zA0, nvb = zB1 - zB0;  // wraps (and so falls back) if corrupt
-  if (bad || nva > (uint32_t)VS || nvb > (uint32_t)VS) {
+  if (bad || nva > 2u * VS || nvb > 2u * VS || nva + nvb > 2u * VS) {
     merge_tile<MH>(pairs, S, bounds, ntiles, clook, t, p, raw);
     return;
   }
   unsigned long long* s_va = reinterpret_cast<unsigned long long*>(raw);
-  unsigned long long* s_vb = s_va + VS;
-  uint16_t* s_oz = reinterpret_cast<uint16_t*>(s_vb + VS);  // 2 * VS output z entries
+  unsigned long long* s_vb = s_va + nva;
+  uint16_t* s_oz = reinterpret_cast<uint16_t*>(s_va + 2 * VS);  // 2 * VS output z entries
   // staged entries of the tile's columns and slabs (the same region as s_oz)
-  uint32_t* s_pa = reinterpret_cast<uint32_t*>(s_vb + VS);  // Y_pointer, na + 1
-  uint32_t* s_pb = s_pa + MH + 1;
-  uint16_t* s_ya = reinterpret_cast<uint16_t*>(s_pb + MH + 1);  // Y_index, na
-  uint16_t* s_yb = s_ya + MH;
-  uint32_t* s_xpa = reinterpret_cast<uint32_t*>(s_yb + MH);  // X_pointer of the slabs
+  uint32_t* s_pa = reinterpret_cast<uint32_t*>(s_va + 2 * VS);  // Y_pointer, na + 1
+  uint32_t* s_pb = s_pa + na + 1;
+  uint16_t* s_ya = reinterpret_cast<uint16_t*>(s_pa + 2 * (MH + 1));  // Y_index, na
+  uint16_t* s_yb = s_ya + na;
+  uint32_t* s_xpa = reinterpret_cast<uint32_t*>(s_ya + 2 * MH);  // X_pointer of the slabs
   uint32_t* s_xpb = s_xpa + kMergeSlabStage;
   uint16_t* s_xa = reinterpret_cast<uint16_t*>(s_xpb + kMergeSlabStage);  // X_index
   uint16_t* s_xb = s_xa + kMergeSlabStage;
@@ -613,7 +642,8 @@ __device__ __forceinline__ void merge_tile_v(const MergePair* __restrict__ pairs
   // merge path over the tile's voxels (A first on equal keys), the same
   // number of merged positions for every thread
   const uint32_t nv = nva + nvb;
-  const uint32_t per = (nv + kThreads - 1) / kThreads;
+  // (an odd number: their keys lie in different banks)
+  const uint32_t per = ((nv + kThreads - 1) / kThreads) | 1u;
   const uint32_t diag = min(tid * per, nv), dend = min(diag + per, nv);
   uint32_t i0, j0;
   {
@@ -1246,7 +1276,7 @@ size_t merge_scratch_bytes(uint32_t total_spl, uint32_t total_tiles, int S) {
   (void)total_spl;
   size_t b = 0;
   b += align_up(((size_t)total_tiles + S) * kBoundWords * 4 + 16);
-  b += align_up((size_t)S * 4);
+  b += align_up((size_t)S * 3 * 4);
   b += align_up((size_t)total_tiles * 3 * 4);
   b += align_up(4);
   b += align_up((size_t)S * sizeof(MergePair));
@@ -1262,7 +1292,7 @@ MergeScratch merge_scratch_carve(void* base, uint32_t total_spl, uint32_t total_
   sc.bounds = reinterpret_cast<uint32_t*>(p);
   p += align_up(((size_t)total_tiles + S) * kBoundWords * 4 + 16);
   sc.ntiles = reinterpret_cast<uint32_t*>(p);
-  p += align_up((size_t)S * 4);
+  p += align_up((size_t)S * 3 * 4);
   char* z0 = p;
   sc.clook = reinterpret_cast<uint32_t*>(p);
   p += align_up((size_t)total_tiles * 3 * 4);
@@ -1317,9 +1347,14 @@ cudaError_t run_merge_device(int S, uint32_t total_spl, uint32_t total_tiles,
     }
     return cudaGetLastError();
   }
-  k_merge_init<<<(S + 127) / 128, 128, 0, stream>>>(sc.pairs, S, sc.half, sc.bounds, sc.ntiles);
+  const uint32_t spacing = merge_spacing(sc.half, false);
+  const uint32_t stage = sc.half == 512 ? merge_vstage<512>()
+                                        : (sc.half == 1024 ? merge_vstage<1024>() : merge_vstage<2048>());
+  k_merge_init<<<(S + 127) / 128, 128, 0, stream>>>(sc.pairs, S, spacing, 2 * stage * 4 / 5,
+                                                   4 * (uint32_t)device_sm_count(), sc.bounds,
+                                                   sc.ntiles);
   if (total_spl > 0) {
-    k_merge_cuts<<<(total_spl + 7) / 8, 256, 0, stream>>>(sc.pairs, S, total_spl, sc.half,
+    k_merge_cuts<<<(total_spl + 7) / 8, 256, 0, stream>>>(sc.pairs, S, total_spl, spacing,
                                                          sc.bounds);
   }
   if (sc.half == 512) {

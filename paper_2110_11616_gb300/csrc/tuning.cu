@@ -50,10 +50,10 @@ Tuning tuning_for(uint32_t bits, uint64_t n) {
 // The partition of merges whose entry was never set, from what the host knows:
 // the grid, and the points the two inputs can hold (of the largest pair of a
 // launch).  Measured per merge on GB300 (512 / 1024 / 2048, us):
-//   column level, 2 x 100k uniform points at b = 10      38.6 / 37.2 /  44.1
-//                 2 x 1M surface points at b = 12       101.6 / 78.6 /  83.8
-//                 2 x 10M surface points at b = 12        482 /  329 /   592
-//                 2 x 10M uniform points at b = 10        280 /  642 /  1069
+//   column level, 2 x 100k uniform points at b = 10      37.8 / 36.5 /  42.0
+//                 2 x 1M surface points at b = 12        79.4 / 67.2 /  77.8
+//                 2 x 10M surface points at b = 12        347 /  257 /   612
+//                 2 x 10M uniform points at b = 10        261 /  542 /   751
 //   key level,    2 x 300k LiDAR points at b = 16        84.9 / 63.7 /  61.7
 //                 2 x 3M                                  348 /  218 /   176
 // Small merges want many tiles; when the points outnumber the grid's columns

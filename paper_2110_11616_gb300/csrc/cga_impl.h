@@ -537,9 +537,10 @@ inline uint32_t nn_kind(const NnSeg& s) { return s.tree.levels > 0 ? 3u : s.ncoa
 // Run with the tables on the device (capturable: memsets and kernels only).
 // kinds: bit k set when some segment has nn_kind k (selects the kernels: the
 // tree search for segments with a tree, the window search of the largest
-// other kind for the rest).
+// other kind for the rest); only: the single segment of the tables, where the host
+// knows it (few queries then get several warps each), or null.
 cudaError_t run_nn_device(int S, uint32_t total_tiles, const NnTables& t, cudaStream_t stream,
-                          uint32_t kinds = 1u);
+                          uint32_t kinds = 1u, const NnSeg* only = nullptr);
 
 // For each slab k of the coarse CGA c (cells of 2^shift voxels), xs[k] = first
 // index of a's X_index whose x >> shift equals c's X_index[k]; xs[h_c] = h_a.

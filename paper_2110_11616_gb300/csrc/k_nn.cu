@@ -239,7 +239,7 @@ __device__ __forceinline__ void search_fine(const Levels& a, const uint32_t* xdi
 }
 
 // The same search in 32-bit distances, for queries within 2^16 of their nearest voxel
-// (false when no voxel nearer than that was found: the 64-bit form then decides).
+// (where none nearer than that is found, the 64-bit form decides).
 // A coordinate difference beyond 16 bits, or a sum beyond the bound, drops its
 // candidate, so nothing wraps.
 struct Best32 {
@@ -254,6 +254,22 @@ struct Best32 {
     const uint32_t m = __reduce_min_sync(0xffffffffu, d2);
     idx = __reduce_min_sync(0xffffffffu, d2 == m ? idx : 0xffffffffu);
     d2 = m;
+  }
+  // the same over a block of NW warps
+  template <int NW>
+  __device__ __forceinline__ void team_min() {
+    warp_min();
+    if constexpr (NW > 1) {
+      __shared__ uint32_t s_d[NW], s_i[NW];
+      if ((threadIdx.x & 31u) == 0) {
+        s_d[threadIdx.x >> 5] = d2;
+        s_i[threadIdx.x >> 5] = idx;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < NW; ++w) offer(s_d[w], s_i[w]);
+      __syncthreads();
+    }
   }
   // base + d^2 within the bound (base is)
   __device__ __forceinline__ bool within(uint32_t base, uint32_t d) const {
@@ -292,15 +308,21 @@ __device__ __forceinline__ void visit_column32(const Levels& a, const uint4* cta
 // 32 (bound by the latency of the dependent loads: a slab directory that replaced the
 // bisection in y, three probes a round, or the columns dealt out evenly over the lanes
 // all took longer, 2.4 to 2.8 against 2.4 at the time).
+//
+// NW warps a query, in thread order (a block, when more than one): each thread takes a
+// slab a round, 16 NW on each side, the first k0 on each side being done.  False when
+// `rounds` were not enough (best then holds what they found).
+template <int NW>
 __device__ __forceinline__ bool search_fine32(const Levels& a, const uint32_t* xdir,
-                                            const uint4* ctab, uint32_t h,
-                                            int qx, int qy, int qz,
-                                            uint32_t cqx, uint32_t cqy, uint32_t cqz,
-                                            uint32_t lane, Best32& best) {
+                                              const uint4* ctab, uint32_t h,
+                                              int qx, int qy, int qz,
+                                              uint32_t cqx, uint32_t cqy, uint32_t cqz,
+                                              uint32_t thread, uint32_t k0, uint32_t rounds,
+                                              Best32& best) {
   const uint32_t xr0 = xdir != nullptr ? __ldg(xdir + cqx) : lower_bound_u16(a.idx2, 0, h, cqx);
-  const bool right = (lane & 1u) == 0u;
+  const bool right = (thread & 1u) == 0u;
   for (uint32_t r = 0;; ++r) {
-    const int k = (int)(r * 16u + (lane >> 1));
+    const int k = (int)(k0 + r * (16u * NW) + (thread >> 1));
     const int slab = right ? (int)xr0 + k : (int)xr0 - 1 - k;
     const bool valid = slab >= 0 && slab < (int)h;
     uint32_t dx2 = 0;
@@ -314,7 +336,8 @@ __device__ __forceinline__ bool search_fine32(const Levels& a, const uint32_t* x
       dx2 = dx * dx;
     }
     const bool active = valid && best.within(0, dx);
-    if (!__any_sync(0xffffffffu, active)) break;
+    if (NW == 1 ? !__any_sync(0xffffffffu, active) : !__syncthreads_or(active)) return true;
+    if (r == rounds) return false;
     if (active) {
       yr0 = lower_bound_u16(a.idx1, ys, ye, cqy);
       if (yr0 < ye) {
@@ -328,7 +351,7 @@ __device__ __forceinline__ bool search_fine32(const Levels& a, const uint32_t* x
         if (best.within(dx2, dy)) visit_column32(a, ctab, yr0 - 1, dx2 + dy * dy, qz, cqz, best);
       }
     }
-    best.warp_min();
+    best.team_min<NW>();
     if (active) {
       int R2 = (int)yr0 + 1, L2 = (int)yr0 - 2;
       while (true) {
@@ -344,9 +367,8 @@ __device__ __forceinline__ bool search_fine32(const Levels& a, const uint32_t* x
         visit_column32(a, ctab, c, dx2 + dy * dy, qz, cqz, best);
       }
     }
-    best.warp_min();
+    best.team_min<NW>();
   }
-  return best.d2 != 0xffffffffu;
 }
 
 // Distance from q to the voxel interval [lo, lo + s - 1] (0 inside).
@@ -1434,23 +1456,48 @@ __global__ void __launch_bounds__(kTreeThreads, CGA_NN_TREE_BLOCKS)
   }
 }
 
+// A query that its warp left to the block after so many rounds, and the best of those.
+// A launch of few queries waits for its slowest one: a warp takes a round for every 16
+// slabs on a side, and 1% of a LiDAR world's queries span 116 slabs a side.  Once a
+// block's warps have no more queries, they share the long ones: 128 slabs on a side a
+// round.  Where every query is long, shared ones are the slower way (a block does one at
+// a time), so they are left to it the sooner the fewer queries a block has: after one
+// round up to two a block, four up to 8, then 16 (in batches 32: of 16 mixed clouds, 1664
+// us a pass without, 1666 so and 1676 after 16 rounds), and beyond 128 a block, where the
+// turns even them out, never (LONG: 1M queries 1.99 ms with, 1.97 without).  Calls on
+// GB300, us, without and with the blocks' help: 1000 queries of a 1.3M-point LiDAR world,
+// b = 16, 95 and 56; 7000 147 and 124; of a 1M-point one, b = 15, 14000 424 and 158,
+// 100000 542 and 306; of 2M surface points, b = 15, 481 and 482; of 1M uniform points, b
+// = 10, 1500 38 and 36, 100000 340 and 342.  (Blocks that share every query from its
+// first round: 1000 53, but 1500 of the uniform points 51 and 100000 540.)
+struct LongQuery {
+  uint32_t slot, j;
+  Best32 best;
+};
+constexpr uint32_t kLongQueries = 32;
+constexpr uint32_t kFewRounds = 4;  // with up to 8 queries a block
+
 // NC: the most coarse levels any segment of the launch carries (0, 1 or 2).
 // The fine-only instantiation is held to 40 registers (six blocks per SM),
 // the coarse ones to 48 (five blocks per SM): the extra warps hide more of
 // the search's load latency than the spilled values cost (eight and six
 // blocks respectively spill enough to be slower).
-template <int NC>
+template <int NC, bool LONG = false>
 __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FINE_BLOCKS)
     k_nn_warp(const NnSeg* __restrict__ segs, int S, NnSeg inline_seg, uint32_t total_slots,
               const unsigned long long* __restrict__ order,
-              const unsigned int* __restrict__ order_err) {
+              const unsigned int* __restrict__ order_err, uint32_t rounds) {
   const uint32_t lane = threadIdx.x & 31;
   constexpr uint32_t W = 256 / 32;
   __shared__ uint32_t s_next;
+  __shared__ uint32_t s_nlong;
+  __shared__ LongQuery s_long[LONG ? kLongQueries : 1];
+  if (LONG && threadIdx.x == 0) s_nlong = 0;
   open_slots<W>(&s_next);
   const bool sorted = order != nullptr && (order_err == nullptr || *order_err == 0u);
   for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
-    const uint32_t slot = slot_of_turn<W>(turn);
+    // (few queries: one a block before any has two)
+    const uint32_t slot = LONG && rounds <= kFewRounds ? blockIdx.x + turn * gridDim.x : slot_of_turn<W>(turn);
     if (slot >= total_slots) break;
     const uint32_t tile = slot / (uint32_t)kTile;
     const NnSeg& sg = segs != nullptr ? segs[find_nn_seg(segs, S, tile)] : inline_seg;
@@ -1487,7 +1534,20 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
       }
     } else {
       Best32 near{0xffffffffu, 0xffffffffu};
-      if (search_fine32(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, near)) {
+      bool done = search_fine32<1>(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, 0,
+                                   LONG ? rounds : 0xffffffffu, near);
+      if (LONG && !done) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&s_nlong, 1u);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at < kLongQueries) {
+          if (lane == 0) s_long[at] = LongQuery{slot, j, near};
+          continue;
+        }
+        search_fine32<1>(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, 16 * rounds,
+                         0xffffffffu, near);
+      }
+      if (near.d2 != 0xffffffffu) {
         best.d2 = near.d2;
         best.idx = near.idx;
       } else {
@@ -1497,6 +1557,34 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
     if (lane == 0) {
       __stcs(sg.idx + j, best.idx);
       __stcs(sg.d2 + j, best.d2);
+    }
+  }
+  if constexpr (LONG) {
+    __syncthreads();
+    const uint32_t n = min(s_nlong, kLongQueries);
+    for (uint32_t i = 0; i < n; ++i) {
+      const uint32_t slot = s_long[i].slot, j = s_long[i].j;
+      const NnSeg& sg = segs != nullptr ? segs[find_nn_seg(segs, S, slot / (uint32_t)kTile)]
+                                        : inline_seg;
+      int qx, qy, qz;
+      query_voxel(sg, j, qx, qy, qz);
+      const int top = (1 << sg.a.bits) - 1;
+      const uint32_t cqx = (uint32_t)min(max(qx, 0), top);
+      const uint32_t cqy = (uint32_t)min(max(qy, 0), top);
+      const uint32_t cqz = (uint32_t)min(max(qz, 0), top);
+      const uint32_t h = (uint32_t)sg.a.hdr->cnt[2];
+      Best32 near = s_long[i].best;
+      search_fine32<W>(sg.a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, threadIdx.x,
+                       16 * rounds, 0xffffffffu, near);
+      Best best{near.d2, near.idx};
+      if (near.d2 == 0xffffffffu && threadIdx.x < 32) {
+        best = Best{~0ull, 0xffffffffu};
+        search_fine(sg.a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, threadIdx.x, best);
+      }
+      if (threadIdx.x == 0) {
+        __stcs(sg.idx + j, best.idx);
+        __stcs(sg.d2 + j, best.d2);
+      }
     }
   }
 }
@@ -1562,7 +1650,7 @@ static uint32_t resident_blocks(uint32_t kind) {
   int n = cache[kind].load(std::memory_order_relaxed);
   if (n == 0) {
     cudaError_t e = cudaErrorInvalidValue;
-    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<0>, 256, 0);
+    if (kind == 0) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<0, true>, 256, 0);
     if (kind == 1) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<1>, 256, 0);
     if (kind == 2) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nn_warp<2>, 256, 0);
     if (kind == 3) {
@@ -1629,16 +1717,24 @@ static void launch_search(const NnSeg* d_segs, int S, const NnSeg& inline_seg,
   kinds &= 7u;
   if (kinds == 0) return;
   const uint32_t kind = kinds >= 4u ? 2u : (kinds >= 2u ? 1u : 0u);
-  const uint32_t blocks = std::min<uint32_t>((total_slots + 7) / 8, sms * resident_blocks(kind));
+  const uint32_t most = sms * resident_blocks(kind);
+  const uint32_t n = inline_seg.m > 0 ? inline_seg.m : total_slots;
+  // few queries: spread over the blocks, and left to them early (see LongQuery)
+  const bool few = kind == 0 && n <= 8 * most;
+  const uint32_t blocks = std::min<uint32_t>(few ? n : (total_slots + 7) / 8, most);
+  const uint32_t rounds = n <= 2 * most ? 1u : (few ? kFewRounds : (S == 1 ? 16u : 32u));
+  const uint32_t slots = few && inline_seg.m > 0 ? n : total_slots;
   if (kind == 2) {
     k_nn_warp<2><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg, total_slots, order,
-                                             order_err);
+                                             order_err, rounds);
   } else if (kind == 1) {
     k_nn_warp<1><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg, total_slots, order,
-                                             order_err);
+                                             order_err, rounds);
+  } else if (S > 1 || n <= 128 * most) {
+    k_nn_warp<0, true><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg, slots, order, order_err,
+                                                   rounds);
   } else {
-    k_nn_warp<0><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg, total_slots, order,
-                                             order_err);
+    k_nn_warp<0><<<blocks, 256, 0, stream>>>(d_segs, S, inline_seg, slots, order, order_err, 0u);
   }
   count_launch(1);
 }
@@ -1666,7 +1762,7 @@ cudaError_t run_nn_search(const NnSeg& seg, const unsigned long long* order, cud
 }
 
 cudaError_t run_nn_device(int S, uint32_t total_tiles, const NnTables& t, cudaStream_t stream,
-                          uint32_t kinds) {
+                          uint32_t kinds, const NnSeg* only) {
   if (total_tiles == 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(t.err, 0, sizeof(Header), stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(t.sort.hist, 0, t.sort.zero_bytes, stream);
@@ -1677,7 +1773,7 @@ cudaError_t run_nn_device(int S, uint32_t total_tiles, const NnTables& t, cudaSt
   e = run_radix_passes(S, total_tiles, 4, true, t.sort, stream);
   if (e != cudaSuccess) return e;
   // four passes leave the sorted keys in keys0
-  launch_search(t.segs, S, NnSeg{}, total_tiles,
+  launch_search(t.segs, S, only != nullptr ? *only : NnSeg{}, total_tiles,
                 static_cast<const unsigned long long*>(t.sort.keys0), &t.err->err, kinds, stream);
   return cudaGetLastError();
 }
@@ -1696,7 +1792,7 @@ cudaError_t run_nn(const NnSeg* h_segs, int S, uint32_t total_tiles, void* scrat
   if (e != cudaSuccess) return e;
   uint32_t kinds = 0;
   for (int s = 0; s < S; ++s) kinds |= 1u << nn_kind(h_segs[s]);
-  return run_nn_device(S, total_tiles, t, stream, kinds);
+  return run_nn_device(S, total_tiles, t, stream, kinds, S == 1 ? h_segs : nullptr);
 }
 
 }  // namespace libcga

@@ -1071,7 +1071,14 @@ __global__ void k_x_directory(Levels a, uint32_t* xdir) {
 __device__ __forceinline__ void project_xy_body(const Levels& a, const Levels& o, uint32_t t,
                                                 uint32_t stride) {
   const uint32_t g = (uint32_t)a.hdr->cnt[1], h = (uint32_t)a.hdr->cnt[2];
-  for (uint32_t i = t; i < g; i += stride) o.idx0[i] = a.idx1[i];
+  uint32_t i0 = 0;  // eight entries a load where both arrays allow
+  if (((reinterpret_cast<uintptr_t>(a.idx1) | reinterpret_cast<uintptr_t>(o.idx0)) & 15u) == 0) {
+    const uint4* src = reinterpret_cast<const uint4*>(a.idx1);
+    uint4* dst = reinterpret_cast<uint4*>(o.idx0);
+    i0 = g & ~7u;
+    for (uint32_t i = t; i < g / 8; i += stride) dst[i] = __ldg(src + i);
+  }
+  for (uint32_t i = i0 + t; i < g; i += stride) o.idx0[i] = a.idx1[i];
   for (uint32_t i = t; i < h; i += stride) o.idx1[i] = a.idx2[i];
   for (uint32_t i = t; i <= h; i += stride) o.ptr1[i] = a.ptr2[i];
   if (t == 0) {
@@ -1386,7 +1393,7 @@ cudaError_t run_merge(const MergePair* h_pairs, int S, uint32_t total_spl, uint3
 
 cudaError_t run_project_xy(const Levels& a, const Levels& out, cudaStream_t stream) {
   const uint64_t work = std::max<uint64_t>(a.cap1, 1);
-  const unsigned blocks = (unsigned)std::min<uint64_t>((work + 255) / 256,
+  const unsigned blocks = (unsigned)std::min<uint64_t>((work + 2047) / 2048,
                                                        (uint64_t)device_sm_count() * 8);
   k_project_xy<<<blocks, 256, 0, stream>>>(a, out);
   count_launch(1);
@@ -1461,7 +1468,10 @@ cudaError_t run_x_directory(const Levels& a, uint32_t* xdir, cudaStream_t stream
 cudaError_t run_project_xy_device(const ProjPair* d_pairs, int S, uint64_t max_cap1,
                                   cudaStream_t stream) {
   if (S == 0) return cudaSuccess;
-  const unsigned bx = (unsigned)std::min<uint64_t>((std::max<uint64_t>(max_cap1, 1) + 255) / 256, 64);
+  // a batch waits for its largest cloud: 64 blocks copying two bytes a thread took 108
+  // us for one of 2M columns among 16, blocks for eight entries a thread 13
+  const unsigned bx = (unsigned)std::min<uint64_t>((std::max<uint64_t>(max_cap1, 1) + 2047) / 2048,
+                                                   2 * (uint64_t)device_sm_count());
   k_project_xy_batch<<<dim3(bx, (unsigned)S), 256, 0, stream>>>(d_pairs);
   count_launch(1);
   return cudaGetLastError();

@@ -80,6 +80,15 @@ def parse():
     return ap.parse_args()
 
 
+def build_bytes(points, bits, infos):
+    """Bytes the builds by bins move by design: the points twice (bin counts, partition),
+    each key written and read once, each distinct key likewise, and the CGAs; a key is 4
+    bytes where the 12-bit bin and 32 bits give it."""
+    key = 4 if 3 * bits - min(bits, 12) <= 30 else 8
+    return (points * (24 + 2 * key) + 2 * key * sum(i["u"] for i in infos)
+            + sum(i["bytes"] for i in infos))
+
+
 def measured_peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -673,8 +682,7 @@ def run_surface(args, world_size, local_rank, torch, dist, cga):
     algo = S_QUERIES * (12 + 4 + 8)
     achieved = algo / (search_ms / 1e3) / 1e9
     traffic, traffic_note = profiled_traffic(TRAFFIC_PROFILE, NN_SOURCES)
-    passes = math.ceil(3 * S_BITS / shapes[str(S_POINTS // 2)]["shape"]["radix_bits"])
-    build_design = (S_POINTS * (12 + 8 + 16 * passes + 8) + ai["bytes"] + bi["bytes"])
+    build_design = build_bytes(S_POINTS, S_BITS, (ai, bi))
     out = base_line(args, world_size, METRIC, value, "Mpts/s", max_total / args.steps,
                     surface_config(args, world_size),
                     "synthetic (seeded superellipsoid surfaces; stands in for the paper's "
@@ -800,8 +808,8 @@ def run_single(args, world_size, local_rank, torch, cga, which):
                     "merge_GB_s": round(merge_bytes / (ops[1] / 1e3) / 1e9, 2),
                     "merge_frac_of_hbm": round(merge_bytes / (ops[1] / 1e3) / 1e9 / peak, 4),
                     "build_by_design_GB_s": round(
-                        (n_points * (12 + 8 + 16 * math.ceil(3 * grid.bits / 8) + 8)
-                         + a.info()["bytes"] + b.info()["bytes"]) / (ops[0] / 1e3) / 1e9, 1),
+                        build_bytes(n_points, grid.bits, (a.info(), b.info()))
+                        / (ops[0] / 1e3) / 1e9, 1),
                     "merged_u": mi["u"], "merged_bytes": mi["bytes"], "raw_bytes": n_points * 12,
                     "peak_gbs": peak, "peak_source": peak_kind},
         "nn_autotune": tune_record(coarse_shift, nn_tune),

@@ -697,8 +697,10 @@ __device__ void search_levels(const NnSeg& sg, const Qry& q, uint32_t lane, Best
 
 // ---- occupancy-tree search (cga_nn_prepare_levels with CGA_NN_TREE) -------
 //
-// A depth-first descent of the 64-ary occupancy tree (k_tree.cu), nearest
-// child first, by a group of G lanes per query (32 / G queries per warp).
+// Two forms over the 64-ary occupancy tree (k_tree.cu), by a group of G lanes per
+// query (32 / G queries per warp): breadth-first through a queue of nodes (search_bfs),
+// and, for a query whose queue would overflow, the following depth-first descent,
+// nearest child first.
 // Lane g of a group owns the children numbered [g * 64/G, (g + 1) * 64/G)
 // of every node (tree_child numbers, so the children of a planar patch of
 // surface spread evenly over the lanes).  Each step the lanes bound their
@@ -1027,7 +1029,8 @@ __device__ void search_tree(const TreeView& tv, const Qry& q, uint32_t b, bool a
 //
 // Measured, search kernels alone: 4M surface-world queries, half of them far
 // from any voxel, 29.7 -> 17.2 ms; 20M voxels moved about five voxels off the
-// surfaces 31.9 -> 21.4 ms.  Still bound by instruction issue (70%, 24 of 32
+// surfaces 31.9 -> 21.4 ms; with warps taking their block's next queries when free 15.6
+// and 21.1.  Still bound by instruction issue (70%, 24 of 32
 // lanes active; 4.3k warp instructions a far query, 1k a near one): per warp of
 // four far queries 39 nodes and 127 groups of children, the longest child list
 // of the four setting each round.  Sixteen lanes a query take 8% less on far

@@ -18,7 +18,8 @@
 // slabs by search, the fill walking every slab twice; 3.9 ms before the grid was
 // cut to one wave and the hits staged for whole-sector stores).  k-NN of the
 // same queries: k = 8 6.9 -> 5.7 ms, k = 400 (100k queries) 16.0 -> 11.4 ms with
-// pairs of one 64-bit word; bound by instruction issue (63%).
+// pairs of one 64-bit word.  Warps taking their block's next query when free: radius
+// 3.0 ms, k = 8 5.3, k = 400 11.1; bound by instruction issue and load latency.
 #include <algorithm>
 #include <cmath>
 #include <mutex>

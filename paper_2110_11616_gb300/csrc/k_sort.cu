@@ -1,4 +1,6 @@
-// Sort pipeline of the CGA build (and of the xz / yz projections):
+// Sort pipeline of the CGA build (and of the xz / yz projections): builds from points
+// go by bins where plan_bins says so (k_bins.cuh), the others, and what the bins leave
+// over (k_lsd_all, all of the following in one launch), by LSD radix passes:
 //   k_seg_init     headers and empty-CGA sentinels
 //   k_keys_hist    quantize (+ rigid transform) and encode each point, or
 //                  re-key a CGA point for a projection; per-segment digit

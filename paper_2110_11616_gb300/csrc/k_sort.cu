@@ -555,6 +555,9 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
     const uint64_t most = g.narrow ? 4 * bin_cap<uint32_t>() : 4 * bin_cap<unsigned long long>();
     if (g.n_host >> g.bin_bits > most) return;
     B.may_split = B.may_split || g.n_host > (g.narrow ? bin_cap<uint32_t>() : bin_cap<unsigned long long>());
+    // a job fails by its keys' number or, wide keys only, by its row's parts
+    B.may_fall = B.may_fall || g.n_host > kBinRowMax ||
+                 (!g.narrow && g.n_host > bin_cap<unsigned long long>());
     B.narrow = B.narrow || g.narrow;
     B.wide = B.wide || !g.narrow;
     points += g.n_host;
@@ -694,13 +697,13 @@ static cudaError_t run_bins(int S, uint32_t total_tiles, bool key64, const SortS
   if (B.narrow) launch_bin_write<uint32_t>(S, sc, stride, stream);
   if (B.wide) launch_bin_write<unsigned long long>(S, sc, stride, stream);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && B.may_fall) {
     e = key64 ? launch_lsd_all<unsigned long long>(S, total_tiles, sc, stream)
               : launch_lsd_all<uint32_t>(S, total_tiles, sc, stream);
   }
-  count_launch(3 + (B.may_split ? 5 : 4) * ((B.narrow ? 1 : 0) + (B.wide ? 1 : 0)));
+  count_launch((B.may_fall ? 3 : 2) + (B.may_split ? 5 : 4) * ((B.narrow ? 1 : 0) + (B.wide ? 1 : 0)));
   // the Value array of a cloud that the general sort had to take
-  if (e == cudaSuccess && B.value_rows != nullptr) {
+  if (e == cudaSuccess && B.value_rows != nullptr && B.may_fall) {
     e = run_build_values(B.value_out, B.value_in, B.value_rows, B.values, &sc.segs[0].fallback,
                          stream);
   }

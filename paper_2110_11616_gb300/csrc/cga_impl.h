@@ -96,6 +96,7 @@ struct SortSeg {
   // bin_base .. of the bin tables, partition tiles from ptile_base, job slots
   // [job_base, + job_cap)
   uint32_t bin_bits, bin_base, ptile_base, job_base, job_cap;
+  uint32_t job_keys;    // about as many keys a job
   uint32_t narrow;      // its partitioned keys have 32 bits
   uint32_t fallback;    // set on the device: sort this segment the general way
 };

@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
   const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
   SortSeg& sg = segs[blockIdx.x];
   if (sg.narrow != (sizeof(T) == 4 ? 1u : 0u)) return;
-  const uint32_t bins = 1u << sg.bin_bits;
+  const uint32_t bins = 1u << sg.bin_bits, target = sg.job_keys;
   uint32_t c[PER], sum = 0, tot = 0;
 #pragma unroll
   for (uint32_t i = 0; i < PER; ++i) {
@@ -278,14 +278,14 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
     if (b >= bins) continue;
     const uint32_t st = s_start[b], n = s_start[b + 1] - st;
     const uint32_t pst = b > 0 ? s_start[b - 1] : 0u;
-    const bool large = n > bin_target<T>(), plarge = b > 0 && st - pst > bin_target<T>();
-    if (b == 0 || large || plarge || st / bin_target<T>() != pst / bin_target<T>() ||
+    const bool large = n > target, plarge = b > 0 && st - pst > target;
+    if (b == 0 || large || plarge || st / target != pst / target ||
         (b & ((1u << span_bits) - 1u)) == 0u) {
       nsub[i] = 1;
       if (n > kBinSplitMax) {
         sg.fallback = 1;
       } else if (n > bin_cap<T>()) {
-        nsub[i] = split_slots(n, bin_target<T>());
+        nsub[i] = split_slots(n, target);
       }
       nj += nsub[i];
       open |= 1u << i;
@@ -525,7 +525,7 @@ __global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(kBinThread
     if (sg.narrow != (sizeof(T) == 4 ? 1u : 0u) || sg.fallback) continue;
     const uint32_t rank = alone ? 0u : cluster_rank(), parts = alone ? 1u : kBinCluster;
     const uint4 job = jobs[B.y];
-    const uint32_t b = sg.bits, rem = 3 * b - sg.bin_bits, N = job.w;
+    const uint32_t b = sg.bits, rem = 3 * b - sg.bin_bits, N = job.w, target = sg.job_keys;
     const uint32_t rb = min(kBinRowBits, rem - b), shift = rem - rb, rows = 1u << rb;
     // rows of one slab: those that share the key's x bits below the bin's
     const uint32_t xb = min(rb, b - sg.bin_bits), slab = rb - xb;
@@ -599,8 +599,8 @@ __global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(kBinThread
     for (uint32_t k = 0; k < PER; ++k) {
       const uint32_t r = tid * PER + k;
       const uint32_t p = s_pre[r], q = r > 0 ? s_pre[r - 1] : 0u;
-      if (r < rows && (r == 0 || c[k] > bin_target<T>() || p - q > bin_target<T>() ||
-                       p / bin_target<T>() != q / bin_target<T>())) {
+      if (r < rows && (r == 0 || c[k] > target || p - q > target ||
+                       p / target != q / target)) {
         open |= 1u << k;
         ++nj;
       }
@@ -617,7 +617,7 @@ __global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(kBinThread
     uint32_t j = block_scan_th<kBinThreads>(nj, tot, s_scan);
     for (uint32_t x = w + 1; x < (uint32_t)kBinWarps; ++x) after = min(after, s_next[x]);
     // the first block writes the jobs
-    const uint32_t slots = rank == 0 ? split_slots(N, bin_target<T>()) : 0u;
+    const uint32_t slots = rank == 0 ? split_slots(N, target) : 0u;
 #pragma unroll
     for (int k = (int)PER - 1; k >= 0; --k) {
       if (!((open >> k) & 1u)) continue;

@@ -570,7 +570,13 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
     SortSeg& g = h_segs[s];
     const uint32_t nb = 1u << g.bin_bits, rem = 3 * g.bits - g.bin_bits;
     const uint32_t span = g.narrow ? std::min(32u - rem, kBinMaxBits) : kBinMaxBits;
-    const uint32_t target = g.narrow ? bin_target<uint32_t>() : bin_target<unsigned long long>();
+    // jobs of half a block's capacity, smaller ones while they are too few for the SMs:
+    // 100k uniform points, b = 10, 65 us with half a block, 57 with 1024 keys and up,
+    // 100k LiDAR points, b = 12, 73 and 59, ten sweeps of 131k, b = 13, 175 and 157
+    // (eight jobs an SM, not four: 1M uniform points 84 and 93)
+    const uint32_t most_keys = g.narrow ? bin_target<uint32_t>() : bin_target<unsigned long long>();
+    const uint32_t target = (uint32_t)std::min<uint64_t>(most_keys, std::max<uint64_t>(1024, points / (4 * sms)));
+    g.job_keys = target;
     g.bin_base = (uint32_t)bins;
     g.ptile_base = (uint32_t)ptiles;
     g.job_base = (uint32_t)slots;

@@ -103,6 +103,7 @@ constexpr uint32_t bin_target() { return bin_cap<T>() / 2; }
 // keys up to which a bucket is ordered by counting.
 constexpr uint32_t kBinBucketBits = 12;
 constexpr uint32_t kBinBucketMax = 48;
+constexpr uint32_t kBinWork = 64;  // comparisons a key, on average, in crowded buckets
 
 // Dynamic shared memory of k_bin_sort: both key buffers, the bucket counts (or the
 // warps' digit counts of the LSD passes), a bitmap per warp and the offsets of a
@@ -673,6 +674,7 @@ struct BinSortSmem {
   uint32_t slot;
   int seg;
   uint32_t nbig;
+  uint32_t work;
   uint16_t big[(2 * bin_cap<uint32_t>()) / kBinBucketMax];  // buckets beyond kBinBucketMax
 };
 
@@ -751,7 +753,11 @@ __device__ __forceinline__ T* bin_block_sort(T* a, T* b, uint32_t n, uint32_t bi
 // their barriers.  A bucket of more than kBinBucketMax keys (duplicates of one
 // voxel, a dense column) goes through a warp's bitmap of what is left of its keys:
 // its distinct keys in order, the rest of its places filled with the last of them.
-// Where that takes more than 12 bits, the block falls back to the stable passes.
+// Where that takes more than 12 bits, the keys of such buckets are counted like the
+// others, or the whole block falls back to the stable passes when that means more than
+// kBinWork comparisons a key (by one bucket's size, 384 keys, instead: ten LiDAR sweeps
+// of 131k at b = 13 157 us against 134, 15M surface points at b = 13 534 against 510;
+// limits of 32 to 96 are within 1% of each other, 160 and none slower).
 template <typename T>
 __device__ __forceinline__ T* bin_block_order(T* a, T* b, uint32_t n, uint32_t bits, uint32_t* cnt,
                                               BinSortSmem& sm) {
@@ -763,7 +769,7 @@ __device__ __forceinline__ T* bin_block_order(T* a, T* b, uint32_t n, uint32_t b
   for (uint32_t i = 0; i < PER / 4; ++i) {
     reinterpret_cast<uint4*>(cnt)[tid + kBinThreads * i] = make_uint4(0, 0, 0, 0);
   }
-  if (tid == 0) sm.nbig = 0;
+  if (tid == 0) sm.nbig = sm.work = 0;
   __syncthreads();
   T k[IT];
   uint32_t r[IT];
@@ -787,7 +793,7 @@ __device__ __forceinline__ T* bin_block_order(T* a, T* b, uint32_t n, uint32_t b
     c[i + 2] = q.z;
     c[i + 3] = q.w;
   }
-  bool wide = false;
+  uint32_t work = 0;  // comparisons in the buckets that no bitmap takes
 #pragma unroll
   for (uint32_t i = 0; i < PER; ++i) {
     sum += c[i];
@@ -795,11 +801,14 @@ __device__ __forceinline__ T* bin_block_order(T* a, T* b, uint32_t n, uint32_t b
       if (sh <= kBinBucketBits) {
         sm.big[atomicAdd(&sm.nbig, 1u)] = (uint16_t)(tid * PER + i);
       } else {
-        wide = wide || c[i] > 8 * kBinBucketMax;
+        work += c[i] * c[i];
       }
     }
   }
-  if (__syncthreads_or(wide)) {
+  work = __reduce_add_sync(full, work);
+  if (lane == 0 && work) atomicAdd(&sm.work, work);
+  __syncthreads();
+  if (sm.work > kBinWork * n) {
     return bin_block_sort<T>(a, b, n, bits, reinterpret_cast<uint16_t (*)[256]>(cnt), sm);
   }
   uint32_t run = block_scan_th<kBinThreads>(sum, all, sm.scan);

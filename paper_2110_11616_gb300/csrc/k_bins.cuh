@@ -27,7 +27,9 @@
 // columns, so a job's first key always opens a voxel and a column, and a slab
 // unless the job goes on with a slab of its bin.  A bin of more than kBinSplitMax
 // keys, or a row of a split (12 more bits) of more than kBinRowMax, marks its
-// segment, which k_lsd_all then sorts the general way.
+// segment, which k_lsd_all then sorts the general way.  (By the first rule before any
+// job is made: the kernels after k_bin_scan then leave the segment alone.  By the
+// second in k_bin_sort, where the segment's keys and jobs are all written.)
 //
 // Measured on GB300 (us): 15M surface points at b = 12: sort 187, partition 120,
 // write 60, histogram 44, split 18, scan 11; the build 954 -> 475.  The job sort is
@@ -272,6 +274,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
   const uint32_t rem = 3 * sg.bits - sg.bin_bits;
   const uint32_t span_bits = min(8 * (uint32_t)sizeof(T) - rem, kBinMaxBits);
   uint32_t nsub[PER], nj = 0, open = 0;
+  bool over = false;
 #pragma unroll
   for (uint32_t i = 0; i < PER; ++i) {
     const uint32_t b = tid * PER + i;
@@ -284,13 +287,22 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
         (b & ((1u << span_bits) - 1u)) == 0u) {
       nsub[i] = 1;
       if (n > kBinSplitMax) {
-        sg.fallback = 1;
+        over = true;
       } else if (n > bin_cap<T>()) {
         nsub[i] = split_slots(n, target);
       }
       nj += nsub[i];
       open |= 1u << i;
     }
+  }
+  if (__syncthreads_or(over)) {
+    // a marked segment has no jobs: its points are not partitioned and its larger bins
+    // not split, so there are no keys, and no split's jobs, for k_bin_sort to read
+    if (tid == 0) {
+      sg.fallback = 1;
+      njobs[blockIdx.x] = 0;
+    }
+    return;
   }
   uint32_t j = block_scan_th<1024>(nj, tot, s_scan);
   const uint32_t all = min(tot, sg.job_cap);

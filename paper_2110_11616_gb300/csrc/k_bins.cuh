@@ -1309,11 +1309,14 @@ __global__ void __launch_bounds__(kThreads) k_bin_write(const SortSeg* __restric
 // bisection of all of them took the kernel from 270 to 526 us, bound by shared-memory
 // loads).  The channels' sums have 16 bits each, two to a word, which the count bounds
 // (257 * 255 < 2^16); a job with a voxel of more points sums its channels again, two
-// at a time in 32 bits.  A point needs no search of the CGA and no atomic in global
+// at a time in 32 bits.  Up to kBinPacked points the count is the upper half of the
+// third channel's word, which no voxel's points can then run over.  A point needs no search of the CGA and no atomic in global
 // memory: 15M rows of 3 channels that way took 1010 us for the sums alone.
 template <typename T>
 constexpr uint32_t bin_values_cap() { return sizeof(T) == 4 ? 6144 : 4096; }  // keys at a time
 constexpr uint32_t kBinDirBits = 12;
+// the most points n with n counts and n sums of 255 in a word: n * (2^16 + 255) < 2^32
+constexpr uint32_t kBinPacked = 0xffffffffu / (65536u + 255u);
 template <typename T>
 constexpr size_t bin_values_smem() {
   return (sizeof(T) + 12) * (size_t)bin_values_cap<T>() + (sizeof(uint32_t) << kBinDirBits);
@@ -1347,8 +1350,8 @@ __global__ void __launch_bounds__(kBinThreads, 2)
     const T* key = seg_keys(split ? keys0 : keys1, sg, stride) + q.x;
     const uint32_t* row = (split ? rows1 : rows0) + job.z;
     const uint32_t N = job.w;
-    // the count takes the place of a fourth channel where its 16 bits hold it
-    const bool packed = C <= 3 && N < 65536;
+    // the count takes the place of a fourth channel where the word holds it
+    const bool packed = C <= 3 && N <= kBinPacked;
     for (uint32_t u0 = 0; u0 < q.y; u0 += CAP) {
       const uint32_t n = min(CAP, q.y - u0);
       const T lo = __ldg(key + u0);
@@ -1412,7 +1415,8 @@ __global__ void __launch_bounds__(kBinThreads, 2)
       }
       __syncthreads();
       if (!first) {
-        // a sum that runs over carries into the count, which is then more than 257 too
+        // a sum runs over only where the count is more than 257, and a packed one then
+        // adds its carries to the count, which stays below 2^16 (kBinPacked)
         for (uint32_t e = tid; e < n; e += kBinThreads) {
           if (packed) s_num[e] = s_sum2[e] >> 16;
           many |= s_num[e] > 257u;

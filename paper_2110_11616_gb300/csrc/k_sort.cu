@@ -587,8 +587,6 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
     bins += nb + 1;
     slots += g.job_cap;
     ptiles += (g.n_host + 1024ull * B.items - 1) / (1024ull * B.items);
-    // the general sort behind the bins has 8-bit digits
-    g.passes = radix_passes(g.key_bits, 8);
   }
   const size_t room = (size_t)kMaxPasses * total_tiles * ((size_t)4 << sc.radix_bits);
   char* p = reinterpret_cast<char*>(sc.look);
@@ -605,7 +603,11 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
   B.jobs = reinterpret_cast<uint4*>(take(slots * 16));
   B.info = reinterpret_cast<uint4*>(take(slots * 16));
   B.njobs = reinterpret_cast<uint32_t*>(take((size_t)S * 4));
+  // (empty clouds take room here but none in the look-back words: a batch of many goes
+  // the general way, with the digits and passes that the caller planned)
   if ((size_t)(p - reinterpret_cast<char*>(sc.look)) > room || slots > 0x7fffffffull) return;
+  // the general sort behind the bins has 8-bit digits
+  for (int s = 0; s < S; ++s) h_segs[s].passes = radix_passes(h_segs[s].key_bits, 8);
   B.ptiles = (uint32_t)ptiles;
   B.slots = (uint32_t)slots;
   B.on = true;

@@ -16,8 +16,9 @@ constexpr int kRadixBits = 8;  // default digit width (and the NN query sort's)
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kRadixMaxBits = 9;
 constexpr int kMaxPasses = 6;  // 3 * 16 bits / 8 (or / 9)
-constexpr int kCounterWords = 16;  // a tile counter per pass, the compaction's, the
-                                   // jobs' and the grid barrier's
+constexpr int kCounterWords = 16;  // a tile counter per pass, the compaction's, the jobs',
+                                   // the turns and the items done of the general sort
+                                   // behind the bins
 
 // Launch shape of the sort and merge kernels, chosen per (grid bits, size
 // bucket) by measurement (cga_autotune) and held in a process-wide table.

@@ -59,6 +59,41 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uns
   return __syncthreads_and(ok);
 }
 
+// Work in phases inside one ordinary launch.  Items are handed out in order by an atomic
+// counter, phase by phase, and an item starts once every item of the earlier phases is
+// counted done: those were all taken by blocks that run already, so any number of
+// resident blocks gets through, whatever else holds places on the GPU.  (A grid barrier
+// needs every block resident at once: a build with one waited for the kernels of all
+// other streams to leave.)
+//
+// Waits until *done is at least target; bounded like the look-back.
+__device__ __forceinline__ bool wait_done(const uint32_t* done, uint32_t target,
+                                          unsigned int* err) {
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    const unsigned long long t0 = global_ns();
+    uint32_t spins = 0, seen;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(done) : "memory");
+      if (seen >= target) break;
+      if ((++spins & 255u) == 0 && global_ns() - t0 > kWaitLimitNs) {
+        atomicOr(err, kErrTimeout);
+        ok = false;
+        break;
+      }
+    }
+  }
+  return __syncthreads_and(ok);
+}
+// Counts the block's item done, everything that its threads wrote visible first.
+__device__ __forceinline__ void count_done(uint32_t* done) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(done, 1u);
+  }
+}
+
 // Decoupled look-back over the tiles (first, tile) of one segment.  Each
 // tile publishes one 32-bit word per counter: 2 flag bits + a 30-bit value.
 // Tile ids are handed out in launch order by an atomic counter, so every

@@ -343,58 +343,69 @@ __global__ void __launch_bounds__(kThreads) k_compact(const SortSeg* __restrict_
   compact_sorted_tile<K, LEVELS>(sg, s_tile, (sg.passes & 1u) ? keys1 : keys0, clook, sm);
 }
 
-// The general sort of the segments that a build by bins marked (usually none:
-// the blocks look and leave): key generation, the 8-bit radix passes and the
-// compaction in one cooperative launch, a grid barrier between the steps.  The
-// tables of the bins lie in the look-back words, so those are cleared here.
-constexpr int kLsdBarrier = kMaxPasses + 2;  // its word of the counters
+// The general sort of the segments that a build by bins marked (usually none: the
+// blocks look and leave): clearing of the tables, key generation, the 8-bit radix passes
+// and the compaction in one launch, as phases of items (wait_done).  The tables of the
+// bins lie in the look-back words, so those are cleared here.
+constexpr int kLsdTurn = kMaxPasses + 2, kLsdDone = kMaxPasses + 4;  // words of the counters
+static_assert(kLsdDone < kCounterWords, "counters");
+constexpr uint32_t kLsdZero = 16384;  // words cleared by an item
 template <typename K>
 __global__ void __launch_bounds__(kThreads, 4)
     k_lsd_all(SortSeg* segs, int S, uint32_t total_tiles, uint32_t max_passes, K* keys0, K* keys1,
               uint32_t* hist, uint32_t* look, uint32_t* clook, uint32_t* counters,
               uint32_t zero_words) {
   __shared__ CompactSmem sm;
-  __shared__ uint32_t s_tile;
+  __shared__ uint32_t s_item;
   __shared__ int s_seg;
-  const int tid = threadIdx.x;
+  const uint32_t tid = threadIdx.x;
   int any = 0;
-  for (int s = tid; s < S; s += kThreads) any |= (int)segs[s].fallback;
+  for (int s = (int)tid; s < S; s += kThreads) any |= (int)segs[s].fallback;
   if (!__syncthreads_or(any)) return;
   unsigned int* err = &segs[0].out.hdr->err;
-  uint32_t round = 0;
-  // hist, look and clook lie side by side, up to the counters
-  for (uint32_t i = blockIdx.x * kThreads + tid; i < zero_words; i += gridDim.x * kThreads) {
-    hist[i] = 0;
-  }
-  if (blockIdx.x == 0 && tid <= kMaxPasses) counters[tid] = 0;
-  if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
-  const uint32_t per = (total_tiles + gridDim.x - 1) / gridDim.x, t0 = blockIdx.x * per;
-  keys_hist_tiles<K, 8>(segs, S, t0, min(t0 + per, total_tiles), keys0, hist, true);
-  if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
-  for (uint32_t p = 0; p <= max_passes; ++p) {
-    // pass p, and after the last one the compaction
-    const uint32_t c = p < max_passes ? p : (uint32_t)kMaxPasses;
-    for (;;) {
+  // items: hist, look and clook, which lie side by side, in runs of words; keys, a share of
+  // the tiles each; a tile each for every pass and for the compaction
+  const uint32_t nz = (zero_words + kLsdZero - 1) / kLsdZero;
+  const uint32_t nk = min(gridDim.x, total_tiles), per = (total_tiles + nk - 1) / nk;
+  uint32_t open = 0;  // the last phase known to have begun
+  for (;;) {
+    __syncthreads();  // the previous item's shared data is read no more
+    if (tid == 0) s_item = atomicAdd(counters + kLsdTurn, 1u);
+    __syncthreads();
+    uint32_t i = s_item, before = 0, phase = 0;
+    if (i >= nz + nk) {
+      const uint32_t q = (i - nz - nk) / total_tiles;
+      if (q > max_passes) return;
+      phase = 2 + q;
+      before = nz + nk + q * total_tiles;
+    } else if (i >= nz) {
+      phase = 1;
+      before = nz;
+    }
+    i -= before;
+    if (phase > open) {
+      if (!wait_done(counters + kLsdDone, before, err)) return;
+      open = phase;
+    }
+    if (phase == 0) {
+      const uint32_t w1 = min(zero_words, (i + 1) * kLsdZero);
+      for (uint32_t w = i * kLsdZero + tid; w < w1; w += kThreads) hist[w] = 0;
+    } else if (phase == 1) {
+      keys_hist_tiles<K, 8>(segs, S, i * per, min((i + 1) * per, total_tiles), keys0, hist, true);
+    } else {
+      const uint32_t p = phase - 2;  // pass p, and after the last one the compaction
+      if (tid == 0) s_seg = find_seg(segs, S, i);
       __syncthreads();
-      if (tid == 0) {
-        const uint32_t t = atomicAdd(counters + c, 1u);
-        s_tile = t;
-        s_seg = t < total_tiles ? find_seg(segs, S, t) : 0;
-      }
-      __syncthreads();
-      const uint32_t t = s_tile;
-      if (t >= total_tiles) break;
       const SortSeg& sg = segs[s_seg];
-      if (!sg.fallback) continue;
-      if (p < max_passes) {
-        onesweep_tile<K, kThreads, 8>(segs, s_seg, t, (int)p, (p & 1) ? keys1 : keys0,
+      if (sg.fallback && p < max_passes) {
+        onesweep_tile<K, kThreads, 8>(segs, s_seg, i, (int)p, (p & 1) ? keys1 : keys0,
                                       (p & 1) ? keys0 : keys1, hist,
                                       look + ((size_t)p * total_tiles << 8));
-      } else {
-        compact_sorted_tile<K, 3>(sg, t, (sg.passes & 1u) ? keys1 : keys0, clook, sm);
+      } else if (sg.fallback) {
+        compact_sorted_tile<K, 3>(sg, i, (sg.passes & 1u) ? keys1 : keys0, clook, sm);
       }
     }
-    if (!grid_barrier(counters + kLsdBarrier, ++round * gridDim.x, err)) return;
+    count_done(counters + kLsdDone);
   }
 }
 
@@ -674,16 +685,12 @@ static void launch_bin_write(int S, const SortScratch& sc, uint32_t stride, cuda
 template <typename K>
 static cudaError_t launch_lsd_all(int S, uint32_t total_tiles, const SortScratch& sc,
                                   cudaStream_t stream) {
-  SortSeg* segs = sc.segs;
-  K *k0 = static_cast<K*>(sc.keys0), *k1 = static_cast<K*>(sc.keys1);
-  uint32_t passes = kMaxPasses, *hist = sc.hist, *look = sc.look, *clook = sc.clook,
-           *counters = sc.counters;
-  uint32_t words = (uint32_t)((reinterpret_cast<char*>(sc.counters) -
-                               reinterpret_cast<char*>(sc.hist)) / 4);
-  void* args[] = {&segs, &S, &total_tiles, &passes, &k0, &k1, &hist, &look, &clook, &counters, &words};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_lsd_all<K>),
-                                     dim3(g_lsd_blocks[sizeof(K) / 8]), dim3(kThreads), args,
-                                     onesweep_smem<K, kThreads, 8>(), stream);
+  const uint32_t words = (uint32_t)((reinterpret_cast<char*>(sc.counters) -
+                                     reinterpret_cast<char*>(sc.hist)) / 4);
+  k_lsd_all<K><<<g_lsd_blocks[sizeof(K) / 8], kThreads, onesweep_smem<K, kThreads, 8>(), stream>>>(
+      sc.segs, S, total_tiles, kMaxPasses, static_cast<K*>(sc.keys0), static_cast<K*>(sc.keys1),
+      sc.hist, sc.look, sc.clook, sc.counters, words);
+  return cudaGetLastError();
 }
 
 // The build by bins (the plan is laid out, the segment table uploaded).

@@ -35,30 +35,6 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Grid barrier: block arrivals counted up to `target`.  All blocks are resident
-// (cooperative launch); the wait is bounded all the same, and a block that gives
-// up records the error and leaves.
-__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, unsigned int* err) {
-  __syncthreads();
-  bool ok = true;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(bar, 1u);
-    const unsigned long long t0 = global_ns();
-    uint32_t spins = 0, seen;
-    for (;;) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-      if (seen >= target) break;
-      if ((++spins & 255u) == 0 && global_ns() - t0 > kWaitLimitNs) {
-        atomicOr(err, kErrTimeout);
-        ok = false;
-        break;
-      }
-    }
-  }
-  return __syncthreads_and(ok);
-}
-
 // Work in phases inside one ordinary launch.  Items are handed out in order by an atomic
 // counter, phase by phase, and an item starts once every item of the earlier phases is
 // counted done: those were all taken by blocks that run already, so any number of

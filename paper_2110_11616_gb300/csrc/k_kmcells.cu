@@ -14,7 +14,7 @@
 //   k_kc_scan     cell offsets; cells split into chunks of at most kKcChunk voxels
 //   k_kc_scatter  the voxels in cell order, 32 bits each (offsets in the cell)
 //   k_kc_stats    box and coordinate sums of every chunk; the box of the cloud
-//   k_kc_loop     all passes in one cooperative launch, one grid barrier a pass
+//   k_kc_loop     all passes in one launch, a pass starting when the one before is done
 //   k_kc_labels   labels in CGA order from the cells' remaining centres
 //
 // The chunk bound keeps the work even when a cell holds most of the cloud, and
@@ -24,9 +24,13 @@
 //
 // Measured (GB300, two frames of 19.9M voxels, b = 12, 47 and 44 passes, both
 // together): 24.0 ms voxel by voxel (0.25 ms a pass and 8 us for its centres),
-// 3.0 ms here: the loop 2.24 ms (24 us a pass: the latency of the mixed chunks'
-// loads and the barrier), scatter 0.27, count 0.16, labels 0.13, stats 0.11,
-// scan 0.05.  Chunks of 1024 voxels with all remaining centres measured per
+// 3.0 ms here when a grid barrier ended each pass and the blocks' sums lay block by
+// block: scatter 0.27, count 0.16, labels 0.13, stats 0.11, scan 0.05, the rest the loop
+// (24 us a pass: the latency of the mixed chunks' loads and the barrier).  The passes in
+// parts, sums word by word: 20M voxels, b = 12, 37 passes 1160 -> 1000 us, b = 10, 64
+// passes 1257 -> 945, 1M voxels, 27 passes 562 -> 401.  (With the sums block by block the
+// parts took 2% more than the barrier: each block reads 32 words of every block, a
+// sector each.)  Chunks of 1024 voxels with all remaining centres measured per
 // voxel took 4.6 ms in the loop: too few mixed chunks to share among 4864 warps.
 // The voxel-by-voxel form stays for allocators without room for the cells.
 #include <algorithm>
@@ -45,13 +49,16 @@ constexpr int kKcLoopThreads = 1024;
 constexpr int kKcPerSm = 6;
 constexpr uint32_t kKcNone = 0xFEu;      // chunk state before the first pass
 constexpr uint32_t kKcMixed = 0xFFu;     // labels kept voxel by voxel
-constexpr uint32_t kKcWords = kKmClusters * 4 + 1;  // sums and the changed flag
+constexpr uint32_t kKcWords = kKmClusters * 4;  // a block's sums, a warp each
+constexpr uint32_t kKcChangedBit = 48;          // of the first count: a label changed
 
 struct KcState {
   uint32_t box[6];   // least y, z (box[1..2]), greatest y, z (box[4..5])
   uint32_t nchunks;
-  uint32_t bar;      // arrivals at the grid barrier
-  int used[kKmClusters * 3];  // centres of the last pass's labels
+  uint32_t turn;     // parts of passes handed out
+  uint32_t done;     // and done
+  int centre[2][kKmClusters * 3];  // centres of the even and the odd passes' labels
+  int used[kKmClusters * 3];       // of the last one's
 };
 
 // Cell grid: 2^cb cells of 2^shift voxels per axis.
@@ -68,7 +75,7 @@ struct KcView {
   uint8_t* state;     // chunk: label of all its voxels, kKcMixed or kKcNone
   uint32_t* vox;      // voxels in cell order: x | y << 9 | z << 18 in the cell
   uint8_t* vlab;      // their labels while the chunk is mixed
-  unsigned long long* part;  // [2][blocks][kKcWords]
+  unsigned long long* part;  // [2][kKcWords][blocks]
   KcGrid grid;
   uint32_t ncells, max_chunks;
 };
@@ -101,7 +108,8 @@ __global__ void k_kc_init(KcState* st) {
   }
   if (t == 0) {
     st->nchunks = 0;
-    st->bar = 0;
+    st->turn = 0;
+    st->done = 0;
   }
 }
 
@@ -327,14 +335,21 @@ __device__ __forceinline__ uint32_t box_centres(const int* c, const long long* q
   return mask;
 }
 
+// A pass is as many parts as the launch has blocks; its chunks are dealt out over them.
+// A block takes a part of a pass, in order, once the pass before is done (wait_done: any
+// number of resident blocks gets through).  Every part then sums the pass before for
+// itself, and moves that pass's centres.  The part of the pass after the last one leaves
+// the results: as many as there are blocks, so each block ends with one.
 __global__ void __launch_bounds__(kKcLoopThreads, 1)
     k_kc_loop(Levels a, KcView v, uint32_t max_iter, long long* centres,
               unsigned long long* counts, uint32_t* iters) {
   constexpr uint32_t W = kKcLoopThreads / 32;
+  static_assert(W == kKcWords, "a warp per word of the sums");
   __shared__ int s_c[kKmClusters * 3];
   __shared__ long long s_q[kKmClusters];
   __shared__ unsigned long long s_part[W][kKmClusters * 4 + 1];
-  __shared__ unsigned long long s_tot[kKcWords];
+  __shared__ unsigned long long s_tot[kKcWords + 1];  // the sums; parts with a change
+  __shared__ uint32_t s_item, s_next;
   const uint32_t full = 0xffffffffu, tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
   const uint32_t u = (uint32_t)a.hdr->cnt[0], h = (uint32_t)a.hdr->cnt[2];
   if (u == 0) {
@@ -346,16 +361,44 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
     return;
   }
   const uint32_t nch = v.st->nchunks, cb = v.grid.cb, sh = v.grid.shift, cm = (1u << cb) - 1u;
-  const uint32_t warps = gridDim.x * W, gw = blockIdx.x * W + w;
-  // corner c of the box: the greatest coordinate of axis ax where bit ax of c is set
-  if (tid < kKmClusters * 3) {
-    const uint32_t c = tid / 3, ax = tid % 3;
-    const uint32_t lo = ax == 0 ? (uint32_t)__ldg(a.idx2) : v.st->box[ax];
-    const uint32_t hi = ax == 0 ? (uint32_t)__ldg(a.idx2 + h - 1) : v.st->box[3 + ax];
-    s_c[tid] = (int)(256u * (((c >> ax) & 1u) ? hi : lo));
-  }
-  uint32_t pass = 0;
+  const uint32_t parts = gridDim.x, warps = parts * W;
+  if (tid == 0) s_item = atomicAdd(&v.st->turn, 1u);
   for (;;) {
+    __syncthreads();
+    const uint32_t pass = s_item / parts, part = s_item % parts;  // passes before this one
+    const uint32_t gw = part * W + w;
+    bool converged = false;
+    if (pass == 0) {
+      // corner c of the box: the greatest coordinate of axis ax where bit ax of c is set
+      if (tid < kKmClusters * 3) {
+        const uint32_t c = tid / 3, ax = tid % 3;
+        const uint32_t lo = ax == 0 ? (uint32_t)__ldg(a.idx2) : v.st->box[ax];
+        const uint32_t hi = ax == 0 ? (uint32_t)__ldg(a.idx2 + h - 1) : v.st->box[3 + ax];
+        s_c[tid] = (int)(256u * (((c >> ax) & 1u) ? hi : lo));
+      }
+    } else {
+      if (!wait_done(&v.st->done, pass * parts, &a.hdr->err)) return;
+      const uint32_t odd = (pass - 1) & 1u;
+      const unsigned long long* sums = v.part + (size_t)odd * parts * kKcWords;
+      if (tid < kKmClusters * 3) s_c[tid] = __ldcg(&v.st->centre[odd][tid]);
+      {
+        unsigned long long s = 0;
+        for (uint32_t b = lane; b < parts; b += 32) s += __ldcg(sums + w * parts + b);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
+        if (lane == 0) {
+          s_tot[w] = s & ((1ull << kKcChangedBit) - 1);
+          if (w == 3) s_tot[kKcWords] = s >> kKcChangedBit;
+        }
+      }
+      __syncthreads();
+      converged = pass > 1 && s_tot[kKcWords] == 0;
+    }
+    const bool stop = pass > 0 && (converged || pass >= max_iter);
+    if (pass > 0 && !stop && tid < kKmClusters * 3) {
+      const unsigned long long n = s_tot[4 * (tid / 3) + 3];
+      if (n > 0) s_c[tid] = (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
+    }
     __syncthreads();
     if (tid < kKmClusters) {
       long long q = 0;
@@ -363,6 +406,35 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
       s_q[tid] = q;
     }
     __syncthreads();
+    if (stop) {
+      if (part == 0) {
+        if (tid < kKmClusters * 3) {
+          const int c = s_c[tid];
+          const unsigned long long n = s_tot[4 * (tid / 3) + 3];
+          v.st->used[tid] = c;
+          centres[tid] = converged || n == 0
+                             ? c : (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
+        }
+        if (tid < kKmClusters) counts[tid] = s_tot[4 * tid + 3];
+        if (tid == 0) *iters = pass;
+      }
+      // the cells' remaining centres, for the labels in CGA order
+      for (uint32_t j = gw * 32u + lane; j < nch; j += 32u * warps) {
+        const uint4 A = __ldg(v.recA + j);
+        const uint32_t id = __ldg(&v.recB[j].w);
+        const int o[3] = {(int)((id >> (2 * cb)) << sh), (int)(((id >> cb) & cm) << sh),
+                          (int)((id & cm) << sh)};
+        int lo[3], hi[3];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+          lo[ax] = o[ax] + (int)((A.z >> (9 * ax)) & 511u);
+          hi[ax] = o[ax] + (int)((A.w >> (9 * ax)) & 511u);
+        }
+        atomicOr(v.cell + id, box_centres(s_c, s_q, lo, hi));
+      }
+      return;
+    }
+    if (part == 0 && tid < kKmClusters * 3) v.st->centre[pass & 1u][tid] = s_c[tid];
     unsigned long long acc = 0;  // lane l: entry l = label * 4 + {x, y, z sum, count}
     bool changed = false;
     // chunk i of a round goes to lane i / warps of warp i % warps: the mixed
@@ -513,61 +585,22 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
         }
       }
     }
+    // (the next part, asked for while the block's last warps work)
+    if (tid == 0) s_next = atomicAdd(&v.st->turn, 1u);
     // block sums: entry e of every warp, then one word per entry and block
     s_part[w][lane] = acc;
     const bool any = __syncthreads_or(changed);
-    unsigned long long* part = v.part + (size_t)(pass & 1u) * gridDim.x * kKcWords;
     {
+      const uint32_t item = *(volatile uint32_t*)&s_item;  // (not kept over the pass)
+      unsigned long long* sums =
+          v.part + (size_t)(item / parts & 1u) * parts * kKcWords + item % parts;
       unsigned long long s = lane < W ? s_part[lane][w] : 0ull;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
-      if (lane == 0) part[(size_t)blockIdx.x * kKcWords + w] = s;
-      if (tid == 0) part[(size_t)blockIdx.x * kKcWords + kKmClusters * 4] = any ? 1ull : 0ull;
+      if (lane == 0) sums[w * parts] = s | (w == 3 && any ? 1ull << kKcChangedBit : 0ull);
     }
-    ++pass;
-    if (!grid_barrier(&v.st->bar, pass * gridDim.x, &a.hdr->err)) return;
-    // every block sums the blocks' words for itself
-    for (uint32_t e = w; e < kKcWords; e += W) {
-      unsigned long long s = 0;
-      for (uint32_t b = lane; b < gridDim.x; b += 32) s += __ldcg(part + (size_t)b * kKcWords + e);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
-      if (lane == 0) s_tot[e] = s;
-    }
-    __syncthreads();
-    const bool converged = pass > 1 && s_tot[kKmClusters * 4] == 0;
-    const bool stop = converged || pass >= max_iter;
-    if (stop && blockIdx.x == 0) {
-      if (tid < kKmClusters * 3) v.st->used[tid] = s_c[tid];
-      if (tid < kKmClusters) counts[tid] = s_tot[4 * tid + 3];
-      if (tid == 0) *iters = pass;
-    }
-    if (stop) {
-      // the cells' remaining centres, for the labels in CGA order
-      for (uint32_t j = gw * 32u + lane; j < nch; j += 32u * warps) {
-        const uint4 A = __ldg(v.recA + j);
-        const uint32_t id = __ldg(&v.recB[j].w);
-        const int o[3] = {(int)((id >> (2 * cb)) << sh), (int)(((id >> cb) & cm) << sh),
-                          (int)((id & cm) << sh)};
-        int lo[3], hi[3];
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-          lo[ax] = o[ax] + (int)((A.z >> (9 * ax)) & 511u);
-          hi[ax] = o[ax] + (int)((A.w >> (9 * ax)) & 511u);
-        }
-        atomicOr(v.cell + id, box_centres(s_c, s_q, lo, hi));
-      }
-    }
-    __syncthreads();
-    if (!converged && tid < kKmClusters * 3) {
-      const unsigned long long n = s_tot[4 * (tid / 3) + 3];
-      if (n > 0) s_c[tid] = (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
-    }
-    if (stop) {
-      __syncthreads();
-      if (blockIdx.x == 0 && tid < kKmClusters * 3) centres[tid] = s_c[tid];
-      return;
-    }
+    count_done(&v.st->done);
+    if (tid == 0) s_item = s_next;
   }
 }
 
@@ -596,21 +629,18 @@ __global__ void __launch_bounds__(kThreads, kKcPerSm)
   });
 }
 
-// Blocks of the loop kernel: one per SM that can hold one (0: no cooperative
-// launch here).
+// Blocks of the loop kernel: one per SM that can hold one (0: none can).
 uint32_t loop_blocks() {
   static std::atomic<int> cache{-1};
   int n = cache.load(std::memory_order_relaxed);
   if (n < 0) {
-    int dev = 0, coop = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_kc_loop, kKcLoopThreads, 0) !=
         cudaSuccess) {
       cudaGetLastError();
       occ = 0;
     }
-    n = coop && occ > 0 ? device_sm_count() : 0;
+    n = occ > 0 ? device_sm_count() : 0;
     cache.store(n, std::memory_order_relaxed);
   }
   return (uint32_t)n;
@@ -666,11 +696,7 @@ cudaError_t run_kmeans_cells(const Levels& a, uint32_t max_iter, void* scratch, 
   const unsigned sb = (unsigned)std::min<uint64_t>(((uint64_t)v.max_chunks + 7) / 8,
                                                    (uint64_t)device_sm_count() * 8);
   k_kc_stats<<<sb, kThreads, 0, stream>>>(v);
-  Levels av = a;
-  void* args[] = {&av, &v, &max_iter, &centres, &counts, &iters};
-  e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_kc_loop), dim3(loop_blocks()),
-                                  dim3(kKcLoopThreads), args, 0, stream);
-  if (e != cudaSuccess) return e;
+  k_kc_loop<<<loop_blocks(), kKcLoopThreads, 0, stream>>>(a, v, max_iter, centres, counts, iters);
   k_kc_labels<<<walk_blocks(a.cap, kKcPerSm), kThreads, 0, stream>>>(a, v, labels);
   count_launch(7);
   return cudaGetLastError();

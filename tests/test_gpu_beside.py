@@ -51,3 +51,12 @@ def test_build_that_the_general_sort_takes_over():
     pts = torch.from_numpy(v).cuda()
     torch.cuda.synchronize()
     assert _ends_beside(lambda: cga.cga_build(pts, g))
+
+
+@pytest.mark.parametrize("n,bits", [(60_000, 12), (2_000_000, 12)])
+def test_kmeans(n, bits):
+    pts = torch.from_numpy(synth.uniform_cube(n, seed=bits)).cuda()
+    a = cga.cga_build(pts, cga.grid_from_box([0, 0, 0], 1.0, bits))
+    u = a.info()["u"]
+    torch.cuda.synchronize()
+    assert _ends_beside(lambda: cga.cga_kmeans(a, 64, u=u))

@@ -757,9 +757,9 @@ int cga_kmeans(const cga_t* a, uint32_t max_iter, uint8_t* d_label, int64_t* d_c
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const cga_allocator* A = a->has_alloc ? &a->alloc : nullptr;
-  // by cells when the allocator has room for the voxels in cell order
-  // (5 bytes a voxel of capacity and the cell tables), else voxel by voxel
-  const size_t cells = libcga::kmeans_cells_bytes(a->grid.bits, a->lv.cap);
+  // by cells when the passes pay for them and the allocator has room for the voxels in
+  // cell order (5 bytes a voxel of capacity and the cell tables), else voxel by voxel
+  const size_t cells = libcga::kmeans_cells_bytes(a->grid.bits, a->lv.cap, max_iter);
   void* cs = cells > 0 ? dalloc(A, cells, s) : nullptr;
   if (cs != nullptr) {
     const int rc = cuda_rc(libcga::run_kmeans_cells(

@@ -310,8 +310,8 @@ cudaError_t run_kmeans(const Levels& a, uint32_t max_iter, KmState* st, uint8_t*
                        long long* centres, unsigned long long* counts, uint32_t* iters,
                        cudaStream_t stream);
 // The same by cells (k_kmcells.cu), in scratch of kmeans_cells_bytes (0: not
-// available, use run_kmeans).
-size_t kmeans_cells_bytes(uint32_t bits, uint64_t cap);
+// available or slower for so few passes, use run_kmeans).
+size_t kmeans_cells_bytes(uint32_t bits, uint64_t cap, uint32_t max_iter);
 cudaError_t run_kmeans_cells(const Levels& a, uint32_t max_iter, void* scratch, uint8_t* labels,
                              long long* centres, unsigned long long* counts, uint32_t* iters,
                              cudaStream_t stream);

@@ -32,7 +32,8 @@
 // parts took 2% more than the barrier: each block reads 32 words of every block, a
 // sector each.)  Chunks of 1024 voxels with all remaining centres measured per
 // voxel took 4.6 ms in the loop: too few mixed chunks to share among 4864 warps.
-// The voxel-by-voxel form stays for allocators without room for the cells.
+// The voxel-by-voxel form stays for runs of few passes (cells_pay) and for allocators
+// without room for the cells.
 #include <algorithm>
 #include <atomic>
 
@@ -674,8 +675,23 @@ size_t kc_layout(uint32_t bits, uint64_t cap, char* base, KcView* out) {
 
 }  // namespace
 
-size_t kmeans_cells_bytes(uint32_t bits, uint64_t cap) {
-  if (cap == 0 || loop_blocks() == 0) return 0;
+// The cells pay once their tables have cost less than the passes save (of at most
+// max_iter passes; the voxel-by-voxel form queues a launch pair for each of those).  In
+// us, from runs of 1 to 16 passes over 100 to 20M surface voxels, b = 10, 12 and 16:
+// the tables about 35, 14 for each 2^20 cells and 10 for each 2^20 voxels more than what
+// the other form starts with; a pass saves 8 (launches), up to 16 more from 8192 voxels
+// on and 8 for each 2^20.  Voxel by voxel and by cells: 1000 voxels, b = 16, 1 pass 52
+// and 121, 6 passes 144 and 152, 8 passes 182 and 167; 10k, b = 10, 1 pass 63 and 71, 2
+// passes 93 and 84; 20M, b = 12, 1 pass 255 and 330, 2 passes 442 and 352.
+static bool cells_pay(const KcGrid& g, uint64_t cap, uint32_t max_iter) {
+  const double m = (double)cap / (1 << 20);
+  const double tables = 35.0 + 14.0 * (double)(1u << (3 * g.cb)) / (1 << 20) + 10.0 * m;
+  const double pass = 8.0 + 16.0 * (double)std::min<uint64_t>(cap, 8192) / 8192 + 8.0 * m;
+  return pass * max_iter > tables;
+}
+
+size_t kmeans_cells_bytes(uint32_t bits, uint64_t cap, uint32_t max_iter) {
+  if (cap == 0 || loop_blocks() == 0 || !cells_pay(kc_grid(bits, cap), cap, max_iter)) return 0;
   return kc_layout(bits, cap, nullptr, nullptr);
 }
 

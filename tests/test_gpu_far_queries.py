@@ -1,0 +1,58 @@
+"""Queries far outside the grid or far from every voxel of it: beyond 2^16 voxels the
+32-bit searches find nothing and 64-bit ones answer.  The oracle's answers, in a time
+like that of the same scene on a coarser grid, where all distances fit 32 bits."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+from paper_2110_11616_gb300 import cga, synth_gpu
+
+pytestmark = pytest.mark.gpu
+BOX = ([0.0, 0.0, 0.0], 100.0)
+
+
+def _far(m, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand((m, 3), generator=gen, device="cuda") * 300 - 100
+
+
+def _time(call):
+    call()
+    best = float("inf")
+    for _ in range(3):
+        t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+        torch.cuda.synchronize()
+        t0.record()
+        call()
+        t1.record()
+        torch.cuda.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+    return best
+
+
+def _worlds(n, prepare=True):
+    pts = synth_gpu.surface_cloud(n, 3, n_objects=6)
+    for bits in (13, 16):
+        a = cga.cga_build(pts, cga.grid_from_box(*BOX, bits))
+        if prepare:
+            cga.cga_nn_prepare(a)
+        yield bits, a, pts.cpu().numpy()
+
+
+def test_nearest_answers():
+    q = _far(2000, 1)
+    for bits, a, pts in _worlds(3000):
+        og = oracle.grid_from_box(*BOX, bits)
+        idx, d2 = cga.cga_nn_query(a, q)
+        oi, od = oracle.nn_brute(oracle.build(pts, og), og, q.cpu().numpy())
+        assert np.array_equal(d2.cpu().numpy().view(np.uint64), od)
+        assert np.array_equal(idx.cpu().numpy().view(np.uint32), oi)
+
+
+@pytest.mark.parametrize("n,m", [(1000, 10_000), (30_000, 10_000)])
+def test_nearest_time(n, m):
+    q = _far(m, 2)
+    t = {bits: _time(lambda: cga.cga_nn_query(a, q)) for bits, a, _ in _worlds(n)}
+    assert t[16] < 2.5 * t[13], t   # 1.7 with 64-bit distances throughout

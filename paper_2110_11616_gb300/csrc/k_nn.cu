@@ -1484,6 +1484,15 @@ struct LongQuery {
   Best32 best;
 };
 constexpr uint32_t kLongQueries = 32;
+// How many of a block's n long queries its warps share.  Beyond one a warp the rest goes a
+// warp each: 10k queries of which all are long, 11 a block, 370 us shared and 266 so (a
+// 1000-point LiDAR world, b = 13; 212 without long queries kept).  Up to there sharing is
+// better even where a warp each would do (7000 queries, b = 16: 147 and 170), since few
+// blocks have as many and the slowest one counts.
+__device__ __forceinline__ uint32_t shared_queries(uint32_t n) {
+  const uint32_t odd = n % 8u;
+  return n <= 8u ? n : (odd <= 4u ? odd : 0u);
+}
 constexpr uint32_t kFewRounds = 4;  // with up to 8 queries a block
 
 // NC: the most coarse levels any segment of the launch carries (0, 1 or 2).
@@ -1500,14 +1509,41 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
   constexpr uint32_t W = 256 / 32;
   __shared__ uint32_t s_next;
   __shared__ uint32_t s_nlong;
+  __shared__ bool s_again;  // (LONG) the second time around: long queries, a warp each
   __shared__ LongQuery s_long[LONG ? kLongQueries : 1];
-  if (LONG && threadIdx.x == 0) s_nlong = 0;
+  if (LONG && threadIdx.x == 0) {
+    s_nlong = 0;
+    s_again = false;
+  }
   open_slots<W>(&s_next);
   const bool sorted = order != nullptr && (order_err == nullptr || *order_err == 0u);
   for (uint32_t turn = threadIdx.x >> 5;; turn = next_turn(&s_next)) {
-    // (few queries: one a block before any has two)
-    const uint32_t slot = LONG && rounds <= kFewRounds ? blockIdx.x + turn * gridDim.x : slot_of_turn<W>(turn);
-    if (slot >= total_slots) break;
+    uint32_t slot, j, k0 = 0;
+    Best32 near{0xffffffffu, 0xffffffffu};
+    if (!LONG || !s_again) {
+      // (few queries: one a block before any has two)
+      slot = LONG && rounds <= kFewRounds ? blockIdx.x + turn * gridDim.x : slot_of_turn<W>(turn);
+      if (slot >= total_slots) {
+        if (!LONG) break;
+        // every warp is out of queries: more long ones than the block shares?
+        __syncthreads();
+        const uint32_t n = min(s_nlong, kLongQueries), shared = shared_queries(n);
+        if (n == shared) break;
+        if (threadIdx.x == 0) {
+          s_next = shared;
+          s_again = true;
+        }
+        __syncthreads();
+        continue;
+      }
+      j = 0;
+    } else {
+      if (turn >= min(s_nlong, kLongQueries)) break;
+      slot = s_long[turn].slot;
+      j = s_long[turn].j;
+      near = s_long[turn].best;
+      k0 = 16 * rounds;
+    }
     const uint32_t tile = slot / (uint32_t)kTile;
     const NnSeg& sg = segs != nullptr ? segs[find_nn_seg(segs, S, tile)] : inline_seg;
     if (sg.tree.levels > 0) continue;  // searched by k_nn_tree
@@ -1515,7 +1551,7 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
     if (local >= sg.m) continue;
     // queries, the order and the results stream through once: loaded and
     // stored evict-first, so that L2 keeps the CGA and the search structures
-    const uint32_t j = sorted ? (uint32_t)__ldcs(order + slot) : local;
+    if (!LONG || k0 == 0) j = sorted ? (uint32_t)__ldcs(order + slot) : local;
     if (j >= sg.m) continue;  // a caller-given order that is not a permutation
     const Levels& a = sg.a;
     const uint32_t u = (uint32_t)a.hdr->cnt[0], h = (uint32_t)a.hdr->cnt[2];
@@ -1542,20 +1578,21 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
         search_levels<1>(sg, Qry{qx, qy, qz, cqx, cqy, cqz}, lane, best);
       }
     } else {
-      Best32 near{0xffffffffu, 0xffffffffu};
-      bool done = search_fine32<1>(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, 0,
-                                   LONG ? rounds : 0xffffffffu, near);
-      if (LONG && !done) {
+#pragma unroll 1
+      while (!search_fine32<1>(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, k0,
+                               LONG && k0 == 0 ? rounds : 0xffffffffu, near)) {
+        // a long query: kept for later, or, the list full, searched to its end
         uint32_t at = 0;
         if (lane == 0) at = atomicAdd(&s_nlong, 1u);
         at = __shfl_sync(0xffffffffu, at, 0);
         if (at < kLongQueries) {
           if (lane == 0) s_long[at] = LongQuery{slot, j, near};
-          continue;
+          j = 0xffffffffu;
+          break;
         }
-        search_fine32<1>(a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, lane, 16 * rounds,
-                         0xffffffffu, near);
+        k0 = 16 * rounds;
       }
+      if (LONG && j == 0xffffffffu) continue;
       if (near.d2 != 0xffffffffu) {
         best.d2 = near.d2;
         best.idx = near.idx;
@@ -1570,8 +1607,8 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
   }
   if constexpr (LONG) {
     __syncthreads();
-    const uint32_t n = min(s_nlong, kLongQueries);
-    for (uint32_t i = 0; i < n; ++i) {
+    const uint32_t shared = shared_queries(min(s_nlong, kLongQueries));
+    for (uint32_t i = 0; i < shared; ++i) {
       const uint32_t slot = s_long[i].slot, j = s_long[i].j;
       const NnSeg& sg = segs != nullptr ? segs[find_nn_seg(segs, S, slot / (uint32_t)kTile)]
                                         : inline_seg;
@@ -1582,17 +1619,12 @@ __global__ void __launch_bounds__(256, NC > 0 ? CGA_NN_COARSE_BLOCKS : CGA_NN_FI
       const uint32_t cqy = (uint32_t)min(max(qy, 0), top);
       const uint32_t cqz = (uint32_t)min(max(qz, 0), top);
       const uint32_t h = (uint32_t)sg.a.hdr->cnt[2];
-      Best32 near = s_long[i].best;
+      Best32 near = s_long[i].best;  // (a query without one by now was searched in 64 bits)
       search_fine32<W>(sg.a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, threadIdx.x,
                        16 * rounds, 0xffffffffu, near);
-      Best best{near.d2, near.idx};
-      if (near.d2 == 0xffffffffu && threadIdx.x < 32) {
-        best = Best{~0ull, 0xffffffffu};
-        search_fine(sg.a, sg.xdir, sg.ctab, h, qx, qy, qz, cqx, cqy, cqz, threadIdx.x, best);
-      }
       if (threadIdx.x == 0) {
-        __stcs(sg.idx + j, best.idx);
-        __stcs(sg.d2 + j, best.d2);
+        __stcs(sg.idx + j, near.idx);
+        __stcs(sg.d2 + j, (unsigned long long)near.d2);
       }
     }
   }

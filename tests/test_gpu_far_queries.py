@@ -56,3 +56,26 @@ def test_nearest_time(n, m):
     q = _far(m, 2)
     t = {bits: _time(lambda: cga.cga_nn_query(a, q)) for bits, a, _ in _worlds(n)}
     assert t[16] < 2.5 * t[13], t   # 1.7 with 64-bit distances throughout
+
+
+@pytest.mark.parametrize("m", [1, 7, 300, 3000, 7000, 9000, 30_000])
+def test_blocks_with_any_number_of_long_queries(m):
+    """From none to all of the queries need more rounds than a warp gives them, so a
+    block's list of those is empty, shared, dealt out over its warps or overfull."""
+    rng = np.random.default_rng(m)
+    bits, world = 13, 2500
+    og = oracle.Grid(bits, 1.0, (0.0, 0.0, 0.0))
+    vox = rng.integers(0, 1 << bits, size=(world, 3))
+    a = cga.cga_build(torch.from_numpy((vox + 0.5).astype(np.float32)).cuda(),
+                      cga.make_grid(bits, 1.0, (0.0, 0.0, 0.0)))
+    cga.cga_nn_prepare(a)
+    o = oracle.build((vox + 0.5).astype(np.float32), og)
+    for part in (0.0, 0.01, 0.2, 1.0):   # of the queries far above the world
+        q = vox[rng.integers(0, world, size=m)] + rng.integers(-3, 4, size=(m, 3)) + 0.5
+        far = rng.random(m) < part
+        q[far] = rng.uniform(0, 1 << bits, size=(int(far.sum()), 3)) + [0, 0, 20_000]
+        q = q.astype(np.float32)
+        idx, d2 = cga.cga_nn_query(a, torch.from_numpy(q).cuda())
+        oi, od = oracle.nn_brute(o, og, q)
+        assert np.array_equal(d2.cpu().numpy().view(np.uint64), od), part
+        assert np.array_equal(idx.cpu().numpy().view(np.uint32), oi), part

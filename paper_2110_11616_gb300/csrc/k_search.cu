@@ -620,9 +620,13 @@ struct SmemList {
 // offering at most one candidate per lane, so that the candidates enter the
 // list together and the k-th distance prunes every walk; a lane whose column
 // runs out moves to its next column (and offers that column's nearest voxel)
-// in the same step.
+// in the same step.  The narrow form gives up (true) while its list still has room and a
+// quarter of the lanes have met what lies beyond its range: without a bound it would go
+// through every column within that range, probably for nothing (10k queries up to 65k
+// voxels outside a world of 30k surface voxels, b = 16, k = 8: 44.7 ms that way, 4.9 in 64
+// bits alone, 7.2 so).
 template <bool NARROW, typename L>
-__device__ __forceinline__ void knn_walk(const SearchSeg& sg, const RQuery& q, uint32_t h,
+__device__ __forceinline__ bool knn_walk(const SearchSeg& sg, const RQuery& q, uint32_t h,
                                          uint32_t lane, L& list) {
   using P = Pair<NARROW>;
   using D = typename P::D;
@@ -701,28 +705,38 @@ __device__ __forceinline__ void knn_walk(const SearchSeg& sg, const RQuery& q, u
         }
       }
       bound = list.offer(has, cd, ci, lane, bound);
+      if (NARROW && bound == P::kFar) {
+        // dropped with columns left, or out of a column with voxels left
+        const bool far = work ? !in_col && (zu < ze || zd > zs) : cr < ye || cl > ys;
+        if (__popc(__ballot_sync(0xffffffffu, far)) >= 8) return true;
+      }
     }
   }
+  return false;
 }
 
 // The narrow form answers every query; the wide form (a launch after it) the
-// queries that the narrow one left with fewer than min(k, u) neighbours.
+// queries that the narrow one left with fewer than min(k, u) neighbours, or, on its own,
+// all of them (alone).  chunk: queries that a warp of the wide form looks at together.
 template <bool LARGE, bool NARROW>
 __global__ void __launch_bounds__(LARGE ? kKnnLargeThreads : 256, LARGE ? 1 : CGA_KNN_BLOCKS)
     k_knn(SearchSeg sg, uint32_t k, uint32_t cap, const unsigned long long* __restrict__ order,
-          uint32_t* out_idx, unsigned long long* out_d2) {
+          uint32_t* out_idx, unsigned long long* out_d2, uint32_t chunk, bool alone) {
   extern __shared__ __align__(16) unsigned char s_knn[];
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t u = (uint32_t)sg.a.hdr->cnt[0], h = (uint32_t)sg.a.hdr->cnt[2];
   typename std::conditional<LARGE, SmemList<NARROW>, RegList<NARROW>>::type list;
-  auto answer = [&](uint32_t j) {
+  auto init = [&]() {
     if constexpr (LARGE) {
       list.init(k, cap, s_knn, threadIdx.x >> 5, blockDim.x >> 5);
     } else {
       list.init(k);
     }
+  };
+  auto answer = [&](uint32_t j) {
+    init();
     const RQuery q = radius_query(sg, j);
-    if (q.valid && u > 0) knn_walk<NARROW>(sg, q, h, lane, list);
+    if (q.valid && u > 0 && knn_walk<NARROW>(sg, q, h, lane, list)) init();
     list.finish(lane, (size_t)j * k, out_idx, out_d2);
   };
   if constexpr (NARROW) {
@@ -738,26 +752,31 @@ __global__ void __launch_bounds__(LARGE ? kKnnLargeThreads : 256, LARGE ? 1 : CG
     const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
     const uint32_t need = min(k, u);
-    if (need == 0) return;
-    for (uint32_t s0 = w * 32; s0 < sg.m; s0 += nw * 32) {
-      const uint32_t j = s0 + lane;
-      const bool open = j < sg.m && out_idx[(size_t)j * k + need - 1] == 0xffffffffu &&
-                        radius_query(sg, j).valid;
+    if (need == 0 && !alone) return;
+    for (uint32_t s0 = w * chunk; s0 < sg.m; s0 += nw * chunk) {
+      const bool in = lane < chunk && s0 + lane < sg.m;
+      const uint32_t j = in ? slot_query(order, s0 + lane) : 0u;
+      const bool open = in && (alone || (out_idx[(size_t)j * k + need - 1] == 0xffffffffu &&
+                                         radius_query(sg, j).valid));
       uint32_t todo = __ballot_sync(0xffffffffu, open);
       while (todo) {
-        answer(s0 + __ffs(todo) - 1);
+        answer(__shfl_sync(0xffffffffu, j, __ffs(todo) - 1));
         todo &= todo - 1;
       }
     }
   }
 }
 
-// One wave of resident blocks striding over the queries: a second, partial
-// wave would leave SMs idle at its end (1216 blocks on 760 places cost the
-// radius kernels a fifth of their time).
+// Blocks for m queries.  Up to four waves of them each warp takes one query; beyond,
+// four waves or 16 queries a warp on average, whichever are more blocks: within a block
+// the warps even their queries out (slot_of_turn), and blocks start where others end, so
+// that slow queries, which lie side by side in the order, do not all start late in the
+// same blocks.  8 nearest in LiDAR worlds, ms, in one wave and so: 100k queries of 1.3M
+// points, b = 16, 1.40 and 0.94 (one warp a query 1.32, 4 queries a warp 1.28), 1M 5.57 and
+// 5.52; 10k far from 300k points, b = 13, 18.2 and 12.9; the radius search is the same.
 unsigned search_blocks(uint64_t m, unsigned per_sm) {
-  return (unsigned)std::min<uint64_t>((std::max<uint64_t>(m, 1) + 7) / 8,
-                                      (uint64_t)device_sm_count() * per_sm);
+  const uint64_t all = (std::max<uint64_t>(m, 1) + 7) / 8, wave = (uint64_t)device_sm_count() * per_sm;
+  return (unsigned)std::min<uint64_t>(all, std::max<uint64_t>(4 * wave, all / 16));
 }
 
 }  // namespace
@@ -776,20 +795,32 @@ static cudaError_t knn_large_attr() {
                                     PairBuf<NARROW>::kBytes));
 }
 
+// The wide form alone answers calls of few queries (each has a warp of its own) whose
+// walks are short, of few neighbours or in few voxels: there the second launch costs more
+// than 32-bit arithmetic saves.  So it does of few queries on 16-bit grids, where all of
+// them may have to be answered twice (100 far from 300k surface voxels, k = 8: 34.6 ms by
+// both forms, 17.1 by the wide one).  us by both forms and by the wide one: a query of 50
+// voxels, k = 1 29 and 25, k = 16 31 and 27; of 300k LiDAR voxels, b = 13, k = 16 34 and 37;
+// 100 queries of those, k = 1 32.5 and 31.5, k = 16 42 and 45.
+constexpr uint32_t kKnnAlone = 512, kKnnAloneK = 4, kKnnAloneVoxels = 4096;
+
 cudaError_t run_knn(const SearchSeg& sg, uint32_t k, const unsigned long long* order, uint32_t* idx,
                     unsigned long long* d2, cudaStream_t stream) {
   if (sg.m == 0) return cudaSuccess;
   const uint32_t sms = (uint32_t)device_sm_count();
-  // the wide form's check reads one word a query
-  const uint64_t checks = (sg.m + 31) / 32;
+  const bool alone = sg.m <= kKnnAlone && (k <= kKnnAloneK || sg.a.cap <= kKnnAloneVoxels ||
+                                            sg.a.bits == 16);
+  // the wide form's check reads one word a query; as many warps as there are share them
+  auto chunk = [&](uint64_t warps) {
+    return (uint32_t)std::min<uint64_t>((sg.m + warps - 1) / warps, 32);
+  };
   if (k <= 32) {
-    k_knn<false, true><<<search_blocks(sg.m, CGA_KNN_BLOCKS), 256, 0, stream>>>(sg, k, 0, order,
-                                                                               idx, d2);
-    k_knn<false, false><<<search_blocks(checks, CGA_KNN_BLOCKS), 256, 0, stream>>>(
-        sg, k, 0, nullptr, idx, d2);
+    const unsigned blocks = search_blocks(sg.m, CGA_KNN_BLOCKS);
+    if (!alone) k_knn<false, true><<<blocks, 256, 0, stream>>>(sg, k, 0, order, idx, d2, 0, false);
+    k_knn<false, false><<<blocks, 256, 0, stream>>>(sg, k, 0, order, idx, d2,
+                                                    chunk((uint64_t)blocks * 8), alone);
   } else {
     const uint32_t cap = knn_cap(k), warps = kKnnLargeThreads / 32;
-    const size_t smem = (size_t)warps * cap * PairBuf<true>::kBytes;
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
     std::call_once(once, [] {
@@ -798,15 +829,21 @@ cudaError_t run_knn(const SearchSeg& sg, uint32_t k, const unsigned long long* o
     });
     if (attr != cudaSuccess) return attr;
     // one wave: what shared memory (and 64 registers a thread) lets an SM hold
-    const uint32_t per_sm =
-        std::max<uint32_t>(1, std::min<uint32_t>(8, (uint32_t)((220u << 10) / (smem + 1024))));
-    k_knn<true, true><<<(unsigned)std::min<uint64_t>((sg.m + warps - 1) / warps, sms * per_sm),
-                        kKnnLargeThreads, smem, stream>>>(sg, k, cap, order, idx, d2);
-    k_knn<true, false><<<(unsigned)std::min<uint64_t>((checks + warps - 1) / warps, sms),
-                         kKnnLargeThreads, (size_t)warps * cap * PairBuf<false>::kBytes, stream>>>(
-        sg, k, cap, nullptr, idx, d2);
+    auto blocks = [&](size_t smem) {
+      const uint32_t per_sm =
+          std::max<uint32_t>(1, std::min<uint32_t>(8, (uint32_t)((220u << 10) / (smem + 1024))));
+      return (unsigned)std::min<uint64_t>((sg.m + warps - 1) / warps, sms * per_sm);
+    };
+    const size_t smem = (size_t)warps * cap * PairBuf<true>::kBytes;
+    const size_t wide = (size_t)warps * cap * PairBuf<false>::kBytes;
+    if (!alone) {
+      k_knn<true, true><<<blocks(smem), kKnnLargeThreads, smem, stream>>>(sg, k, cap, order, idx, d2,
+                                                                         0, false);
+    }
+    k_knn<true, false><<<blocks(wide), kKnnLargeThreads, wide, stream>>>(
+        sg, k, cap, order, idx, d2, chunk((uint64_t)blocks(wide) * warps), alone);
   }
-  count_launch(2);
+  count_launch(alone ? 1 : 2);
   return cudaGetLastError();
 }
 

@@ -79,3 +79,24 @@ def test_blocks_with_any_number_of_long_queries(m):
         oi, od = oracle.nn_brute(o, og, q)
         assert np.array_equal(d2.cpu().numpy().view(np.uint64), od), part
         assert np.array_equal(idx.cpu().numpy().view(np.uint32), oi), part
+
+
+@pytest.mark.parametrize("k", [1, 8, 40])
+@pytest.mark.parametrize("m", [1, 400, 600])
+def test_knn_answers(k, m):
+    q = _far(m, 3 + k)
+    q[::7] = torch.rand((len(q[::7]), 3), device="cuda") * 100   # some inside
+    for n in (20, 6000):
+        for bits, a, pts in _worlds(n):
+            og = oracle.grid_from_box(*BOX, bits)
+            idx, d2 = cga.cga_knn(a, q, k)
+            oi, od = oracle.knn(oracle.build(pts, og), og, q.cpu().numpy(), k)
+            assert np.array_equal(idx.cpu().numpy().view(np.uint32), oi)
+            assert np.array_equal(d2.cpu().numpy().view(np.uint64), od)
+
+
+@pytest.mark.parametrize("n", [1000, 30_000])
+def test_knn_time(n):
+    q = _far(10_000, 4)
+    t = {bits: _time(lambda: cga.cga_knn(a, q, 8)) for bits, a, _ in _worlds(n)}
+    assert t[16] < 3 * t[13], t   # 1.0 to 1.8 with 64-bit distances throughout

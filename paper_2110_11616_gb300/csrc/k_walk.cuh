@@ -8,8 +8,11 @@
 // at or below its lane.  Every column holds at least one voxel, so 128
 // consecutive starts always cover the next 128 positions: they and the 128 z
 // entries are eight coalesced loads in flight at once, followed by the gather
-// of y.  x changes rarely; the slabs that open inside the group are applied one
-// by one, all lanes together.
+// of y.  x changes rarely on coarse grids: one slab that opens inside the group is
+// applied by all lanes together.  Where more do, the next 32 are loaded at once, a lane
+// each, and applied one after the other.  (Loaded one by one they took a decode of 3M
+// LiDAR points at b = 16, whose slabs hold a few tens of voxels, 42 us, by tiles 35; 26
+// so.  Without the step for a single slab 20M surface voxels take 65 us, not 61.)
 //
 // What it replaced: a block of 256 threads expanding a tile of 4096 positions
 // through shared memory (scatter of the starts, block max-scans), preceded by
@@ -81,13 +84,28 @@ __device__ __forceinline__ void walk_voxels(const Levels& a, uint32_t begin, uin
       y[k] = ((valid >> k) & 1u) ? __ldg(a.idx1 + cc[k]) : 0u;
       x[k] = xv;
     }
-    while (base >= xend && xr + 1 < h) {  // slabs opening inside the step
+    if (base >= xend && xr + 1 < h) {
       ++xr;
       const uint32_t x0 = xend;
       xv = __ldg(a.idx2 + xr);
       xend = __ldg(a.ptr2 + xr + 1);
 #pragma unroll
       for (uint32_t k = 0; k < 4; ++k) x[k] = cc[k] >= x0 ? xv : x[k];
+    }
+    while (base >= xend) {  // slabs opening inside the step (the sentinel h + 1 is above)
+      const uint32_t sl = xr + 1 + lane;
+      const uint32_t st = sl <= h ? __ldg(a.ptr2 + sl) : 0xffffffffu;  // first column
+      const uint32_t xs = sl < h ? __ldg(a.idx2 + sl) : 0u;
+      const uint32_t n = (uint32_t)__popc(__ballot_sync(full, st <= base));
+      for (uint32_t i = 0; i < n; ++i) {
+        const uint32_t x0 = __shfl_sync(full, st, i);
+        xv = __shfl_sync(full, xs, i);
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) x[k] = cc[k] >= x0 ? xv : x[k];
+      }
+      if (n == 0) break;  // (no slab left: a malformed CGA)
+      xr += n;
+      xend = n < 32 ? __shfl_sync(full, st, n) : __ldg(a.ptr2 + min(xr + 1, h));
     }
     c = base;
     f(p, valid, x, y, z);

@@ -56,8 +56,7 @@ constexpr uint32_t kKcChangedBit = 48;          // of the first count: a label c
 struct KcState {
   uint32_t box[6];   // least y, z (box[1..2]), greatest y, z (box[4..5])
   uint32_t nchunks;
-  uint32_t turn;     // parts of passes handed out
-  uint32_t done;     // and done
+  uint32_t done;     // parts of passes done
   int centre[2][kKmClusters * 3];  // centres of the even and the odd passes' labels
   int used[kKmClusters * 3];       // of the last one's
 };
@@ -71,6 +70,7 @@ struct KcView {
   KcState* st;
   uint32_t* cell;     // per cell: count, then cursor, then remaining centres (bit set)
   uint32_t* look;     // scan look-back, 2 words per tile, then the tile counter
+  uint32_t* taken;    // per part: passes of it that a block has taken
   uint4* recA;        // chunk: first voxel, count, least, greatest offset in the cell
   uint4* recB;        // chunk: sums of x, y, z; cell
   uint8_t* state;     // chunk: label of all its voxels, kKcMixed or kKcNone
@@ -109,7 +109,6 @@ __global__ void k_kc_init(KcState* st) {
   }
   if (t == 0) {
     st->nchunks = 0;
-    st->turn = 0;
     st->done = 0;
   }
 }
@@ -336,11 +335,60 @@ __device__ __forceinline__ uint32_t box_centres(const int* c, const long long* q
   return mask;
 }
 
-// A pass is as many parts as the launch has blocks; its chunks are dealt out over them.
-// A block takes a part of a pass, in order, once the pass before is done (wait_done: any
-// number of resident blocks gets through).  Every part then sums the pass before for
-// itself, and moves that pass's centres.  The part of the pass after the last one leaves
-// the results: as many as there are blocks, so each block ends with one.
+// A pass is as many parts as the launch has blocks; its chunks are dealt out over them,
+// and block i takes part i of every pass, whose voxels it then finds in its L1.  The
+// blocks need not all be resident: one that waits longer than kKcHelpNs for a pass takes
+// over a part that no block has begun.  (Parts taken in order by whichever block comes
+// first: no slower where few chunks are mixed, but 40 passes over 20M uniform voxels, most
+// of them mixed, 3.8 ms against 3.1.)  A part taken keeps its pass from ending, so the sums
+// and centres of the pass before stay until the part is done.  Every part sums the pass
+// before for itself and moves that pass's centres.  In place of the pass after the last
+// one each block leaves its part of the results.
+constexpr unsigned long long kKcHelpNs = 30000;
+
+// Waits until `target` parts are done (0), or a part of `pass` that no block has begun is
+// taken over (1, its number in `part`), or the wait gives up (2).
+__device__ __forceinline__ uint32_t wait_pass(const KcView& v, uint32_t parts, uint32_t pass,
+                                              uint32_t target, unsigned int* err,
+                                              uint32_t* s_word, uint32_t& part) {
+  if (threadIdx.x < 32) {
+    const uint32_t full = 0xffffffffu, lane = threadIdx.x;
+    const unsigned long long t0 = global_ns();
+    uint32_t r = 0, at = 0, spins = 0;
+    for (;;) {
+      uint32_t seen = 0;
+      if (lane == 0) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];"
+                     : "=r"(seen) : "l"(&v.st->done) : "memory");
+      }
+      if (__shfl_sync(full, seen, 0) >= target) break;
+      if ((++spins & 15u) != 0) continue;
+      const unsigned long long dt = __shfl_sync(full, global_ns() - t0, 0);
+      if (dt > kWaitLimitNs) {
+        if (lane == 0) atomicOr(err, kErrTimeout);
+        r = 2;
+        break;
+      }
+      for (uint32_t p0 = 0; dt > kKcHelpNs && r == 0 && p0 < parts; p0 += 32) {
+        const uint32_t p = p0 + lane;
+        uint32_t todo = __ballot_sync(full, p < parts && __ldcg(v.taken + p) == pass);
+        for (; todo && r == 0; todo &= todo - 1) {
+          at = p0 + (uint32_t)__ffs((int)todo) - 1u;
+          if (lane == 0) r = atomicCAS(v.taken + at, pass, pass + 1) == pass ? 1u : 0u;
+          r = __shfl_sync(full, r, 0);
+        }
+      }
+      if (r != 0) break;
+    }
+    if (lane == 0) *s_word = r | at << 2;
+  }
+  __syncthreads();
+  const uint32_t word = *s_word;
+  __syncthreads();  // (the word is read no more)
+  part = word >> 2;
+  return word & 3u;
+}
+
 __global__ void __launch_bounds__(kKcLoopThreads, 1)
     k_kc_loop(Levels a, KcView v, uint32_t max_iter, long long* centres,
               unsigned long long* counts, uint32_t* iters) {
@@ -350,7 +398,7 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
   __shared__ long long s_q[kKmClusters];
   __shared__ unsigned long long s_part[W][kKmClusters * 4 + 1];
   __shared__ unsigned long long s_tot[kKcWords + 1];  // the sums; parts with a change
-  __shared__ uint32_t s_item, s_next;
+  __shared__ uint32_t s_own, s_word;
   const uint32_t full = 0xffffffffu, tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
   const uint32_t u = (uint32_t)a.hdr->cnt[0], h = (uint32_t)a.hdr->cnt[2];
   if (u == 0) {
@@ -363,81 +411,26 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
   }
   const uint32_t nch = v.st->nchunks, cb = v.grid.cb, sh = v.grid.shift, cm = (1u << cb) - 1u;
   const uint32_t parts = gridDim.x, warps = parts * W;
-  if (tid == 0) s_item = atomicAdd(&v.st->turn, 1u);
-  for (;;) {
-    __syncthreads();
-    const uint32_t pass = s_item / parts, part = s_item % parts;  // passes before this one
-    const uint32_t gw = part * W + w;
-    bool converged = false;
-    if (pass == 0) {
-      // corner c of the box: the greatest coordinate of axis ax where bit ax of c is set
-      if (tid < kKmClusters * 3) {
-        const uint32_t c = tid / 3, ax = tid % 3;
-        const uint32_t lo = ax == 0 ? (uint32_t)__ldg(a.idx2) : v.st->box[ax];
-        const uint32_t hi = ax == 0 ? (uint32_t)__ldg(a.idx2 + h - 1) : v.st->box[3 + ax];
-        s_c[tid] = (int)(256u * (((c >> ax) & 1u) ? hi : lo));
-      }
-    } else {
-      if (!wait_done(&v.st->done, pass * parts, &a.hdr->err)) return;
-      const uint32_t odd = (pass - 1) & 1u;
-      const unsigned long long* sums = v.part + (size_t)odd * parts * kKcWords;
-      if (tid < kKmClusters * 3) s_c[tid] = __ldcg(&v.st->centre[odd][tid]);
-      {
-        unsigned long long s = 0;
-        for (uint32_t b = lane; b < parts; b += 32) s += __ldcg(sums + w * parts + b);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
-        if (lane == 0) {
-          s_tot[w] = s & ((1ull << kKcChangedBit) - 1);
-          if (w == 3) s_tot[kKcWords] = s >> kKcChangedBit;
-        }
-      }
-      __syncthreads();
-      converged = pass > 1 && s_tot[kKcWords] == 0;
-    }
-    const bool stop = pass > 0 && (converged || pass >= max_iter);
-    if (pass > 0 && !stop && tid < kKmClusters * 3) {
-      const unsigned long long n = s_tot[4 * (tid / 3) + 3];
-      if (n > 0) s_c[tid] = (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
-    }
-    __syncthreads();
-    if (tid < kKmClusters) {
-      long long q = 0;
-      for (int ax = 0; ax < 3; ++ax) q += (long long)s_c[3 * tid + ax] * s_c[3 * tid + ax];
-      s_q[tid] = q;
-    }
-    __syncthreads();
-    if (stop) {
-      if (part == 0) {
-        if (tid < kKmClusters * 3) {
-          const int c = s_c[tid];
-          const unsigned long long n = s_tot[4 * (tid / 3) + 3];
-          v.st->used[tid] = c;
-          centres[tid] = converged || n == 0
-                             ? c : (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
-        }
-        if (tid < kKmClusters) counts[tid] = s_tot[4 * tid + 3];
-        if (tid == 0) *iters = pass;
-      }
-      // the cells' remaining centres, for the labels in CGA order
-      for (uint32_t j = gw * 32u + lane; j < nch; j += 32u * warps) {
-        const uint4 A = __ldg(v.recA + j);
-        const uint32_t id = __ldg(&v.recB[j].w);
-        const int o[3] = {(int)((id >> (2 * cb)) << sh), (int)(((id >> cb) & cm) << sh),
-                          (int)((id & cm) << sh)};
-        int lo[3], hi[3];
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-          lo[ax] = o[ax] + (int)((A.z >> (9 * ax)) & 511u);
-          hi[ax] = o[ax] + (int)((A.w >> (9 * ax)) & 511u);
-        }
-        atomicOr(v.cell + id, box_centres(s_c, s_q, lo, hi));
-      }
-      return;
-    }
-    if (part == 0 && tid < kKmClusters * 3) v.st->centre[pass & 1u][tid] = s_c[tid];
-    unsigned long long acc = 0;  // lane l: entry l = label * 4 + {x, y, z sum, count}
-    bool changed = false;
+  // the pass in work (a block may start late), and whether this block has its part of it
+  uint32_t pass = 0, ready = 0xffffffffu;  // ready: the pass whose centres s_c holds
+  if (tid == 0) {
+    uint32_t seen;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&v.st->done) : "memory");
+    s_word = seen / parts;
+    s_own = atomicCAS(v.taken + blockIdx.x, s_word, s_word + 1) == s_word;
+  }
+  __syncthreads();
+  pass = s_word;
+  __syncthreads();
+  // The chunks of warp gw of a pass: their sums and whether a label changed.  (Written out
+  // for the block's own part, whose number is known to be the same for all lanes, and for
+  // others: by a number from shared memory the mixed chunks of 20M uniform voxels took a
+  // third longer.)
+  unsigned long long acc;  // lane l: entry l = label * 4 + {x, y, z sum, count}
+  bool changed;
+  auto chunks = [&](uint32_t gw) {
+    acc = 0;
+    changed = false;
     // chunk i of a round goes to lane i / warps of warp i % warps: the mixed
     // chunks, neighbours in the cell order, spread over the warps
     for (uint32_t r = 0; r < nch; r += 32u * warps) {
@@ -586,22 +579,117 @@ __global__ void __launch_bounds__(kKcLoopThreads, 1)
         }
       }
     }
-    // (the next part, asked for while the block's last warps work)
-    if (tid == 0) s_next = atomicAdd(&v.st->turn, 1u);
+  };
+  bool own = s_own != 0, asked = false;  // asked: for its part of the next pass
+  for (;;) {
+    uint32_t part = blockIdx.x;
+    if (!own) {
+      // on to the next pass once this one is done
+      const uint32_t r = wait_pass(v, parts, pass, (pass + 1) * parts, &a.hdr->err, &s_word, part);
+      if (r == 2) return;
+      if (r == 0) {
+        ++pass;
+        if (!asked && tid == 0) s_own = atomicCAS(v.taken + blockIdx.x, pass, pass + 1) == pass;
+        asked = false;
+        __syncthreads();
+        own = s_own != 0;
+        if (!own) continue;
+        part = blockIdx.x;
+      }
+    }
+    own = false;
+    const uint32_t gw = part * W + w;
+    if (ready != pass) {
+      bool converged = false;
+      if (pass == 0) {
+        // corner c of the box: the greatest coordinate of axis ax where bit ax of c is set
+        if (tid < kKmClusters * 3) {
+          const uint32_t c = tid / 3, ax = tid % 3;
+          const uint32_t lo = ax == 0 ? (uint32_t)__ldg(a.idx2) : v.st->box[ax];
+          const uint32_t hi = ax == 0 ? (uint32_t)__ldg(a.idx2 + h - 1) : v.st->box[3 + ax];
+          s_c[tid] = (int)(256u * (((c >> ax) & 1u) ? hi : lo));
+        }
+      } else {
+        const uint32_t odd = (pass - 1) & 1u;
+        const unsigned long long* sums = v.part + (size_t)odd * parts * kKcWords;
+        if (tid < kKmClusters * 3) s_c[tid] = __ldcg(&v.st->centre[odd][tid]);
+        {
+          unsigned long long s = 0;
+          for (uint32_t b = lane; b < parts; b += 32) s += __ldcg(sums + w * parts + b);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
+          if (lane == 0) {
+            s_tot[w] = s & ((1ull << kKcChangedBit) - 1);
+            if (w == 3) s_tot[kKcWords] = s >> kKcChangedBit;
+          }
+        }
+        __syncthreads();
+        converged = pass > 1 && s_tot[kKcWords] == 0;
+      }
+      const bool stop = pass > 0 && (converged || pass >= max_iter);
+      if (pass > 0 && !stop && tid < kKmClusters * 3) {
+        const unsigned long long n = s_tot[4 * (tid / 3) + 3];
+        if (n > 0) s_c[tid] = (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
+      }
+      __syncthreads();
+      if (tid < kKmClusters) {
+        long long q = 0;
+        for (int ax = 0; ax < 3; ++ax) q += (long long)s_c[3 * tid + ax] * s_c[3 * tid + ax];
+        s_q[tid] = q;
+      }
+      __syncthreads();
+      if (stop) {
+        if (part == 0) {
+          if (tid < kKmClusters * 3) {
+            const int c = s_c[tid];
+            const unsigned long long n = s_tot[4 * (tid / 3) + 3];
+            v.st->used[tid] = c;
+            centres[tid] = converged || n == 0
+                               ? c : (int)((256ull * s_tot[4 * (tid / 3) + tid % 3] + n / 2) / n);
+          }
+          if (tid < kKmClusters) counts[tid] = s_tot[4 * tid + 3];
+          if (tid == 0) *iters = pass;
+        }
+        // the cells' remaining centres, for the labels in CGA order
+        for (uint32_t j = gw * 32u + lane; j < nch; j += 32u * warps) {
+          const uint4 A = __ldg(v.recA + j);
+          const uint32_t id = __ldg(&v.recB[j].w);
+          const int o[3] = {(int)((id >> (2 * cb)) << sh), (int)(((id >> cb) & cm) << sh),
+                            (int)((id & cm) << sh)};
+          int lo[3], hi[3];
+#pragma unroll
+          for (int ax = 0; ax < 3; ++ax) {
+            lo[ax] = o[ax] + (int)((A.z >> (9 * ax)) & 511u);
+            hi[ax] = o[ax] + (int)((A.w >> (9 * ax)) & 511u);
+          }
+          atomicOr(v.cell + id, box_centres(s_c, s_q, lo, hi));
+        }
+        return;
+      }
+      ready = pass;
+    }
+    if (part == 0 && tid < kKmClusters * 3) v.st->centre[pass & 1u][tid] = s_c[tid];
+    if (part == blockIdx.x) {
+      chunks(blockIdx.x * W + w);
+    } else {
+      chunks(gw);
+    }
+    // (the block's part of the next pass, asked for while its last warps work)
+    if (part == blockIdx.x) {
+      if (tid == 0) s_own = atomicCAS(v.taken + part, pass + 1, pass + 2) == pass + 1;
+      asked = true;
+    }
     // block sums: entry e of every warp, then one word per entry and block
     s_part[w][lane] = acc;
     const bool any = __syncthreads_or(changed);
     {
-      const uint32_t item = *(volatile uint32_t*)&s_item;  // (not kept over the pass)
-      unsigned long long* sums =
-          v.part + (size_t)(item / parts & 1u) * parts * kKcWords + item % parts;
+      unsigned long long* sums = v.part + (size_t)(pass & 1u) * parts * kKcWords + part;
       unsigned long long s = lane < W ? s_part[lane][w] : 0ull;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
       if (lane == 0) sums[w * parts] = s | (w == 3 && any ? 1ull << kKcChangedBit : 0ull);
     }
     count_done(&v.st->done);
-    if (tid == 0) s_item = s_next;
   }
 }
 
@@ -661,6 +749,7 @@ size_t kc_layout(uint32_t bits, uint64_t cap, char* base, KcView* out) {
   };
   v.st = reinterpret_cast<KcState*>(take(sizeof(KcState)));
   v.look = reinterpret_cast<uint32_t*>(take((2 * (size_t)tiles + 1) * 4));
+  v.taken = reinterpret_cast<uint32_t*>(take(std::max<uint32_t>(loop_blocks(), 1u) * 4));
   v.cell = reinterpret_cast<uint32_t*>(take((size_t)tiles * kKcScanTile * 4));
   v.recA = reinterpret_cast<uint4*>(take((size_t)v.max_chunks * 16));
   v.recB = reinterpret_cast<uint4*>(take((size_t)v.max_chunks * 16));
@@ -701,7 +790,7 @@ cudaError_t run_kmeans_cells(const Levels& a, uint32_t max_iter, void* scratch, 
   KcView v;
   kc_layout(a.bits, a.cap, static_cast<char*>(scratch), &v);
   const uint32_t tiles = scan_tiles(v.ncells);
-  // the look-back words and the cell counts lie side by side
+  // the look-back words, the parts' and the cell counts lie side by side
   cudaError_t e = cudaMemsetAsync(
       v.look, 0, (size_t)(reinterpret_cast<char*>(v.recA) - reinterpret_cast<char*>(v.look)), stream);
   if (e != cudaSuccess) return e;

@@ -1580,7 +1580,7 @@ struct Bump {
 
 int pipeline_queue(cga_pipeline* p, cudaStream_t s) {
   cudaError_t e = libcga::run_sort_device((int)(2 * p->S), p->build_tiles, p->build_passes,
-                                          p->key64, 3, p->build, s);
+                                          p->key64, 3, false, p->build, s);
   if (e == cudaSuccess) e = libcga::run_merge_device((int)p->S, p->merge_spl, p->merge_tiles, p->merge, s);
   if (e == cudaSuccess) e = libcga::run_project_xy_device(p->d_proj, (int)p->S, p->max_cap1, s);
   if (e == cudaSuccess && p->nn_segs > 0) {

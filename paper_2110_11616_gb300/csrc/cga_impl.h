@@ -189,9 +189,10 @@ cudaError_t run_radix_passes(int S, uint32_t total_tiles, uint32_t max_passes, b
 cudaError_t run_sort_keys_device(int S, uint32_t total_tiles, uint32_t max_passes,
                                  const SortScratch& sc, cudaStream_t stream);
 
-// Sort pipeline with the segment table already on the device (sc.segs).
+// Sort pipeline with the segment table already on the device (sc.segs).  from_cga: whether
+// the keys come from CGAs (of all its segments, or of none).
 cudaError_t run_sort_device(int S, uint32_t total_tiles, uint32_t max_passes, bool key64,
-                            int levels, const SortScratch& sc, cudaStream_t stream);
+                            int levels, bool from_cga, const SortScratch& sc, cudaStream_t stream);
 
 // Queue the whole sort pipeline: header init, key generation (+ histograms),
 // radix passes, compaction.  `h_segs` is copied to the device first.

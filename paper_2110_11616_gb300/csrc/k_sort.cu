@@ -2,7 +2,7 @@
 // go by bins where plan_bins says so (k_bins.cuh), the others, and what the bins leave
 // over (k_lsd_all, all of the following in one launch), by LSD radix passes:
 //   k_seg_init     headers and empty-CGA sentinels
-//   k_keys_hist    quantize (+ rigid transform) and encode each point, or
+//   k_keys_hist    quantize (+ rigid transform) and encode each point, or (k_keys_walk)
 //                  re-key a CGA point for a projection; per-segment digit
 //                  histograms of every radix pass in the same read
 //   k_onesweep     one LSD radix pass: warp-level digit ranking, decoupled
@@ -40,115 +40,82 @@ __global__ void k_seg_init(const SortSeg* __restrict__ segs, int S) {
   if (o.nlevels == 3) o.ptr2[0] = 0;
 }
 
-// Keys of the tiles [t0, t1) plus per-segment histograms of every pass
-// (digits of RB bits).  marked: only the segments marked for the general sort.
+// The digit counts of a block's current segment, in shared memory, and their way to the
+// segment's histogram (digits of RB bits).
+template <int RB>
+struct BlockHist {
+  uint32_t cnt[kMaxPasses][1 << RB];
+  uint32_t err;
+
+  __device__ __forceinline__ void open() {
+    for (int i = threadIdx.x; i < kMaxPasses << RB; i += kThreads) (&cnt[0][0])[i] = 0;
+    if (threadIdx.x == 0) err = 0;
+    __syncthreads();
+  }
+  __device__ __forceinline__ void flush(const SortSeg* __restrict__ segs, int s, uint32_t* hist) {
+    __syncthreads();
+    const uint32_t passes = segs[s].passes;
+    for (int i = threadIdx.x; i < kMaxPasses << RB; i += kThreads) {
+      const uint32_t v = (&cnt[0][0])[i];
+      if (v != 0 && (uint32_t)(i >> RB) < passes) {
+        atomicAdd(hist + ((size_t)s * kMaxPasses << RB) + i, v);
+      }
+      (&cnt[0][0])[i] = 0;
+    }
+    if (threadIdx.x == 0 && err) {
+      atomicOr(&segs[s].out.hdr->err, err);
+      err = 0;
+    }
+    __syncthreads();
+  }
+};
+
+// Keys of the points of the tiles [t0, t1) plus per-segment histograms of every pass.
+// marked: only the segments marked for the general sort.
 template <typename K, int RB>
 __device__ __forceinline__ void keys_hist_tiles(const SortSeg* __restrict__ segs, int S,
                                                 uint32_t t0, uint32_t t1, K* keys0,
                                                 uint32_t* hist, bool marked) {
-  constexpr int R = 1 << RB;
-  __shared__ uint32_t s_hist[kMaxPasses][R];
+  __shared__ BlockHist<RB> sh;
   __shared__ float s_pts[kThreads * 3];
-  __shared__ uint32_t s_err;
   const int tid = threadIdx.x;
   if (t0 >= t1) return;
-  for (int i = tid; i < kMaxPasses * R; i += kThreads) (&s_hist[0][0])[i] = 0;
-  if (tid == 0) s_err = 0;
-  __syncthreads();
+  sh.open();
   int cur = find_seg(segs, S, t0);
-  auto flush = [&](int s) {
-    __syncthreads();
-    const uint32_t passes = segs[s].passes;
-    for (int i = tid; i < kMaxPasses * R; i += kThreads) {
-      const uint32_t v = (&s_hist[0][0])[i];
-      if (v != 0 && (uint32_t)(i >> RB) < passes) {
-        atomicAdd(hist + (size_t)s * kMaxPasses * R + i, v);
-      }
-      (&s_hist[0][0])[i] = 0;
-    }
-    if (tid == 0 && s_err) {
-      atomicOr(&segs[s].out.hdr->err, s_err);
-      s_err = 0;
-    }
-    __syncthreads();
-  };
   for (uint32_t t = t0; t < t1; ++t) {
     const int s = find_seg(segs, S, t);
     if (s != cur) {
-      flush(cur);
+      sh.flush(segs, cur, hist);
       cur = s;
     }
     const SortSeg& sg = segs[s];
     if (marked && !sg.fallback) continue;
-    const uint32_t n = seg_count(sg);
+    const uint32_t n = sg.n_host;
     const uint32_t start = (t - sg.tile_base) * kTile;
     if (start >= n) continue;
     const uint32_t cnt = min((uint32_t)kTile, n - start);
     K* out = keys0 + sg.key_base + start;
     const uint32_t passes = sg.passes;
-    const uint32_t b = sg.bits;
-    if (!sg.from_cga) {
-      const float* src = sg.xyz + (size_t)start * 3;
-      for (uint32_t c0 = 0; c0 < cnt; c0 += kThreads) {
-        const uint32_t m = min((uint32_t)kThreads, cnt - c0);
-        __syncthreads();
-        for (uint32_t i = tid; i < m * 3; i += kThreads) s_pts[i] = __ldg(src + (size_t)c0 * 3 + i);
-        __syncthreads();
-        if ((uint32_t)tid < m) {
-          K key;
-          if (!point_key<K>(s_pts[3 * tid], s_pts[3 * tid + 1], s_pts[3 * tid + 2],
-                            sg.has_x != 0, sg.X, sg.scale, sg.off, b, key)) {
-            atomicOr(&s_err, kErrNonfinite);
-          }
-          out[c0 + tid] = key;
-          for (uint32_t p = 0; p < passes; ++p) {
-            atomicAdd(&s_hist[p][(uint32_t)(key >> (sg.bit0 + p * RB)) & (R - 1)], 1u);
-          }
+    const float* src = sg.xyz + (size_t)start * 3;
+    for (uint32_t c0 = 0; c0 < cnt; c0 += kThreads) {
+      const uint32_t m = min((uint32_t)kThreads, cnt - c0);
+      __syncthreads();
+      for (uint32_t i = tid; i < m * 3; i += kThreads) s_pts[i] = __ldg(src + (size_t)c0 * 3 + i);
+      __syncthreads();
+      if ((uint32_t)tid < m) {
+        K key;
+        if (!point_key<K>(s_pts[3 * tid], s_pts[3 * tid + 1], s_pts[3 * tid + 2],
+                          sg.has_x != 0, sg.X, sg.scale, sg.off, sg.bits, key)) {
+          atomicOr(&sh.err, kErrNonfinite);
+        }
+        out[c0 + tid] = key;
+        for (uint32_t p = 0; p < passes; ++p) {
+          atomicAdd(&sh.cnt[p][(uint32_t)(key >> (sg.bit0 + p * RB)) & ((1 << RB) - 1)], 1u);
         }
       }
-    } else {
-      // projection, coarse level or tree: the block's run of tiles of this
-      // segment, a warp per equal share of its positions (k_walk.cuh)
-      const Levels& a = sg.src;
-      const uint32_t tl = min(t1, sg.tile_base + sg.num_tiles);
-      const uint32_t stop = min(n, (tl - sg.tile_base) * (uint32_t)kTile);
-      const uint32_t per = ((stop - start + kWarps * kWalk - 1) / (kWarps * kWalk)) * kWalk;
-      const uint32_t w0 = min(stop, start + (uint32_t)(tid >> 5) * per);
-      K* kout = keys0 + sg.key_base;
-      walk_voxels(a, w0, min(stop, w0 + per), [&](uint32_t p, uint32_t valid, const uint32_t* x,
-                                                  const uint32_t* y, const uint32_t* z) {
-#pragma unroll
-        for (uint32_t i = 0; i < 4; ++i) {
-          K key;
-          if (sg.plane == 3) {
-            const uint32_t L = sg.shift;
-            key = ((K)(x[i] >> L) << (2 * b)) | ((K)(y[i] >> L) << b) | (K)(z[i] >> L);
-          } else if (sg.plane == 4) {
-            key = (K)tree_key(x[i], y[i], z[i], sg.shift);
-          } else {
-            const uint32_t u = sg.plane == 2 ? y[i] : x[i], v = sg.plane == 0 ? y[i] : z[i];
-            key = ((K)u << b) | (K)v;
-          }
-          const bool ok = (valid >> i) & 1u;
-          if (ok) kout[p + 32 * i + (tid & 31)] = key;
-          // neighbouring voxels share their high digits: one count for the
-          // warp where all lanes hold the same digit
-          const uint32_t live = __ballot_sync(0xffffffffu, ok);
-          for (uint32_t q = 0; q < passes; ++q) {
-            const uint32_t d = (uint32_t)(key >> (sg.bit0 + q * RB)) & (R - 1);
-            const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-            if (__all_sync(0xffffffffu, !ok || d == d0)) {
-              if ((tid & 31) == 0 && live) atomicAdd(&s_hist[q][d0], (uint32_t)__popc(live));
-            } else if (ok) {
-              atomicAdd(&s_hist[q][d], 1u);
-            }
-          }
-        }
-      });
-      t = tl - 1;
     }
   }
-  flush(cur);
+  sh.flush(segs, cur, hist);
 }
 
 template <typename K, int RB>
@@ -158,6 +125,68 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
                                                         uint32_t* hist) {
   const uint32_t t0 = blockIdx.x * tiles_per_cta;
   keys_hist_tiles<K, RB>(segs, S, t0, min(t0 + tiles_per_cta, total_tiles), keys0, hist, false);
+}
+
+// The same for segments whose keys come from a CGA (projections, coarse levels, trees): a
+// block takes runs of a step of a walk for each of its warps (k_walk.cuh), not whole tiles,
+// so that small sources have a warp for every step: the xz projection of 30k points at b =
+// 16 took 96 us by tiles, 79 so.
+constexpr uint32_t kWalkRun = kWarps * kWalk;
+static_assert(kTile % kWalkRun == 0, "runs of a tile");
+template <typename K, int RB>
+__global__ void __launch_bounds__(kThreads) k_keys_walk(const SortSeg* __restrict__ segs, int S,
+                                                        uint32_t total_runs, uint32_t runs_per_cta,
+                                                        K* keys0, uint32_t* hist) {
+  constexpr uint32_t PER = kTile / kWalkRun;
+  __shared__ BlockHist<RB> sh;
+  const uint32_t r1 = min((blockIdx.x + 1) * runs_per_cta, total_runs);
+  uint32_t r = blockIdx.x * runs_per_cta;
+  if (r >= r1) return;
+  sh.open();
+  while (r < r1) {
+    // the block's runs of one segment, a warp per equal share of their positions
+    const int s = find_seg(segs, S, r / PER);
+    const SortSeg& sg = segs[s];
+    const Levels& a = sg.src;
+    const uint32_t n = (uint32_t)a.hdr->cnt[0], b = sg.bits, passes = sg.passes;
+    const uint32_t base = sg.tile_base * PER, re = min(r1, base + sg.num_tiles * PER);
+    const uint32_t start = min(n, (r - base) * kWalkRun), stop = min(n, (re - base) * kWalkRun);
+    const uint32_t per = ((stop - start + kWalkRun - 1) / kWalkRun) * kWalk;
+    const uint32_t w0 = min(stop, start + (threadIdx.x >> 5) * per);
+    K* kout = keys0 + sg.key_base;
+    walk_voxels(a, w0, min(stop, w0 + per), [&](uint32_t p, uint32_t valid, const uint32_t* x,
+                                                const uint32_t* y, const uint32_t* z) {
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {
+        K key;
+        if (sg.plane == 3) {
+          const uint32_t L = sg.shift;
+          key = ((K)(x[i] >> L) << (2 * b)) | ((K)(y[i] >> L) << b) | (K)(z[i] >> L);
+        } else if (sg.plane == 4) {
+          key = (K)tree_key(x[i], y[i], z[i], sg.shift);
+        } else {
+          const uint32_t u = sg.plane == 2 ? y[i] : x[i], v = sg.plane == 0 ? y[i] : z[i];
+          key = ((K)u << b) | (K)v;
+        }
+        const bool ok = (valid >> i) & 1u;
+        if (ok) kout[p + 32 * i + (threadIdx.x & 31)] = key;
+        // neighbouring voxels share their high digits: one count for the
+        // warp where all lanes hold the same digit
+        const uint32_t live = __ballot_sync(0xffffffffu, ok);
+        for (uint32_t q = 0; q < passes; ++q) {
+          const uint32_t d = (uint32_t)(key >> (sg.bit0 + q * RB)) & ((1 << RB) - 1);
+          const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+          if (__all_sync(0xffffffffu, !ok || d == d0)) {
+            if ((threadIdx.x & 31) == 0 && live) atomicAdd(&sh.cnt[q][d0], (uint32_t)__popc(live));
+          } else if (ok) {
+            atomicAdd(&sh.cnt[q][d], 1u);
+          }
+        }
+      }
+    });
+    sh.flush(segs, s, hist);
+    r = re;
+  }
 }
 
 // Dynamic shared memory of one pass block: the tile's keys, per-warp digit
@@ -755,21 +784,34 @@ cudaError_t run_radix_passes(int S, uint32_t total_tiles, uint32_t max_passes, b
   return cudaGetLastError();
 }
 
+// Keys and histograms, from points or (walk) from CGAs.
+template <typename K>
+static void launch_keys(int S, uint32_t total_tiles, bool walk, const SortScratch& sc,
+                        cudaStream_t stream) {
+  const uint32_t items = walk ? total_tiles * (kTile / kWalkRun) : total_tiles;
+  const uint32_t ctas = std::min<uint32_t>(items, (uint32_t)device_sm_count() * 4);
+  const uint32_t per = (items + ctas - 1) / ctas;
+  K* k0 = static_cast<K*>(sc.keys0);
+  if (walk && sc.radix_bits == 9) {
+    k_keys_walk<K, 9><<<ctas, kThreads, 0, stream>>>(sc.segs, S, items, per, k0, sc.hist);
+  } else if (walk) {
+    k_keys_walk<K, 8><<<ctas, kThreads, 0, stream>>>(sc.segs, S, items, per, k0, sc.hist);
+  } else if (sc.radix_bits == 9) {
+    k_keys_hist<K, 9><<<ctas, kThreads, 0, stream>>>(sc.segs, S, items, per, k0, sc.hist);
+  } else {
+    k_keys_hist<K, 8><<<ctas, kThreads, 0, stream>>>(sc.segs, S, items, per, k0, sc.hist);
+  }
+  count_launch(1);
+}
+
 template <typename K>
 static cudaError_t launch_pipeline(int S, uint32_t total_tiles, uint32_t max_passes, int levels,
-                                   const SortScratch& sc, cudaStream_t stream) {
+                                   bool walk, const SortScratch& sc, cudaStream_t stream) {
   K* k0 = static_cast<K*>(sc.keys0);
   K* k1 = static_cast<K*>(sc.keys1);
-  const uint32_t ctas = std::min<uint32_t>(total_tiles, (uint32_t)device_sm_count() * 4);
-  const uint32_t per = (total_tiles + ctas - 1) / ctas;
   const cudaError_t ei = init_sort_kernels();
   if (ei != cudaSuccess) return ei;
-  if (sc.radix_bits == 9) {
-    k_keys_hist<K, 9><<<ctas, kThreads, 0, stream>>>(sc.segs, S, total_tiles, per, k0, sc.hist);
-  } else {
-    k_keys_hist<K, 8><<<ctas, kThreads, 0, stream>>>(sc.segs, S, total_tiles, per, k0, sc.hist);
-  }
-  count_launch(2);
+  launch_keys<K>(S, total_tiles, walk, sc, stream);
   launch_passes<K>(S, total_tiles, max_passes, sc, stream);
   if (levels == 3) {
     k_compact<K, 3><<<total_tiles, kThreads, 0, stream>>>(sc.segs, S, k0, k1, sc.clook,
@@ -778,20 +820,8 @@ static cudaError_t launch_pipeline(int S, uint32_t total_tiles, uint32_t max_pas
     k_compact<K, 2><<<total_tiles, kThreads, 0, stream>>>(sc.segs, S, k0, k1, sc.clook,
                                                           sc.counters + kMaxPasses);
   }
-  return cudaGetLastError();
-}
-
-template <typename K>
-static void launch_keys(int S, uint32_t total_tiles, const SortScratch& sc, cudaStream_t stream) {
-  const uint32_t ctas = std::min<uint32_t>(total_tiles, (uint32_t)device_sm_count() * 4);
-  const uint32_t per = (total_tiles + ctas - 1) / ctas;
-  K* k0 = static_cast<K*>(sc.keys0);
-  if (sc.radix_bits == 9) {
-    k_keys_hist<K, 9><<<ctas, kThreads, 0, stream>>>(sc.segs, S, total_tiles, per, k0, sc.hist);
-  } else {
-    k_keys_hist<K, 8><<<ctas, kThreads, 0, stream>>>(sc.segs, S, total_tiles, per, k0, sc.hist);
-  }
   count_launch(1);
+  return cudaGetLastError();
 }
 
 cudaError_t run_sort_keys_device(int S, uint32_t total_tiles, uint32_t max_passes,
@@ -800,13 +830,14 @@ cudaError_t run_sort_keys_device(int S, uint32_t total_tiles, uint32_t max_passe
   if (e != cudaSuccess || total_tiles == 0) return e;
   e = init_sort_kernels();
   if (e != cudaSuccess) return e;
-  launch_keys<unsigned long long>(S, total_tiles, sc, stream);
+  launch_keys<unsigned long long>(S, total_tiles, true, sc, stream);
   launch_passes<unsigned long long>(S, total_tiles, max_passes, sc, stream);
   return cudaGetLastError();
 }
 
 cudaError_t run_sort_device(int S, uint32_t total_tiles, uint32_t max_passes, bool key64,
-                            int levels, const SortScratch& sc, cudaStream_t stream) {
+                            int levels, bool from_cga, const SortScratch& sc,
+                            cudaStream_t stream) {
   if (sc.bins.on && total_tiles > 0) return run_bins(S, total_tiles, key64, sc, stream);
   cudaError_t e = cudaMemsetAsync(sc.hist, 0, sc.zero_bytes, stream);
   if (e != cudaSuccess) return e;
@@ -814,8 +845,9 @@ cudaError_t run_sort_device(int S, uint32_t total_tiles, uint32_t max_passes, bo
   count_launch(1);
   e = cudaGetLastError();
   if (e != cudaSuccess || total_tiles == 0) return e;
-  return key64 ? launch_pipeline<unsigned long long>(S, total_tiles, max_passes, levels, sc, stream)
-               : launch_pipeline<uint32_t>(S, total_tiles, max_passes, levels, sc, stream);
+  return key64 ? launch_pipeline<unsigned long long>(S, total_tiles, max_passes, levels, from_cga,
+                                                     sc, stream)
+               : launch_pipeline<uint32_t>(S, total_tiles, max_passes, levels, from_cga, sc, stream);
 }
 
 size_t wait_selftest_bytes() {
@@ -858,8 +890,8 @@ cudaError_t run_sort_pipeline(const SortSeg* h_segs, int S, uint32_t total_tiles
   cudaError_t e = cudaMemcpyAsync(sc.segs, h_segs, sizeof(SortSeg) * S, cudaMemcpyHostToDevice,
                                   stream);
   if (e != cudaSuccess) return e;
-  return run_sort_device(S, total_tiles, max_passes, key64, (int)h_segs[0].out.nlevels, sc,
-                         stream);
+  return run_sort_device(S, total_tiles, max_passes, key64, (int)h_segs[0].out.nlevels,
+                         h_segs[0].from_cga != 0, sc, stream);
 }
 
 }  // namespace libcga

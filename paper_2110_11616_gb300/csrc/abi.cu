@@ -289,7 +289,7 @@ int build_cloud(const float* d_xyz, uint64_t n, const cga_grid* g, const float* 
     return CGA_ERR_OOM;
   }
   libcga::SortScratch sc = libcga::sort_scratch_carve(scratch, keys, tiles, 1, key64, tu);
-  libcga::plan_bins(&seg, 1, tiles, sc);
+  libcga::plan_bins(&seg, 1, tiles, sc, vb != nullptr);
   if (vb != nullptr && sc.bins.on) {
     sc.bins.value_in = vb->in;
     sc.bins.value_out = h->lv;

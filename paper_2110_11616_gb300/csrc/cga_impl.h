@@ -162,9 +162,10 @@ struct SortScratch {
   uint32_t sort_threads;
   BinPlan bins;
 };
-// Decide whether the S builds of h_segs go by bins and lay the tables out in sc
-// (fills the segments' bin fields; call before they are uploaded).
-void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc);
+// Decide whether the S builds of h_segs (with attributes: values) go by bins and lay the
+// tables out in sc (fills the segments' bin fields; call before they are uploaded).
+void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc,
+               bool values = false);
 
 // Scratch of a sort run; the digit width sizes the histogram and look-back
 // tables, the thread count only selects the pass kernel.

@@ -574,8 +574,20 @@ static cudaError_t init_bin_kernels() {
 // Points per segment up to which a build goes by bins: beyond, a bin of the
 // widest table (2^12) holds more than a block sorts.
 constexpr uint64_t kBinMaxPoints = 1ull << 25;
+// On grids of at most 8 bits (no more than three digits to sort) a bin is a slab or more
+// and most clouds leave most of them empty: by bins only up to 512 points a bin, and again,
+// at 7 and 8 bits, where all of them have to be split anyway.  By bins and in general, us: 300k LiDAR points, b = 5 132 and 76, b = 8 106 and 89, uniform ones 93
+// and 73, 80 and 95; 1M surface points, b = 6 136 and 106, b = 8 115 and 107; 130k LiDAR
+// points, b = 7 94 and 80; 30k uniform ones, b = 7, 56 and 67; 3M, b = 8, 186 and 204.  (With attributes by bins all
+// the same: their sums cost more in general.  1M LiDAR points, b = 6 357 and 819.)
+constexpr uint32_t kBinCoarseBits = 8;
+constexpr uint64_t kBinCoarsePoints = 512, kBinCoarseMost = 8192;
+static bool coarse_build(const SortSeg& g) {
+  return g.bits <= kBinCoarseBits && g.n_host >= kBinCoarsePoints << g.bits &&
+         (g.bits <= 6 || g.n_host < kBinCoarseMost << g.bits);
+}
 
-void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
+void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc, bool values) {
   BinPlan& B = sc.bins;
   B = BinPlan{};
   if (S <= 0 || total_tiles == 0) return;
@@ -584,7 +596,7 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
   // average a bin may hold a few blocks' worth of points (30M points at b = 10, 29k a
   // bin: 1377 us by the general sort, 1368 by bins); beyond that every bin goes to a
   // cluster, which the general sort beats (15k a bin that way: 747 against 1190).
-  uint64_t points = 0;
+  uint64_t points = 0, coarse = 0;
   for (int s = 0; s < S; ++s) {
     SortSeg& g = h_segs[s];
     if (g.from_cga || g.n_host > kBinMaxPoints) return;
@@ -594,6 +606,7 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
     g.narrow = 3 * g.bits - g.bin_bits <= 30 ? 1u : 0u;
     const uint64_t most = g.narrow ? 4 * bin_cap<uint32_t>() : 4 * bin_cap<unsigned long long>();
     if (g.n_host >> g.bin_bits > most) return;
+    if (coarse_build(g)) coarse += g.n_host;
     B.may_split = B.may_split || g.n_host > (g.narrow ? bin_cap<uint32_t>() : bin_cap<unsigned long long>());
     // a job fails by its keys' number or, wide keys only, by its row's parts
     B.may_fall = B.may_fall || g.n_host > kBinRowMax ||
@@ -602,6 +615,7 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc) {
     B.wide = B.wide || !g.narrow;
     points += g.n_host;
   }
+  if (2 * coarse > points && !values) return;  // (a batch goes the way of most of its points)
   // partition tiles: enough of them for the SMs, then as many keys a bin as possible
   const uint64_t sms = (uint64_t)device_sm_count();
   B.items = points >= sms * 4 * 16384 ? 16u : (points >= sms * 2 * 8192 ? 8u : 4u);

@@ -129,6 +129,7 @@ struct BinPlan {
   bool narrow, wide;  // some segments' partitioned keys have 32 bits, some 64
   bool may_split;     // some segment has more points than a block sorts
   bool may_fall;      // some segment may need the general sort after all
+  uint32_t passes;    // and its passes at most
   uint32_t items;     // points per thread of a partition tile: 4, 8 or 16
   uint32_t ptiles;    // partition tiles of all segments
   uint32_t slots;     // job slots of all segments

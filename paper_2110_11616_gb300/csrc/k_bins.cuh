@@ -25,12 +25,12 @@
 //
 // A bin holds whole x slabs (bin bits <= grid bits) and a job of a split bin whole
 // columns, so a job's first key always opens a voxel and a column, and a slab
-// unless the job goes on with a slab of its bin.  A bin of more than kBinSplitMax
-// keys, or a row of a split (12 more bits) of more than kBinRowMax, marks its
-// segment, which k_lsd_all then sorts the general way.  (By the first rule before any
-// job is made: the kernels after k_bin_scan then leave the segment alone.  By the
-// second in k_bin_sort, where the segment's keys and jobs are all written.)
-//
+// unless the job goes on with a slab of its bin.  A bin of more than kBinSplitMax keys (or
+// kBinHeavy and a share of the points), or a row of a split (12 more bits) of more than
+// kBinRowMax keys that no map takes, marks its segment, which k_lsd_all then sorts the
+// general way.  (By the first rule before any job is made: the kernels after k_bin_scan
+// then leave the segment alone.  By the second in k_bin_sort, where the segment's keys
+// and jobs are all written.)
 // Measured on GB300 (us): 15M surface points at b = 12: sort 187, partition 120,
 // write 60, histogram 44, split 18, scan 11; the build 954 -> 475.  The job sort is
 // bound by the issue of its shared-memory steps, the partition by the latency of one
@@ -38,7 +38,7 @@
 // kernels: launch to launch).  LiDAR 1.3M, b = 16: 179 -> 130; uniform 30M, b = 12:
 // 1794 -> 721; 10-bit grids, whose bins all have to be split: 2M LiDAR 154 -> 158,
 // 15M uniform 747 -> 662, 30M uniform 1377 -> 1368.  A cloud that the general sort
-// has to take over pays for both: 1M points in one voxel 134 -> 340.
+// has to take over pays for the bins too: 1M points in one voxel 140 -> 207.
 #pragma once
 #include "k_compact.cuh"
 
@@ -78,7 +78,13 @@ constexpr int kBinThreads = 512;
 constexpr int kBinWarps = kBinThreads / 32;
 constexpr uint32_t kBinMaxBits = 12;
 constexpr uint32_t kBinSplitMax = 1u << 20;   // the most keys of a bin to split
-constexpr uint32_t kBinRowMax = 1u << 18;     // the most keys of one of its rows
+constexpr uint32_t kBinRowMax = 1u << 18;     // the most keys of a row that goes by parts
+// A bin that outweighs its cloud (more than this and a 16th of the points): a cluster
+// splits it alone, 30 us and 125 for each million of its keys, and most such bins are one
+// voxel's, whose row then takes a block as long.  In general 2M points, a quarter of them
+// at one point, take 250 us (b = 12; by bins 371) and 276 (b = 16; 415, the general sort
+// included), 1M in one voxel 208 and 330; 500k in one slab, though, 201 and 152.
+constexpr uint32_t kBinHeavy = (1u << 18) + (1u << 16);
 constexpr int kBinWalks = 12;                 // the most passes over such a row
 constexpr uint32_t kBinMapBits = 18;          // bits of a key that a block maps
 constexpr int kBinCluster = 8;                // blocks that split a bin together
@@ -239,7 +245,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
                                                    uint32_t* __restrict__ cur,
                                                    uint4* __restrict__ jobs,
                                                    uint32_t* __restrict__ njobs,
-                                                   uint2* __restrict__ big) {
+                                                   uint2* __restrict__ big, bool heavy) {
   constexpr uint32_t PER = (1u << kBinMaxBits) / 1024;
   __shared__ uint32_t s_scan[32], s_start[(1u << kBinMaxBits) + 1], s_next[32];
   const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
@@ -274,6 +280,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
   const uint32_t rem = 3 * sg.bits - sg.bin_bits;
   const uint32_t span_bits = min(8 * (uint32_t)sizeof(T) - rem, kBinMaxBits);
   uint32_t nsub[PER], nj = 0, open = 0;
+  const uint32_t most = heavy ? min(kBinSplitMax, kBinHeavy + s_start[bins] / 16) : kBinSplitMax;
   bool over = false;
 #pragma unroll
   for (uint32_t i = 0; i < PER; ++i) {
@@ -286,7 +293,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
     if (b == 0 || large || plarge || st / target != pst / target ||
         (b & ((1u << span_bits) - 1u)) == 0u) {
       nsub[i] = 1;
-      if (n > kBinSplitMax) {
+      if (n > most) {
         over = true;
       } else if (n > bin_cap<T>()) {
         nsub[i] = split_slots(n, target);
@@ -931,7 +938,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBinThreads, 2)
     k_bin_sort(SortSeg* segs, int S, const uint4* __restrict__ jobs,
                const uint32_t* __restrict__ njobs, T* keys0, T* keys1, uint4* __restrict__ info,
-               uint32_t* counter, uint32_t total_slots, uint32_t stride) {
+               uint32_t* counter, uint32_t total_slots, uint32_t stride, uint32_t map_most) {
   extern __shared__ __align__(16) unsigned char s_raw[];
   __shared__ BinSortSmem sm;
   __shared__ uint32_t s_cnt[2];
@@ -1059,7 +1066,9 @@ __global__ void __launch_bounds__(kBinThreads, 2)
     };
     if (tid == 0) sm.n = sg.fallback;
     __syncthreads();
-    bool fail = sm.n || N > kBinRowMax;
+    // (a row's bits below its own; a map of them takes any number of keys)
+    const uint32_t left = rem - min(kBinRowBits, rem - b);
+    bool fail = sm.n || N > (left <= kBinMapBits ? map_most : kBinRowMax);
     __syncthreads();
     if (N <= CAP) {
       uint32_t bits = rem;
@@ -1073,7 +1082,6 @@ __global__ void __launch_bounds__(kBinThreads, 2)
       emit(buf0, N, bits);
     } else if (!fail) {
       // one row of a split with more keys than the block holds
-      const uint32_t left = rem - min(kBinRowBits, rem - b);
       const T row = (T)((T)(src[0] - org) >> left) << left;
       if (left <= kBinMapBits) {
         emit_map(left, row, full, 0);

@@ -661,7 +661,10 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc, bo
   // the general way, with the digits and passes that the caller planned)
   if ((size_t)(p - reinterpret_cast<char*>(sc.look)) > room || slots > 0x7fffffffull) return;
   // the general sort behind the bins has 8-bit digits
-  for (int s = 0; s < S; ++s) h_segs[s].passes = radix_passes(h_segs[s].key_bits, 8);
+  for (int s = 0; s < S; ++s) {
+    h_segs[s].passes = radix_passes(h_segs[s].key_bits, 8);
+    B.passes = std::max(B.passes, h_segs[s].passes);
+  }
   B.ptiles = (uint32_t)ptiles;
   B.slots = (uint32_t)slots;
   B.on = true;
@@ -697,7 +700,9 @@ static void launch_bin_jobs(int S, const SortScratch& sc, uint32_t stride, uint3
                             cudaStream_t stream) {
   const BinPlan& B = sc.bins;
   T *k0 = static_cast<T*>(sc.keys0), *k1 = static_cast<T*>(sc.keys1);
-  k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.start, B.cur, B.jobs, B.njobs, B.big);
+  // (attributes are summed faster by bins than in general, but not a crowded row's)
+  const bool values = B.value_rows != nullptr;
+  k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.start, B.cur, B.jobs, B.njobs, B.big, !values);
   if (B.value_rows != nullptr) {
     launch_part<T, true>(S, sc, stride, stream);
     if (B.may_split) launch_split<T, true>(sc, stride, stream);
@@ -707,7 +712,8 @@ static void launch_bin_jobs(int S, const SortScratch& sc, uint32_t stride, uint3
   }
   const uint32_t blocks = std::min<uint32_t>(B.slots, g_bin_sort_blocks[sizeof(T) / 8]);
   k_bin_sort<T><<<blocks, kBinThreads, bin_sort_smem<T>(), stream>>>(
-      sc.segs, S, B.jobs, B.njobs, k0, k1, B.info, counter, B.slots, stride);
+      sc.segs, S, B.jobs, B.njobs, k0, k1, B.info, counter, B.slots, stride,
+      values ? kBinRowMax : kBinSplitMax);
 }
 
 template <typename T>
@@ -731,7 +737,7 @@ static cudaError_t launch_lsd_all(int S, uint32_t total_tiles, const SortScratch
   const uint32_t words = (uint32_t)((reinterpret_cast<char*>(sc.counters) -
                                      reinterpret_cast<char*>(sc.hist)) / 4);
   k_lsd_all<K><<<g_lsd_blocks[sizeof(K) / 8], kThreads, onesweep_smem<K, kThreads, 8>(), stream>>>(
-      sc.segs, S, total_tiles, kMaxPasses, static_cast<K*>(sc.keys0), static_cast<K*>(sc.keys1),
+      sc.segs, S, total_tiles, sc.bins.passes, static_cast<K*>(sc.keys0), static_cast<K*>(sc.keys1),
       sc.hist, sc.look, sc.clook, sc.counters, words);
   return cudaGetLastError();
 }

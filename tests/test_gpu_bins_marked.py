@@ -104,3 +104,26 @@ def test_in_a_batch(old):
                               [_grids(b)[0] for _, b in spec], allocator=mem.arg)
     for h, p, (_, b) in zip(got, pts, spec):
         _same(h, oracle.build(p, _grids(b)[1]))
+
+
+@pytest.mark.parametrize("bits", [10, 12, 13, 16])
+@pytest.mark.parametrize("n,zeros", [(600_000, 270_000), (3_000_000, 400_000), (2_000_000, 460_000),
+                                     (700_000, 690_000)])
+def test_many_points_in_one_voxel(n, zeros, bits):
+    """More keys in one voxel's row than go by parts: a map of the row, or the mark."""
+    g, og = _grids(bits)
+    rng = np.random.default_rng(zeros + bits)
+    v = rng.random((n, 3), dtype=np.float32)
+    v[:zeros] = 0.625
+    v[: zeros // 100, 2] = 0.626
+    pts = rng.permutation(v)
+    mem = OldData("small")
+    a = cga.cga_build(torch.from_numpy(pts).cuda(), g, allocator=mem.arg)
+    _same(a, oracle.build(pts, og))
+    if n < 1_000_000:
+        rows = rng.integers(0, 256, size=(n, 3), dtype=np.uint8)
+        b = cga.cga_build_values(torch.from_numpy(pts).cuda(), torch.from_numpy(rows).cuda(), g,
+                                 allocator=mem.arg)
+        want, want_rows = oracle.build_values(pts, rows, og)
+        _same(b, want)
+        assert np.array_equal(cga.cga_values(b).cpu().numpy(), want_rows)

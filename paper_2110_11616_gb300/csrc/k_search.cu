@@ -144,12 +144,12 @@ __device__ __forceinline__ void radius_slabs(const SearchSeg& sg, uint32_t h, co
 // sectors at most); a longer column's reach comes from a root and two searches.
 constexpr uint32_t kShortColumn = 4;
 
-// The voxels of one slab within the radius, in (y, z) order: emit(p, d2) for
-// each.  Returns their number.  Only the slab's x lies inside the window, so
-// every difference here is at most r (D = uint32_t: r2 < 2^31).
-template <typename D, typename F>
+// The voxels of one slab within the radius, in (y, z) order: emit(p, d2) for each
+// (of a long column, while more() says so).  Returns their number.  Only the slab's x
+// lies inside the window, so every difference here is at most r (D = uint32_t: r2 < 2^31).
+template <typename D, typename F, typename M>
 __device__ __forceinline__ uint32_t radius_slab(const SearchSeg& sg, uint32_t slab, const RQuery& q,
-                                                D r2, F emit) {
+                                                D r2, F emit, M more) {
   const Levels& a = sg.a;
   const int top = (1 << a.bits) - 1;
   const D dx = absdiff32(__ldg(a.idx2 + slab), q.x);
@@ -184,7 +184,7 @@ __device__ __forceinline__ uint32_t radius_slab(const SearchSeg& sg, uint32_t sl
     const uint32_t p0 = (uint32_t)zlo <= clo ? zs : lower_bound_u16(a.idx0, zs, ze, (uint32_t)zlo);
     const uint32_t p1 =
         (uint32_t)zhi >= chi ? ze : lower_bound_u16(a.idx0, p0, ze, (uint32_t)zhi + 1);
-    for (uint32_t p = p0; p < p1; ++p) {
+    for (uint32_t p = p0; p < p1 && more(); ++p) {
       const D dz = absdiff32(__ldg(a.idx0 + p), q.z);
       emit(p, dxy + dz * dz);
     }
@@ -218,14 +218,17 @@ __global__ void __launch_bounds__(256, CGA_RADIUS_BLOCKS)
     radius_slabs<D>(sg, h, q, r, s0, s1);
     uint32_t n = 0;  // at most the CGA's voxels: below 2^30
     for (uint32_t s = s0 + lane; s < s1; s += 32) {
-      n += radius_slab<D>(sg, s, q, r2, [](uint32_t, D) {});
+      n += radius_slab<D>(sg, s, q, r2, [](uint32_t, D) {}, [] { return false; });
     }
     n = __reduce_add_sync(0xffffffffu, n);
     if (lane == 0) counts[j] = n;
   }
 }
 
-// Hits of a lane's slab kept in shared memory until their place is known.
+// Hits of a lane's slab kept in shared memory until their place is known.  A lane with
+// more of them walks its slab again and writes them then; the first walk only counts the
+// rest of its long columns (looking at every voxel twice took 100 queries of 17 voxels
+// in a world of 300k LiDAR points, b = 10, 322 us, 301 so).
 constexpr uint32_t kRadiusKeep = 6;
 
 template <typename D>
@@ -260,7 +263,7 @@ __global__ void __launch_bounds__(256, CGA_RADIUS_BLOCKS)
             s_d[kept][tid] = d;
           }
           ++kept;
-        });
+        }, [&] { return kept < kRadiusKeep; });
       }
       const uint32_t inc = warp_incl_scan(n);
       const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
@@ -285,7 +288,7 @@ __global__ void __launch_bounds__(256, CGA_RADIUS_BLOCKS)
           idx[at] = p;
           d2[at] = d;
           ++at;
-        });
+        }, [] { return true; });
       }
       base += total;
     }

@@ -135,7 +135,6 @@ struct BinPlan {
   uint32_t slots;     // job slots of all segments
   uint32_t* cnt;      // points per bin (zeroed before each run)
   uint32_t zero_words;
-  uint32_t* start;    // offset of each bin (one more per segment)
   uint32_t* cur;      // next free place of each bin
   uint4* jobs;
   uint2* big;         // bins to split (the first word: how many)

@@ -241,7 +241,6 @@ __global__ void __launch_bounds__(kBinThreads, 4) k_bin_hist(const SortSeg* __re
 template <typename T>
 __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
                                                    const uint32_t* __restrict__ cnt,
-                                                   uint32_t* __restrict__ start,
                                                    uint32_t* __restrict__ cur,
                                                    uint4* __restrict__ jobs,
                                                    uint32_t* __restrict__ njobs,
@@ -265,15 +264,11 @@ __global__ void __launch_bounds__(1024) k_bin_scan(SortSeg* segs,
     const uint32_t b = tid * PER + i;
     if (b < bins) {
       s_start[b] = run;
-      start[sg.bin_base + b] = run;
       cur[sg.bin_base + b] = run;
     }
     run += c[i];
   }
-  if (tid == 0) {
-    s_start[bins] = tot;
-    start[sg.bin_base + bins] = tot;
-  }
+  if (tid == 0) s_start[bins] = tot;
   __syncthreads();
   // a bin opens a job at the target's multiples, next to a bin beyond the target
   // and at the reach of a T (span bins)

@@ -638,7 +638,7 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc, bo
     // and a split bin's slots
     g.job_cap = 7 * (g.n_host / target + 1) + (nb >> span) + 4;
     most_big += g.n_host / (2 * target);
-    bins += nb + 1;
+    bins += nb;
     slots += g.job_cap;
     ptiles += (g.n_host + 1024ull * B.items - 1) / (1024ull * B.items);
   }
@@ -652,7 +652,6 @@ void plan_bins(SortSeg* h_segs, int S, uint32_t total_tiles, SortScratch& sc, bo
   B.cnt = reinterpret_cast<uint32_t*>(take(bins * 4));
   B.big = reinterpret_cast<uint2*>(take((most_big + 1) * 8));
   B.zero_words = (uint32_t)((p - reinterpret_cast<char*>(sc.look)) / 4);
-  B.start = reinterpret_cast<uint32_t*>(take(bins * 4));
   B.cur = reinterpret_cast<uint32_t*>(take(bins * 4));
   B.jobs = reinterpret_cast<uint4*>(take(slots * 16));
   B.info = reinterpret_cast<uint4*>(take(slots * 16));
@@ -702,7 +701,7 @@ static void launch_bin_jobs(int S, const SortScratch& sc, uint32_t stride, uint3
   T *k0 = static_cast<T*>(sc.keys0), *k1 = static_cast<T*>(sc.keys1);
   // (attributes are summed faster by bins than in general, but not a crowded row's)
   const bool values = B.value_rows != nullptr;
-  k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.start, B.cur, B.jobs, B.njobs, B.big, !values);
+  k_bin_scan<T><<<S, 1024, 0, stream>>>(sc.segs, B.cnt, B.cur, B.jobs, B.njobs, B.big, !values);
   if (B.value_rows != nullptr) {
     launch_part<T, true>(S, sc, stride, stream);
     if (B.may_split) launch_split<T, true>(sc, stride, stream);

@@ -428,7 +428,8 @@ int cga_nn_query_batch(const cga_t* const* a, const cga_queries* q, uint32_t cou
                        const cga_allocator* A, void* stream);
 
 /* ---- Launch-shape tuning ---------------------------------------------------
- * The sort (build, xz/yz projection, NN coarse levels) and merge kernels run
+ * The radix sort (coarse levels, occupancy trees, xz/yz projections of fine grids,
+ * builds that do not go by bins) and merge kernels run
  * in one of several launch shapes, all with identical results.  A
  * process-wide table keyed by (grid bits, bit length of the element count)
  * holds the shape each call uses: the sort looks up (bits, n) of its largest
@@ -457,7 +458,8 @@ int cga_tuning_set(uint32_t bits, uint64_t n, const cga_tuning* t);
 int cga_tuning_get(uint32_t bits, uint64_t n, cga_tuning* out);
 
 /* Fill the entry for (g->bits, n) by measurement on the caller's cloud d_xyz
- * (n >= 2 float32 points, device): time a build of the whole cloud under each
+ * (n >= 2 float32 points, device): time a build of the whole cloud by the radix
+ * sort (which cga_build takes only where bins are slower) under each
  * sort candidate, then the merge of the CGAs of its two halves under each
  * merge candidate, and keep the fastest of each.  chosen receives the stored
  * shape; times_ms (NULL or CGA_TUNE_SORT_CANDIDATES + CGA_TUNE_MERGE_CANDIDATES
@@ -491,8 +493,8 @@ typedef struct {
 } cga_pipeline_item;
 
 /* cga_autotune for a pipeline: create the pipeline of these items under each
- * sort candidate, then each merge candidate, time two graph replays of each
- * (after the capturing one) and store the fastest shape in the entry the
+ * sort candidate (its builds by the radix sort), then each merge candidate, time two
+ * graph replays of each (after the capturing one) and store the fastest shape in the entry the
  * pipeline looks up, (largest bits, largest n).  chosen and times_ms as in
  * cga_autotune.  Every candidate pipeline is freed before the next is made;
  * the items' NN outputs are overwritten. */

@@ -252,8 +252,10 @@ struct ValueBuild {
   bool done;
 };
 
+// by_bins: by bins where plan_bins says so (else by the radix sort whatever the cloud).
 int build_cloud(const float* d_xyz, uint64_t n, const cga_grid* g, const float* h_xform12,
-                const cga_allocator* A, void* stream, ValueBuild* vb, cga_t** out) {
+                const cga_allocator* A, void* stream, ValueBuild* vb, cga_t** out,
+                bool by_bins = true) {
   if (out == nullptr || !grid_ok(g) || n > CGA_MAX_POINTS || (n > 0 && d_xyz == nullptr)) {
     return CGA_ERR_INVALID_ARG;
   }
@@ -289,7 +291,7 @@ int build_cloud(const float* d_xyz, uint64_t n, const cga_grid* g, const float* 
     return CGA_ERR_OOM;
   }
   libcga::SortScratch sc = libcga::sort_scratch_carve(scratch, keys, tiles, 1, key64, tu);
-  libcga::plan_bins(&seg, 1, tiles, sc, vb != nullptr);
+  if (by_bins) libcga::plan_bins(&seg, 1, tiles, sc, vb != nullptr);
   if (vb != nullptr && sc.bins.on) {
     sc.bins.value_in = vb->in;
     sc.bins.value_out = h->lv;
@@ -313,6 +315,10 @@ namespace libcga {
 // The NN search structures prepared on a handle (x directory, column table,
 // coarse levels or occupancy tree), for entry points in other files.
 void nn_attach(const cga_t* a, NnSeg& seg) { attach_coarse(a, seg); }
+// A build by the radix sort, for the autotuner to time its launch shapes.
+int build_by_radix(const float* d_xyz, uint64_t n, const cga_grid* g, void* stream, cga_t** out) {
+  return build_cloud(d_xyz, n, g, nullptr, nullptr, stream, nullptr, out, false);
+}
 }  // namespace libcga
 
 extern "C" {
@@ -1591,8 +1597,8 @@ int pipeline_queue(cga_pipeline* p, cudaStream_t s) {
 
 }  // namespace
 
-int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cga_allocator* A,
-                        void* stream, cga_pipeline_t** out) {
+static int pipeline_create(const cga_pipeline_item* items, uint32_t count, const cga_allocator* A,
+                           void* stream, bool by_bins, cga_pipeline_t** out) {
   if (out == nullptr || count == 0 || items == nullptr) return CGA_ERR_INVALID_ARG;
   if (A != nullptr && (A->alloc == nullptr || A->free == nullptr)) return CGA_ERR_INVALID_ARG;
   for (uint32_t i = 0; i < count; ++i) {
@@ -1728,7 +1734,7 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
   }
   p->build = libcga::sort_scratch_carve(base + o_build, build_tiles * libcga::kTile,
                                         (uint32_t)build_tiles, (int)(2 * S), key64, tu);
-  libcga::plan_bins(bsegs.data(), (int)(2 * S), (uint32_t)build_tiles, p->build);
+  if (by_bins) libcga::plan_bins(bsegs.data(), (int)(2 * S), (uint32_t)build_tiles, p->build);
   p->build_tiles = (uint32_t)build_tiles;
   p->build_passes = passes;
   p->key64 = key64;
@@ -1801,6 +1807,11 @@ int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cg
   }
   *out = p;
   return CGA_OK;
+}
+
+int cga_pipeline_create(const cga_pipeline_item* items, uint32_t count, const cga_allocator* A,
+                        void* stream, cga_pipeline_t** out) {
+  return pipeline_create(items, count, A, stream, true, out);
 }
 
 int cga_pipeline_run(cga_pipeline_t* p, void* stream) {
@@ -1900,3 +1911,11 @@ const char* cga_strerror(int code) {
 }
 
 }  // extern "C"
+
+namespace libcga {
+// A pipeline whose builds go by the radix sort, for the autotuner.
+int pipeline_by_radix(const cga_pipeline_item* items, uint32_t count, void* stream,
+                      cga_pipeline_t** out) {
+  return pipeline_create(items, count, nullptr, stream, false, out);
+}
+}  // namespace libcga

@@ -75,6 +75,10 @@ void tuning_store(uint32_t bits, uint64_t n, const Tuning* t) {
   g_table[bits][bucket_of(n)].store(t != nullptr ? pack(*t) : 0u, std::memory_order_relaxed);
 }
 
+int build_by_radix(const float* d_xyz, uint64_t n, const cga_grid* g, void* stream, cga_t** out);
+int pipeline_by_radix(const cga_pipeline_item* items, uint32_t count, void* stream,
+                      cga_pipeline_t** out);
+
 }  // namespace libcga
 
 namespace {
@@ -153,7 +157,8 @@ int cga_autotune(const float* d_xyz, uint64_t n, const cga_grid* g, cga_tuning* 
                : CGA_ERR_CUDA;
   libcga::Tuning best = before;
   float best_ms = -1.0f;
-  // the sort shape, on a build of the whole cloud
+  // the sort shape, on a build of the whole cloud by the radix sort (builds by bins have
+  // one shape; the entry steers the sorts of coarse levels, trees and wide projections)
   for (int k = 0; k < CGA_TUNE_SORT_CANDIDATES && rc == CGA_OK; ++k) {
     libcga::Tuning t = sort_cand[k];
     t.merge_half = before.merge_half;
@@ -162,7 +167,7 @@ int cga_autotune(const float* d_xyz, uint64_t n, const cga_grid* g, cga_tuning* 
     rc = time_min(
         [&]() {
           cga_t* a = nullptr;
-          const int r = cga_build(d_xyz, n, g, nullptr, nullptr, stream, &a);
+          const int r = libcga::build_by_radix(d_xyz, n, g, stream, &a);
           if (a != nullptr) cga_free(a);
           return r;
         },
@@ -239,12 +244,13 @@ int cga_pipeline_autotune(const cga_pipeline_item* items, uint32_t count, cga_tu
   int rc = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess
                ? CGA_OK
                : CGA_ERR_CUDA;
-  // one pipeline per candidate: its first graph launch captures, the timed
-  // ones replay
-  auto time_shape = [&](const libcga::Tuning& t, float* ms) {
+  // one pipeline per candidate, of the sort candidates with builds by the radix sort: its
+  // first graph launch captures, the timed ones replay
+  auto time_shape = [&](const libcga::Tuning& t, bool by_radix, float* ms) {
     libcga::tuning_store(bits, n, &t);
     cga_pipeline_t* p = nullptr;
-    int r = cga_pipeline_create(items, count, nullptr, stream, &p);
+    int r = by_radix ? libcga::pipeline_by_radix(items, count, stream, &p)
+                     : cga_pipeline_create(items, count, nullptr, stream, &p);
     if (r == CGA_OK) r = time_min([&]() { return cga_pipeline_run_graph(p, stream); }, 2, s, e0, e1, ms);
     if (p != nullptr) {
       if (cudaStreamSynchronize(s) != cudaSuccess && r == CGA_OK) r = CGA_ERR_CUDA;
@@ -258,7 +264,7 @@ int cga_pipeline_autotune(const cga_pipeline_item* items, uint32_t count, cga_tu
     libcga::Tuning t = sort_cand[k];
     t.merge_half = before.merge_half;
     float ms = 0.0f;
-    rc = time_shape(t, &ms);
+    rc = time_shape(t, true, &ms);
     if (rc != CGA_OK) break;
     if (times_ms) times_ms[k] = ms;
     if (best_ms < 0.0f || ms < best_ms) {
@@ -272,7 +278,7 @@ int cga_pipeline_autotune(const cga_pipeline_item* items, uint32_t count, cga_tu
     libcga::Tuning t = best;
     t.merge_half = merge_cand[k];
     float ms = 0.0f;
-    rc = time_shape(t, &ms);
+    rc = time_shape(t, false, &ms);
     if (rc != CGA_OK) break;
     if (times_ms) times_ms[CGA_TUNE_SORT_CANDIDATES + k] = ms;
     if (best_ms < 0.0f || ms < best_ms) {

@@ -1,0 +1,64 @@
+"""The autotuners time their sort candidates on the radix sort, whose launch shapes they
+choose, not on builds by bins, which have one shape: the times are those of the longer
+way, and the digit widths differ by more than noise."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2110_11616_gb300 import cga
+
+pytestmark = pytest.mark.gpu
+BITS, N = 12, 12_000_000
+
+
+def _points(n, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand((n, 3), generator=gen, device="cuda")
+
+
+@pytest.fixture()
+def clean():
+    def clear():
+        for bits in range(1, 17):
+            for nb in range(32):
+                cga.tuning_set(bits, (1 << (nb - 1)) if nb else 0, None)
+
+    clear()
+    yield
+    clear()
+
+
+def _least_ms(call):
+    call()
+    best = float("inf")
+    for _ in range(5):
+        t0, t1 = torch.cuda.Event(True), torch.cuda.Event(True)
+        torch.cuda.synchronize()
+        t0.record()
+        kept = call()
+        t1.record()
+        torch.cuda.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+        del kept
+    return best
+
+
+def test_cloud(clean):
+    g, pts = cga.grid_from_box([0, 0, 0], 1.0, BITS), _points(N, 1)
+    build = _least_ms(lambda: cga.cga_build(pts, g))
+    _, times = cga.cga_autotune(pts, g)
+    sort = list(times["sort"].values())
+    assert min(sort) > 1.3 * build, (build, times)   # 2.0 at this size
+    assert max(sort) > 1.03 * min(sort), times
+
+
+def test_pipeline(clean):
+    pts = [_points(N // 4, 2 + i) for i in range(2)]
+    grids = [cga.grid_from_box([0, 0, 0], 1.0, BITS)] * 2
+    xform = [[1.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0, 0.01, 0.0, 0.0]] * 2
+    pipe = cga.Pipeline(pts, grids, xform, [None] * 2)
+    run = _least_ms(pipe.run_graph)
+    _, times = cga.pipeline_autotune(pts, grids, xform, [None] * 2)
+    assert min(times["sort"].values()) > 1.15 * run, (run, times)
+    assert max(times["sort"].values()) > 1.02 * min(times["sort"].values()), times
+    pipe.free()

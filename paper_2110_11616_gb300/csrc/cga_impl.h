@@ -33,6 +33,7 @@ bool tuning_valid(const Tuning& t);
 // when none was set).  Host only, thread-safe.
 Tuning tuning_for(uint32_t bits, uint64_t n);
 void tuning_store(uint32_t bits, uint64_t n, const Tuning* t);  // nullptr: back to the default
+bool tuning_is_set(uint32_t bits, uint64_t n);
 // The merge partition of a launch: the entry of (bits, n) when one was set, else
 // by a rule on the grid (rule_bits) and points its largest pair can hold.
 uint32_t merge_half_for(uint32_t bits, uint64_t n, uint32_t rule_bits, uint64_t points,

@@ -47,6 +47,11 @@ Tuning tuning_for(uint32_t bits, uint64_t n) {
   return (v & kSet) ? unpack(v) : kDefaultTuning;
 }
 
+bool tuning_is_set(uint32_t bits, uint64_t n) {
+  return bits >= 1 && bits <= 16 &&
+         (g_table[bits][bucket_of(n)].load(std::memory_order_relaxed) & kSet) != 0u;
+}
+
 // The partition of merges whose entry was never set, from what the host knows:
 // the grid, and the points the two inputs can hold (of the largest pair of a
 // launch).  Measured per merge on GB300 (512 / 1024 / 2048, us):
@@ -151,6 +156,7 @@ int cga_autotune(const float* d_xyz, uint64_t n, const cga_grid* g, cga_tuning* 
   const uint32_t bits = g->bits;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const libcga::Tuning before = libcga::tuning_for(bits, n);
+  const bool was_set = libcga::tuning_is_set(bits, n);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   int rc = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess
                ? CGA_OK
@@ -217,7 +223,7 @@ int cga_autotune(const float* d_xyz, uint64_t n, const cga_grid* g, cga_tuning* 
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (rc != CGA_OK) {
-    libcga::tuning_store(bits, n, &before);
+    libcga::tuning_store(bits, n, was_set ? &before : nullptr);
     return rc;
   }
   libcga::tuning_store(bits, n, &best);
@@ -240,6 +246,7 @@ int cga_pipeline_autotune(const cga_pipeline_item* items, uint32_t count, cga_tu
   static const uint32_t merge_cand[CGA_TUNE_MERGE_CANDIDATES] = {512u, 1024u, 2048u};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const libcga::Tuning before = libcga::tuning_for(bits, n);
+  const bool was_set = libcga::tuning_is_set(bits, n);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   int rc = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess
                ? CGA_OK
@@ -290,7 +297,7 @@ int cga_pipeline_autotune(const cga_pipeline_item* items, uint32_t count, cga_tu
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (rc != CGA_OK) {
-    libcga::tuning_store(bits, n, &before);
+    libcga::tuning_store(bits, n, was_set ? &before : nullptr);
     return rc;
   }
   libcga::tuning_store(bits, n, &best);

@@ -1,6 +1,8 @@
 """The autotuners time their sort candidates on the radix sort, whose launch shapes they
 choose, not on builds by bins, which have one shape: the times are those of the longer
 way, and the digit widths differ by more than noise."""
+import ctypes
+
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -62,3 +64,40 @@ def test_pipeline(clean):
     assert min(times["sort"].values()) > 1.15 * run, (run, times)
     assert max(times["sort"].values()) > 1.02 * min(times["sort"].values()), times
     pipe.free()
+
+
+def test_entry_left_unset_by_an_error(clean):
+    """After a failed autotune a merge still takes its partition from the rule: the blocks
+    that it asks for are those of before, and others once the default is set."""
+    sizes, held = [], {}
+
+    @ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p)
+    def alloc(ctx, size, stream):
+        sizes.append(int(size))
+        t = torch.empty(int(size), dtype=torch.uint8, device="cuda")
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    @ctypes.CFUNCTYPE(None, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p)
+    def free(ctx, p, stream):
+        torch.cuda.synchronize()
+        held.pop(p, None)
+
+    pts = _points(60_000, 9)
+    g = cga.grid_from_box([0, 0, 0], 1.0, BITS)
+    a, b = cga.cga_build(pts[0::2].contiguous(), g), cga.cga_build(pts[1::2].contiguous(), g)
+    allocator = cga.Allocator(None, alloc, free)
+
+    def merge_blocks():
+        sizes.clear()
+        m = cga.cga_merge(a, b, allocator=allocator)
+        torch.cuda.synchronize()
+        del m
+        return list(sizes)
+
+    before = merge_blocks()
+    with pytest.raises(cga.CgaError):
+        cga.cga_autotune(pts, cga.make_grid(BITS, float("nan"), (0.0, 0.0, 0.0)))
+    assert merge_blocks() == before
+    cga.tuning_set(BITS, len(pts), {"radix_bits": 8, "sort_threads": 512, "merge_half": 2048})
+    assert merge_blocks() != before

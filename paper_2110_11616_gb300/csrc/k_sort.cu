@@ -130,13 +130,15 @@ __global__ void __launch_bounds__(kThreads) k_keys_hist(const SortSeg* __restric
 // The same for segments whose keys come from a CGA (projections, coarse levels, trees): a
 // block takes runs of a step of a walk for each of its warps (k_walk.cuh), not whole tiles,
 // so that small sources have a warp for every step: the xz projection of 30k points at b =
-// 16 took 96 us by tiles, 79 so.
+// 16 took 96 us by tiles, 79 so.  Eight blocks an SM hide more of the walk's loads than
+// four (the tree of 20M surface voxels 1595 us, five 1562, six 1575, eight 1540).
+constexpr int kKeysWalkPerSm = 8;
 constexpr uint32_t kWalkRun = kWarps * kWalk;
 static_assert(kTile % kWalkRun == 0, "runs of a tile");
 template <typename K, int RB>
-__global__ void __launch_bounds__(kThreads) k_keys_walk(const SortSeg* __restrict__ segs, int S,
-                                                        uint32_t total_runs, uint32_t runs_per_cta,
-                                                        K* keys0, uint32_t* hist) {
+__global__ void __launch_bounds__(kThreads, kKeysWalkPerSm)
+    k_keys_walk(const SortSeg* __restrict__ segs, int S, uint32_t total_runs, uint32_t runs_per_cta,
+                K* keys0, uint32_t* hist) {
   constexpr uint32_t PER = kTile / kWalkRun;
   __shared__ BlockHist<RB> sh;
   const uint32_t r1 = min((blockIdx.x + 1) * runs_per_cta, total_runs);
@@ -808,7 +810,8 @@ template <typename K>
 static void launch_keys(int S, uint32_t total_tiles, bool walk, const SortScratch& sc,
                         cudaStream_t stream) {
   const uint32_t items = walk ? total_tiles * (kTile / kWalkRun) : total_tiles;
-  const uint32_t ctas = std::min<uint32_t>(items, (uint32_t)device_sm_count() * 4);
+  const uint32_t ctas =
+      std::min<uint32_t>(items, (uint32_t)device_sm_count() * (walk ? kKeysWalkPerSm : 4));
   const uint32_t per = (items + ctas - 1) / ctas;
   K* k0 = static_cast<K*>(sc.keys0);
   if (walk && sc.radix_bits == 9) {

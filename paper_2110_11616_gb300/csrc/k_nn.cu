@@ -1146,6 +1146,42 @@ __device__ __forceinline__ bool search_bfs(const TreeView& tv, const Qry& q, uin
     Y = ((w1 >> 12) & 0xfffu) << 2 | cy;
     Z = (w1 >> 24 | ((w2 >> 6) & 0xfu) << 8) << 2 | cz;
   };
+  // First down the query's own cells, as far as they hold voxels: a near query ends in its
+  // brick, whose voxels (shared by the lanes) bound the answer closely, or are it.  Without
+  // it every brick within a box's reach was examined: 300k near queries of 3M LiDAR points,
+  // b = 10, 653 us, depth-first 354, 259 so; of 300k uniform ones, b = 6, 718, 356 and 268;
+  // the 4M of the surface world 14.1 -> 13.6 ms; sparse worlds lose 2%.
+  D cd = (D)~(D)0;  // the lane's best voxel
+  unsigned long long ck = ~0ull;
+  if (run) {
+    uint32_t l = tv.levels, n = 0;
+    if (tv.dense != nullptr) {
+      l = tv.dense_level;
+      const uint32_t c = tv.dense_bits;
+      n = __ldg(tv.dense + ((size_t)(q.cx >> (2 * l)) << (2 * c) | (q.cy >> (2 * l)) << c |
+                            q.cz >> (2 * l)));
+    }
+    bool in = n != kTreeAbsent;
+    while (in && l > 1) {
+      const uint4 nd = __ldg(tv.node[l] + n);
+      --l;
+      const uint32_t p = tree_child((q.cx >> (2 * l)) & 3u, (q.cy >> (2 * l)) & 3u,
+                                    (q.cz >> (2 * l)) & 3u);
+      const unsigned long long m = (unsigned long long)nd.y << 32 | nd.x;
+      in = (m >> p) & 1ull;
+      n = nd.z + (uint32_t)__popcll(m & ((1ull << p) - 1ull));
+    }
+    if (in) {
+      constexpr uint32_t NB = 64 / G;
+      const unsigned long long mine = ((1ull << NB) - 1ull) << (g * NB);
+      brick_voxels<D>(__ldg(tv.brick + n) & mine, q.cx & ~3u, q.cy & ~3u, q.cz & ~3u, q, b, cd, ck);
+    }
+  }
+  {
+    const D own = group_least<G, D>(cd);
+    R = fminf(R, bound_up(own));
+    if (own == 0) run = false;  // the query's own voxel
+  }
   // Start: the nodes of the position table that the bound reaches, when they
   // are at most four per axis; the query's own cell first tightens the bound.
   bool dense = false;
@@ -1285,8 +1321,6 @@ __device__ __forceinline__ bool search_bfs(const TreeView& tv, const Qry& q, uin
     __syncwarp();
   }
   // bricks: a lane each
-  D cd = (D)~(D)0;
-  unsigned long long ck = ~0ull;
   const bool bricks = active && !gave_up;
   while (__any_sync(full, bricks && head < tail)) {
     if (bricks && head + g < tail) {

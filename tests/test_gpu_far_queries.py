@@ -55,7 +55,7 @@ def test_nearest_answers():
 def test_nearest_time(n, m):
     q = _far(m, 2)
     t = {bits: _time(lambda: cga.cga_nn_query(a, q)) for bits, a, _ in _worlds(n)}
-    assert t[16] < 2.5 * t[13], t   # 1.7 with 64-bit distances throughout
+    assert t[16] < 4 * t[13], t   # 0.9 and 2.1; up to 8.7 while the walk had no bound
 
 
 @pytest.mark.parametrize("m", [1, 7, 300, 3000, 7000, 9000, 30_000])
@@ -99,4 +99,4 @@ def test_knn_answers(k, m):
 def test_knn_time(n):
     q = _far(10_000, 4)
     t = {bits: _time(lambda: cga.cga_knn(a, q, 8)) for bits, a, _ in _worlds(n)}
-    assert t[16] < 3 * t[13], t   # 1.0 to 1.8 with 64-bit distances throughout
+    assert t[16] < 4 * t[13], t   # 1.2 and 2.5; up to 15 while the walk had no bound
